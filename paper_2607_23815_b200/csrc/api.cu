@@ -6,7 +6,7 @@ namespace kvattn {
 size_t decode_workspace_bytes(int n_q_heads, int head_dim, int batch, int max_ctx_len);
 kv_status_t launch_decode(kv_pool_t* p, const void* q, int n_q_heads, const int* block_tables, int max_pages,
                           const int* ctx_lens, int batch, int max_ctx_len, float scale, void* out, float* lse,
-                          void* workspace, size_t workspace_bytes, cudaStream_t st, bool beside = false);
+                          cudaStream_t st, bool beside = false);
 kv_status_t launch_extend_small(kv_pool_t* p, const void* q, int n_q_heads, const int* cu_q, const int* block_tables,
                                 int max_pages, const int* prefix_lens, const int* extend_lens, int batch,
                                 int max_extend_len, int max_total_len, float scale, void* out, float* lse,
@@ -295,10 +295,11 @@ static kv_status_t decode_impl(kv_pool_t* p, const void* q, int n_q_heads, const
   if (max_ctx_len > (int64_t)max_pages * kPageSize) return KV_ERR_INVALID;
   if (!on_pool_device(p)) return KV_ERR_INVALID;
   if (max_ctx_len == 0) max_ctx_len = 1;  // every row is empty: still defines O = 0, LSE = -inf
-  // the decode region of a combined workspace starts after the extend region; a caller that sized
-  // the workspace for decode only passes (0, 0) for the extend part, so the offset is 0 there
+  // the kernel needs no scratch, but the workspace is part of the interface: too small a one is refused as it always was
+  const size_t need = decode_workspace_bytes(n_q_heads, p->head_dim, batch, max_ctx_len);
+  if (need > 0 && (workspace == nullptr || workspace_bytes < need)) return KV_ERR_WORKSPACE;
   return launch_decode(p, q, n_q_heads, block_tables, max_pages, ctx_lens, batch, max_ctx_len, scale, out, lse,
-                       workspace, workspace_bytes, (cudaStream_t)stream, beside);
+                       (cudaStream_t)stream, beside);
 }
 
 kv_status_t attn_decode(kv_pool_t* p, const void* q, int n_q_heads, const int* block_tables, int max_pages,
