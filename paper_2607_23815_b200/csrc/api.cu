@@ -11,7 +11,10 @@ kv_status_t launch_extend_small(kv_pool_t* p, const void* q, int n_q_heads, cons
                                 int max_pages, const int* prefix_lens, const int* extend_lens, int batch,
                                 int max_extend_len, int max_total_len, float scale, void* out, float* lse,
                                 cudaStream_t st);
-size_t extend_tc_workspace_bytes(int n_q_heads, int head_dim, int batch, int total_q, int max_total_len);
+size_t extend_tc_workspace_bytes(const kv_pool_t* p, int n_q_heads, int batch, int total_q, int max_total_len);
+size_t extend_tc_min_workspace_bytes(int batch, int total_q);
+kv_status_t launch_extend_combine(kv_pool_t* p, int n_q_heads, int batch, int total_q, int max_extend_len, int max_total_len, void* out, float* lse,
+                                  void* workspace, size_t workspace_bytes, bool early, cudaStream_t st);
 bool extend_tc_supported(const kv_pool_t* p, int n_q_heads);
 kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const int* cu_q, const int* block_tables,
                              int max_pages, const int* prefix_lens, const int* extend_lens, int batch, int total_q,
@@ -40,6 +43,12 @@ static bool heads_supported(const kv_pool_t* p, int n_q_heads) {
   return g == 1 || g == 2 || g == 4 || g == 8;
 }
 
+// Does extend go to the tensor-core kernel?  (It folds a positive scale into the row maximum.)
+static bool uses_tc(const kv_pool_t* p, int n_q_heads, float scale) {
+  const int impl = g_extend_impl.load();
+  return impl != 1 && extend_tc_supported(p, n_q_heads) && scale > 0.f;
+}
+
 static inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 }  // namespace kvattn
 
@@ -57,7 +66,7 @@ size_t attn_workspace_bytes(const kv_pool_t* p, int n_q_heads, int batch_ext, in
                             int batch_dec, int max_ctx_len) {
   if (p == nullptr || n_q_heads <= 0) return 0;
   // the two regions are disjoint so that a mixed step can run both kinds of work at once
-  return align256(extend_tc_workspace_bytes(n_q_heads, p->head_dim, batch_ext, total_q, max_total_len)) +
+  return align256(extend_tc_workspace_bytes(p, n_q_heads, batch_ext, total_q, max_total_len)) +
          align256(decode_workspace_bytes(n_q_heads, p->head_dim, batch_dec, max_ctx_len)) + 256;
 }
 
@@ -319,8 +328,12 @@ kv_status_t attn_mixed(kv_pool_t* p, int n_q_heads, float scale, const attn_exte
   const bool has_dec = dec != nullptr && dec->batch > 0;
   cudaStream_t st = (cudaStream_t)stream;
   size_t ext_bytes = 0;
-  if (has_ext)
-    ext_bytes = align256(extend_tc_workspace_bytes(n_q_heads, p->head_dim, ext->batch, ext->total_q, ext->max_total_len));
+  if (has_ext) {
+    const size_t dec_bytes = has_dec ? decode_workspace_bytes(n_q_heads, p->head_dim, dec->batch, dec->max_ctx_len) : 0;
+    ext_bytes = align256(extend_tc_workspace_bytes(p, n_q_heads, ext->batch, ext->total_q, ext->max_total_len));
+    // (less than attn_workspace_bytes() asks for, but enough to run the extend set without span scheduling)
+    if (ext_bytes + dec_bytes > workspace_bytes) ext_bytes = align256(extend_tc_min_workspace_bytes(ext->batch, ext->total_q));
+  }
   if (ext_bytes > workspace_bytes) return KV_ERR_WORKSPACE;
   char* ws = reinterpret_cast<char*>(workspace);
   if (has_ext && has_dec) {
@@ -343,8 +356,13 @@ kv_status_t attn_mixed(kv_pool_t* p, int n_q_heads, float scale, const attn_exte
                                 ext->extend_lens, ext->batch, ext->total_q, ext->max_extend_len, ext->max_total_len,
                                 scale, ext->out, ext->lse, ws, ext_bytes, cap, st);
     if (s != KV_OK) return s;
-    return decode_impl(p, dec->q, n_q_heads, dec->block_tables, dec->max_pages, dec->ctx_lens, dec->batch, dec->max_ctx_len,
-                       scale, dec->out, dec->lse, ws ? ws + ext_bytes : nullptr, workspace_bytes - ext_bytes, st, true);
+    s = decode_impl(p, dec->q, n_q_heads, dec->block_tables, dec->max_pages, dec->ctx_lens, dec->batch, dec->max_ctx_len,
+                    scale, dec->out, dec->lse, ws ? ws + ext_bytes : nullptr, workspace_bytes - ext_bytes, st, true);
+    if (s != KV_OK) return s;
+    // (the extend kernel's cut items are merged behind both kernels: the decode kernel must be the next in the stream)
+    if (!uses_tc(p, n_q_heads, scale)) return KV_OK;
+    return launch_extend_combine(p, n_q_heads, ext->batch, ext->total_q, ext->max_extend_len, ext->max_total_len, ext->out, ext->lse, ws, ext_bytes,
+                                 false, st);
   }
   if (has_ext)
     return attn_extend(p, ext->q, n_q_heads, ext->cu_q, ext->block_tables, ext->max_pages, ext->prefix_lens,

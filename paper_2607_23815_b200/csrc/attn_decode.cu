@@ -17,6 +17,7 @@
 #include "sm100_ptx.cuh"
 
 namespace kvattn {
+using namespace ptx;
 
 struct DecodeArgs {
   PoolView pool;
@@ -61,20 +62,6 @@ struct DecodeShared {
 template <int D, bool RING>
 constexpr int decode_smem_bytes() {
   return (RING ? DecodeSmem<D>::kRing : DecodeSmem<D>::kPart) + DecodeSmem<D>::kIn + (int)sizeof(DecodeShared);
-}
-
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ uint32_t cluster_addr(uint32_t smem_addr, int cta) {
-  uint32_t a;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr), "r"(cta));
-  return a;
-}
-__device__ __forceinline__ void st_cluster(uint32_t addr, float4 v) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
-}
-__device__ __forceinline__ void st_cluster(uint32_t addr, float2 v) {
-  asm volatile("st.shared::cluster.v2.f32 [%0], {%1,%2};" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
 }
 
 template <int D, bool RING>

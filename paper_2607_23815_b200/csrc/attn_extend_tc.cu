@@ -20,7 +20,8 @@
 //   warp 14     Q loader: one tensor-map (TMA) copy per 64-dim half brings a query tile into shared
 //               memory in the swizzled operand layout, as soon as the MMAs that read the previous
 //               item's tile have finished.
-//   warp 15     idle (launched for the registers it hands to the others).
+//   warp 15     span scheduling: finds the CTA's span and announces its items; else idle (launched for the registers it
+//               hands to the others).
 // The two query tiles ping-pong: while one tile's softmax runs, the tensor core works on the other.
 // All waits are bounded; on expiry the CTA records KV_ERR_TIMEOUT, drains its copies, frees its
 // tensor memory and returns.
@@ -39,13 +40,38 @@ using namespace ptx;
 // CTA was launched with (512 threads x 128 registers), in total and per scheduler (warp index mod 4):
 // 8 x 192 (softmax) + 4 x 72 (epilogue) + 56 + 56 + 40 + 24 = 2000 <= 2048 per lane.
 constexpr int kTcThreads = 512;
-constexpr int kWarpEpilogue = 8, kWarpProducer = 12, kWarpMma = 13, kWarpQ = 14;
+constexpr int kWarpEpilogue = 8, kWarpProducer = 12, kWarpMma = 13, kWarpQ = 14, kWarpSched = 15;
 constexpr int kPlanBuckets = 2048;
 constexpr int kPlanSeqBuckets = 1024;   // length buckets for ranking the sequences (one per plan thread)
 constexpr int kPlanMaxRanked = 8192;    // batches up to this size are ranked by length; larger ones keep their order
 constexpr float kRescaleThreshold = 8.0f;  // log2 units: O is rescaled only when the max grows by more than this
 constexpr int kOptimisticMinLen = 4096;     // batches with a sequence this long use the kernel that skips the maximum search
 constexpr float kOptimisticSum = 65536.0f;  // a row sum of one tile beyond this sends the step to the exact maximum
+
+// Span scheduling, for batches with few work items per SM.  The KV steps of all items, laid end to end, are cut into
+// at most n_spans spans of equal length, one CTA takes one (in attn_mixed: a few neighbouring ones), and an item that a
+// cut goes through leaves partial results that span_combine_kernel merges.  Every CTA finds its span by itself from the
+// length arrays, so no plan kernel runs in front.  The cuts depend on the lengths and on n_spans alone.
+struct SpanArgs {
+  int n_spans, per_cta;  // spans at most; neighbouring spans one CTA takes
+  int max_tp, total_q;   // host-side bounds: tile pairs of a sequence, rows of Q
+  int plan_early;        // the kernel in front is this call's own append: the lengths may be read before waiting for it
+  int4* desc;            // [n_spans][3]: the cut at the start of a span: (first step of the item it goes through among all
+                         // steps, or -1; step of the item; KV head; tile pair), (rows, first row, KV steps of the two tiles)
+  float* part_o;         // [n_spans][2][D / 8][256][8]: a cut item's rows, normalised within the chunk (nullptr: no item is
+                         // cut); eight dims of a row, then the next row, so that a warp's rows are contiguous
+  float* part_lse;       // [n_spans][2][256]: log2-domain log-sum-exp of the chunk
+};
+constexpr int kSpanMinSteps = 2;  // KV steps of a span at least
+constexpr int kSpanSnap = 1;      // a cut this close to the edge of an item moves to the edge
+
+// Who takes which items.
+//  kSchedList: the plan's list, through a work counter (any number of items).
+//  kSchedSpans: equal spans of KV steps (see SpanArgs).
+//  kSchedCluster: one item per cluster of cl_splits CTAs, each with an equal part of its KV steps; their results are merged
+//  through distributed shared memory.  For batches whose items, that many CTAs each, are on the device at once.
+constexpr int kSchedList = 0, kSchedSpans = 1, kSchedCluster = 2;
+constexpr int kMaxClusterSplits = 8;
 
 struct TcArgs {
   PoolView pool;
@@ -70,6 +96,8 @@ struct TcArgs {
   const int4* items;   // two int4 per entry (see ItemRec), cost-sorted
   const int* n_items;  // number of valid entries in items
   int* next_item;      // work counter: the next item of the global list nobody has taken yet
+  SpanArgs span;       // span scheduling and items per cluster (no plan, no counter)
+  int cl_splits;
 };
 
 // ------------------------------------------------------------------------------------------
@@ -337,9 +365,18 @@ struct __align__(1024) TcSmem {
   // takes the next) and announces them here; every role walks the same sequence.
   unsigned long long sched_full[4], sched_empty[4];
   int sched_idx[4];
+  int4 sched_rec[4][3];    // the whole record of an item (see SpanRec)
+  int4 cl_unit;            // one item per cluster: its rows, first row in Q, tile pair, KV head
   float inv_l[2][2][128];  // [tile][item parity][row]: 1 / row sum, handed from the softmax to the epilogue warps
   uint32_t tmem_base;
   int abort_flag;
+};
+
+// Span scheduling: what the scheduler warp announces of a chunk of an item (P and kv_end count from the chunk's first key).
+struct SpanRec {
+  int seq, kvh, tp, P;
+  int E, row0, n_kv0, n_kv1;
+  int kv_end, first_tile, part;  // part: slot of the partial result, -1 for a whole item
 };
 
 struct Item {
@@ -348,6 +385,7 @@ struct Item {
   int ld_tiles;  // KV tiles the producer brings in
   int kv_end;    // keys the item can see at most (fan-out mode: the parent's keys)
   int c_first;   // fan-out mode: first child with a row in the item
+  int first_tile, part;  // span scheduling: first KV tile of the chunk, slot of its partial result (-1: none)
 };
 
 // Fan-out mode: position in the children's part of an item's KV steps.
@@ -401,6 +439,123 @@ __device__ __forceinline__ bool fetch_item(const TcArgs& a, int k, int n_total, 
   return true;
 }
 
+// Span scheduling.  A sequence's items are ordered (KV head, tile pair); position x of the line of all steps is step
+// `off` of the item (seq, kvh, tp) that starts at `at`.
+struct SpanPos {
+  int seq, kvh, tp, off, at;
+};
+
+// Rows of the sequence that count: none if the lengths do not fit the tables, no row past the host-side bounds.
+__device__ __forceinline__ int span_rows(const TcArgs& a, int P, int E, int row0) {
+  if (P < 0 || E <= 0 || row0 < 0 || P + E > a.max_pages * kPageSize) return 0;
+  return min(min(E, (int)min((int64_t)0x7fffffff, ((int64_t)a.span.max_tp * 256) >> a.lg_group)), max(0, a.span.total_q - row0));
+}
+// KV steps of tile pair tp of a sequence with E rows behind P keys
+__device__ __forceinline__ int span_steps(int P, int E, int tp, int lg) { return (P + min(E, ((tp + 1) * 256) >> lg) + 127) >> 7; }
+__device__ __forceinline__ int span_pairs(int E, int lg) { return (int)(((int64_t)E * (1 << lg) + 255) >> 8); }
+// Steps of the first m tile pairs if all of them are full: sum over k = 1 .. m of ceil((P + k * 256 / G) / 128).  A pair's
+// tokens are 256, 128, 64 or 32, so the terms grow by 2, by 1, or by 1 every 2 or 4 pairs.
+__device__ __forceinline__ int span_full_steps(int P, int m, int lg) {
+  const int cp = (P + 127) >> 7;
+  if (lg < 2) return m * cp + (lg == 0 ? m * (m + 1) : (m * (m + 1)) >> 1);
+  const int lq = lg - 1, tokens = 256 >> lg;
+  int sum = 0;
+  for (int r = 1; r <= (1 << lq); ++r) {
+    const int cnt = m >= r ? ((m - r) >> lq) + 1 : 0;
+    sum += cnt * ((P + tokens * r + 127) >> 7) + ((cnt * (cnt - 1)) >> 1);
+  }
+  return sum;
+}
+// Steps of all tile pairs of one KV head of a sequence
+__device__ __forceinline__ int span_head_steps(int P, int E, int lg) {
+  const int pairs = span_pairs(E, lg);
+  return pairs == 0 ? 0 : span_full_steps(P, pairs - 1, lg) + span_steps(P, E, pairs - 1, lg);
+}
+__device__ __forceinline__ int span_count(const SpanArgs& a, int total) {
+  return max(1, min(a.n_spans, (total + kSpanMinSteps - 1) / kSpanMinSteps));
+}
+// Where span s begins, among all steps
+__device__ __forceinline__ int span_cut(int total, int n_spans, int s) {
+  const int each = total / n_spans, rest = total - each * n_spans;
+  return each * s + rest * s / n_spans;
+}
+// Where a cut at step `off` of an item of n steps goes: 0 or n (an edge), or it stays (unless items are not to be cut).
+__device__ __forceinline__ int span_snap(const SpanArgs& a, int off, int n) {
+  if (off <= kSpanSnap) return 0;
+  if (n - off <= kSpanSnap) return n;
+  return a.part_o != nullptr ? off : 2 * off < n ? 0 : n;
+}
+
+// The lengths of 32 sequences, one per lane.
+struct SpanSeqs {
+  int base, P, rows, row0;
+};
+__device__ __forceinline__ void span_load(const TcArgs& a, int base, SpanSeqs& q) {
+  const int seq = base + (threadIdx.x & 31);
+  q.base = base;
+  q.P = q.rows = q.row0 = 0;
+  if (seq < a.batch) {
+    const int P = __ldg(a.prefix_lens + seq), E = __ldg(a.extend_lens + seq);
+    q.row0 = __ldg(a.cu_q + seq);
+    q.P = P;
+    q.rows = span_rows(a, P, E, q.row0);
+    if (blockIdx.x == 0 && P >= 0 && q.rows < E) report(a.pool.status, KV_ERR_BOUNDS);
+  }
+}
+
+// One warp: sums the steps of all sequences and finds the item and step at which span `first_span` begins (seq = batch:
+// nothing to do).
+__device__ __forceinline__ void span_locate(const TcArgs& a, int first_span, SpanPos& pos, int& total, SpanSeqs& q) {
+  const int lane = threadIdx.x & 31, lg = a.lg_group, Hkv = a.pool.n_kv_heads;
+  span_load(a, 0, q);
+  int mine = span_head_steps(q.P, q.rows, lg);
+  total = mine;
+  for (int base = 32; base < a.batch; base += 32) {
+    SpanSeqs t;
+    span_load(a, base, t);
+    total += span_head_steps(t.P, t.rows, lg);
+  }
+  total = __reduce_add_sync(0xffffffffu, total) * Hkv;
+  pos = SpanPos{a.batch, 0, 0, 0, total};
+  const int n_spans = span_count(a.span, total);
+  if (first_span >= n_spans || total == 0) return;
+  const int x = span_cut(total, n_spans, first_span);
+  int before = 0;  // steps of the sequences in front
+  while (true) {
+    int incl = mine * Hkv;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, off);
+      if (lane >= off) incl += u;
+    }
+    const unsigned behind = __ballot_sync(0xffffffffu, before + incl > x);
+    if (behind) {
+      const int l = __ffs(behind) - 1;
+      pos.seq = q.base + l;
+      const int per_head = __shfl_sync(0xffffffffu, mine, l);
+      int rem = x - before - (__shfl_sync(0xffffffffu, incl, l) - per_head * Hkv);
+      const int P = __shfl_sync(0xffffffffu, q.P, l), rows = __shfl_sync(0xffffffffu, q.rows, l);
+      pos.kvh = rem / per_head;
+      rem -= pos.kvh * per_head;
+      // tile pair: the last one with span_full_steps(pair) <= rem, 32 probes at a time
+      int lo = 0, span = span_pairs(rows, lg);
+      while (span > 1) {
+        const int step = (span + 31) >> 5, idx = lo + lane * step, end = lo + span;
+        const int k = __popc(__ballot_sync(0xffffffffu, idx < end && span_full_steps(P, idx, lg) <= rem)) - 1;
+        lo += k * step;
+        span = min(step, end - lo);
+      }
+      pos.tp = lo;
+      pos.off = rem - span_full_steps(P, lo, lg);
+      pos.at = x - pos.off;
+      return;
+    }
+    before += __shfl_sync(0xffffffffu, incl, 31);
+    span_load(a, q.base + 32, q);
+    mine = span_head_steps(q.P, q.rows, lg);
+  }
+}
+
 // Operand descriptors differ only in their low word (start address >> 4 plus the leading-dimension
 // offset field); the high word is a constant.  Issuing an MMA then costs one add, so a single thread
 // keeps the tensor pipe fed.
@@ -429,12 +584,70 @@ __device__ __forceinline__ void issue_pv_mmas(uint32_t o_tmem, uint32_t p_tmem, 
     if (p < np) mma_ts(o_tmem, p_tmem + p * 8, make_desc(kHiV, v_lo + p * (D * 2)), idesc, 1u);
 }
 
+// Partial results lie in pieces of eight dims: [slot][D / 8][256 rows][8].
+// 32 dims of a row, scaled, from registers: four pieces (a warp's 32 rows are contiguous in each).
+__device__ __forceinline__ void store_part8x4(float* dst, const uint32_t (&o)[32], float inv) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(dst + 256 * 8 * i),
+                 "f"(__uint_as_float(o[8 * i]) * inv), "f"(__uint_as_float(o[8 * i + 1]) * inv),
+                 "f"(__uint_as_float(o[8 * i + 2]) * inv), "f"(__uint_as_float(o[8 * i + 3]) * inv),
+                 "f"(__uint_as_float(o[8 * i + 4]) * inv), "f"(__uint_as_float(o[8 * i + 5]) * inv),
+                 "f"(__uint_as_float(o[8 * i + 6]) * inv), "f"(__uint_as_float(o[8 * i + 7]) * inv)
+                 : "memory");
+}
+// Merges piece g of row r over its chunks, in chunk order, U chunks' loads in flight: eight dims as bf16, and the
+// log2-domain log-sum-exp.  slot(k): slot of chunk k; has(k): does chunk k hold a step of the row's tile (else its slot
+// was not written; a chunk without a key the row sees has weight 0).
+template <int D, int U, typename Slot, typename Has>
+__device__ __forceinline__ uint4 merge_part8(const SpanArgs& a, int chunks, int r, int g, Slot slot, Has has, float& lse2) {
+  float mx = -INFINITY, wsum = 0.f, o[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) o[e] = 0.f;
+  for (int base = 0; base < chunks; base += U) {
+    float l[U], x[U][8];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int k = base + u;
+      l[u] = -INFINITY;
+      if (k < chunks && has(k)) {
+        const int sl = slot(k);
+        l[u] = __ldcg(a.part_lse + sl * 256 + r);
+        const float4* src = reinterpret_cast<const float4*>(a.part_o + (((int64_t)sl * (D / 8) + g) * 256 + r) * 8);
+        const float4 v0 = __ldcg(src), v1 = __ldcg(src + 1);
+        x[u][0] = v0.x; x[u][1] = v0.y; x[u][2] = v0.z; x[u][3] = v0.w;
+        x[u][4] = v1.x; x[u][5] = v1.y; x[u][6] = v1.z; x[u][7] = v1.w;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (l[u] == -INFINITY) continue;
+      const float mn = fmaxf(mx, l[u]);
+      const float keep = exp2f(mx - mn), w = exp2f(l[u] - mn);
+      mx = mn;
+      wsum = wsum * keep + w;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) o[e] = o[e] * keep + w * x[u][e];
+    }
+  }
+  const float inv = 1.f / wsum;
+  uint32_t pk[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pk[e]) : "f"(o[2 * e + 1] * inv), "f"(o[2 * e] * inv));
+  lse2 = mx + log2f(wsum);
+  return make_uint4(pk[0], pk[1], pk[2], pk[3]);
+}
+
 // OPT: the softmax warps skip the search for the row maximum after an item's first tile (see there); chosen by the
 // host for batches whose sequences are long, where nearly every step is such a step.
 // FAN: the fan-out mode (TcArgs::mode 2); the other modes are compiled without the walk over the children's tiles.
-template <int D, bool OPT, bool FAN>
+// SCHED: who takes which items (see kSchedList).
+template <int D, bool OPT, bool FAN, int SCHED>
 __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcArgs a, const __grid_constant__ CUtensorMap q_map) {
   using Cfg = TcCfg<D>;
+  constexpr bool SPAN = SCHED == kSchedSpans, CLUSTER = SCHED == kSchedCluster;
+  constexpr bool REC = SPAN || CLUSTER;  // the scheduler warp announces whole records
   extern __shared__ unsigned char smem_raw[];
   // Dynamic shared memory starts on a 1024-byte boundary (this kernel has no static shared memory); the swizzled
   // operand tiles need that.  Checked instead of padded for: the tiles leave no room for padding.
@@ -457,7 +670,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
     }
     for (int s4 = 0; s4 < 4; ++s4) {
       mbar_init(smem_u32(&sm.sched_full[s4]), 1);    // the producer wrote the slot
-      mbar_init(smem_u32(&sm.sched_empty[s4]), 14);  // MMA warp, Q loader, 8 softmax and 4 epilogue warps have read it
+      mbar_init(smem_u32(&sm.sched_empty[s4]), REC ? 15 : 14);  // MMA warp, Q loader, 8 softmax and 4 epilogue warps (and the producer) have read it
     }
     for (int t = 0; t < 2; ++t) {
       mbar_init(smem_u32(&sm.q_full[t]), 1);    // the Q tile's bytes have landed (transaction count)
@@ -474,14 +687,24 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
     tmem_alloc(smem_u32(&sm.tmem_base), 512);
     tmem_relinquish();
   }
+  int cl_P = 0, cl_E = 0, cl_row0 = 0;
+  if (CLUSTER && warp == kWarpSched) {  // the item's lengths are asked for while the CTA is set up
+    const int seq = (int)blockIdx.x / a.cl_splits / a.pool.n_kv_heads / a.span.max_tp;
+    if (!a.span.plan_early) dependency_wait();
+    cl_P = __ldg(a.prefix_lens + seq);
+    cl_E = __ldg(a.extend_lens + seq);
+    cl_row0 = __ldg(a.cu_q + seq);
+    for (int b = lane * 32; b < a.max_pages; b += 1024) prefetch_l2(a.block_tables + (int64_t)seq * a.max_pages + b);
+  }
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = sm.tmem_base;
   // Everything up to here touched only this CTA's own shared and tensor memory and may have run while the kernel in
   // front of this one (the plan, or the plan and the suffix append) was still at work; its results are needed now.
-  dependency_wait();
-  const int n_total = __ldcg(a.n_items) * a.pool.n_kv_heads;
+  // (the scheduler warp reads the lengths first where it may)
+  if (!REC || warp != kWarpSched || !a.span.plan_early) dependency_wait();
+  const int n_total = REC ? 0 : __ldcg(a.n_items) * a.pool.n_kv_heads;
   const int Hkv = a.pool.n_kv_heads;
   // Round r of this CTA works on item sched_get(r) of the global list (>= n_total: no more work).  A warp
   // calls sched_release(r) once it no longer needs the slot.
@@ -493,6 +716,23 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
   auto sched_release = [&](int round) {
     __syncwarp();
     if (lane == 0) mbar_arrive(smem_u32(&sm.sched_empty[round & 3]));
+  };
+  // The item of a round; false: no more work.
+  auto fetch = [&](int round, Item& it) -> bool {
+    if constexpr (REC) {
+      if (!mbar_wait(smem_u32(&sm.sched_full[round & 3]), (round >> 2) & 1, abortp)) return false;
+      const int4 r0 = sm.sched_rec[round & 3][0], r1 = sm.sched_rec[round & 3][1], r2 = sm.sched_rec[round & 3][2];
+      it.seq = r0.x; it.kvh = r0.y; it.tp = r0.z; it.P = r0.w;
+      it.E = r1.x; it.row0 = r1.y; it.n_kv[0] = r1.z; it.n_kv[1] = r1.w;
+      it.kv_end = r2.x; it.first_tile = r2.y; it.part = r2.z;
+      it.c_first = 0;
+      it.ld_tiles = max(it.n_kv[0], it.n_kv[1]);
+      return it.seq >= 0;
+    } else {
+      it.first_tile = 0;
+      it.part = -1;
+      return fetch_item<FAN>(a, sched_get(round), n_total, it);
+    }
   };
 
   if (warp == kWarpProducer) {
@@ -512,20 +752,25 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
       ok = __shfl_sync(0xffffffffu, ok, 0);
     };
     int cur = blockIdx.x;
-    announce(0, cur);
-    for (int round = 0; ok && cur < n_total; ++round) {
-      // The next item is taken and announced one item ahead, so that nobody waits for the counter.  (Taking it
-      // two items ahead would hide the counter's latency from this warp too, but an item that is committed early
-      // cannot go to a CTA that runs out of work: measured slower.)
-      int nxt_idx = 0;
-      if (lane == 0) nxt_idx = atomicAdd(a.next_item, 1);
-      nxt_idx = __shfl_sync(0xffffffffu, nxt_idx, 0);
-      announce(round + 1, nxt_idx);
+    if constexpr (!REC) announce(0, cur);
+    for (int round = 0; ok && (REC || cur < n_total); ++round) {
       Item it;
-      fetch_item<FAN>(a, cur, n_total, it);
-      cur = nxt_idx;
+      if constexpr (REC) {
+        if (!fetch(round, it)) break;
+        sched_release(round);
+      } else {
+        // The next item is taken and announced one item ahead, so that nobody waits for the counter.  (Taking it
+        // two items ahead would hide the counter's latency from this warp too, but an item that is committed early
+        // cannot go to a CTA that runs out of work: measured slower.)
+        int nxt_idx = 0;
+        if (lane == 0) nxt_idx = atomicAdd(a.next_item, 1);
+        nxt_idx = __shfl_sync(0xffffffffu, nxt_idx, 0);
+        announce(round + 1, nxt_idx);
+        fetch_item<FAN>(a, cur, n_total, it);
+        cur = nxt_idx;
+      }
       if (!ok) break;
-      const int* bt = a.block_tables + (int64_t)it.seq * a.max_pages;
+      const int* bt = a.block_tables + (int64_t)it.seq * a.max_pages + (REC ? it.first_tile * 8 : 0);
       const size_t head_off = (size_t)it.kvh * Cfg::kBlockBytes;
       const int n_own = FAN ? (it.P + 127) >> 7 : it.ld_tiles;  // tiles from the sequence's (parent's) own pages
       ChildCur cc{0, 0, 0, 0};
@@ -579,9 +824,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
     // the softmax warps have written P_t, then S_t = Q_t K(j+1)^T into the columns P_t occupied (the tensor
     // core runs MMAs in issue order), so the other tile's MMAs fill the time this tile's softmax takes.
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
-    const uint32_t q_lo0 = (smem_u32(sm.q[0]) >> 4) | (1u << 16);             // low descriptor words: LBO field 16 B
-    const uint32_t k_lo0 = (smem_u32(sm.kv[0]) >> 4) | (1u << 16);
-    const uint32_t v_lo0 = (smem_u32(sm.kv[0]) >> 4) | ((1024u >> 4) << 16);  // V tiles: LBO = 64-dim half
+    // Low descriptor words.  The address field takes 14 bits: in a cluster the upper bits of a shared address name the CTA.
+    auto lo_word = [](const void* p, uint32_t lbo) { return ((smem_u32(p) >> 4) & 0x3FFFu) | ((lbo >> 4) << 16); };
+    const uint32_t q_lo0 = lo_word(sm.q[0], 16), k_lo0 = lo_word(sm.kv[0], 16);
+    const uint32_t v_lo0 = lo_word(sm.kv[0], 1024);  // V tiles: LBO = 64-dim half
     const uint32_t bar_s_full = smem_u32(&sm.s_full[0]), bar_p_full = smem_u32(&sm.p_full[0]);
     const uint32_t bar_q_full = smem_u32(&sm.q_full[0]), bar_o_full = smem_u32(&sm.o_full[0]);
     const uint32_t bar_q_empty = smem_u32(&sm.q_empty[0]), bar_o_empty = smem_u32(&sm.o_empty[0]);
@@ -592,10 +838,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
     uint32_t items_done[2] = {0, 0};    // items per tile so far (phase of q_full)
     bool ok = true;
     Item nxt;
-    bool has_nxt = fetch_item<FAN>(a, sched_get(0), n_total, nxt);
+    bool has_nxt = fetch(0, nxt);
     for (int round = 0; ok && has_nxt; ++round) {
       const Item it = nxt;
-      has_nxt = fetch_item<FAN>(a, sched_get(round + 1), n_total, nxt);
+      has_nxt = fetch(round + 1, nxt);
       sched_release(round);
       if (it.ld_tiles == 0) continue;
       {
@@ -703,7 +949,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
     uint32_t fills[2] = {0, 0};  // tiles loaded so far per buffer (phase of q_empty)
     bool ok = true;
     Item it;
-    for (int round = 0; ok && fetch_item<FAN>(a, sched_get(round), n_total, it); ++round) {
+    for (int round = 0; ok && fetch(round, it); ++round) {
       sched_release(round);
       if (it.ld_tiles == 0) continue;
 #pragma unroll
@@ -726,7 +972,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
       }
       // the next item's query tiles are asked into L2 now, a whole item ahead of their copy to shared memory
       Item nx;
-      if (fetch_item<FAN>(a, sched_get(round + 1), n_total, nx) && nx.ld_tiles > 0 && lane == 0) {
+      if (fetch(round + 1, nx) && nx.ld_tiles > 0 && lane == 0) {
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
           if (nx.n_kv[t] == 0) continue;
@@ -736,8 +982,122 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
         }
       }
     }
-  } else if (warp == 15) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 24;");  // idle warp
+  } else if (warp == kWarpSched) {
+    if constexpr (!REC) {
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 24;");  // idle warp
+    } else if constexpr (CLUSTER) {
+      // =============================== scheduler (one item per cluster) =======================
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+      const int lg = a.lg_group, splits = a.cl_splits;
+      const int unit = (int)blockIdx.x / splits, rank = (int)blockIdx.x - unit * splits;
+      const int rest = unit / Hkv, kvh = unit - rest * Hkv, seq = rest / a.span.max_tp, tp = rest - seq * a.span.max_tp;
+      const int P = cl_P, E = cl_E, row0 = cl_row0;
+      const int rows = span_rows(a, P, E, row0), pairs = span_pairs(rows, lg);
+      if (a.span.plan_early) dependency_wait();
+      if (lane == 0) {
+        if (tp == 0 && kvh == 0 && rank == 0 && P >= 0 && rows < E) report(a.pool.status, KV_ERR_BOUNDS);
+        int n = 0, n0 = 0, n1 = 0, hi = 0;
+        if (tp < pairs) {
+          const int tok_1 = (tp * 256 + 128) >> lg;  // first token of the second tile
+          n0 = (P + min(rows, tok_1) + 127) >> 7;
+          hi = min(rows, ((tp + 1) * 256) >> lg);
+          n = (P + hi + 127) >> 7;
+          n1 = tok_1 < rows ? n : 0;
+        }
+        const int off = n * rank / splits, end = n * (rank + 1) / splits;
+        sm.cl_unit = make_int4(tp < pairs ? min(256, (rows << lg) - tp * 256) : 0, row0, tp, kvh);
+        int round = 0;
+        if (end > off) {
+          sm.sched_rec[0][0] = make_int4(seq, kvh, tp, P - off * 128);
+          sm.sched_rec[0][1] = make_int4(rows, row0, max(0, min(n0, end) - off), max(0, min(n1, end) - off));
+          sm.sched_rec[0][2] = make_int4(P + hi - off * 128, off, -1, 0);
+          mbar_arrive(smem_u32(&sm.sched_full[0]));
+          round = 1;
+        }
+        sm.sched_rec[round][0] = make_int4(-1, 0, 0, 0);
+        sm.sched_rec[round][1] = sm.sched_rec[round][2] = make_int4(0, 0, 0, 0);
+        mbar_arrive(smem_u32(&sm.sched_full[round]));
+      }
+    } else {
+      // =============================== scheduler (span scheduling) ============================
+      // Walks the items from the start of the CTA's first span to the end of its last and announces their chunks.
+      // (Every lane walks; lane 0 writes.)
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+      const int lg = a.lg_group;
+      SpanPos pos;
+      int total, round = 0, span = (int)blockIdx.x * a.span.per_cta;
+      SpanSeqs q;
+      span_locate(a, span, pos, total, q);
+      const int n_spans = span_count(a.span, total);
+      if (a.span.plan_early) dependency_wait();
+      const int span_end = min(span + a.span.per_cta, n_spans);
+      bool ok = true;
+      auto announce = [&](const SpanRec& r) {
+        if (lane == 0) {
+          ok = mbar_wait(smem_u32(&sm.sched_empty[round & 3]), ((round >> 2) & 1) ^ 1, abortp);
+          sm.sched_rec[round & 3][0] = make_int4(r.seq, r.kvh, r.tp, r.P);
+          sm.sched_rec[round & 3][1] = make_int4(r.E, r.row0, r.n_kv0, r.n_kv1);
+          sm.sched_rec[round & 3][2] = make_int4(r.kv_end, r.first_tile, r.part, 0);
+          mbar_arrive(smem_u32(&sm.sched_full[round & 3]));
+        }
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        ++round;
+      };
+      // spans that the batch has no work for leave no cut behind
+      for (int s = max(span, span_end); s < min(((int)blockIdx.x + 1) * a.span.per_cta, a.span.n_spans); ++s)
+        if (lane == 0) a.span.desc[3 * s] = make_int4(-1, 0, 0, 0);
+      bool fresh = true;  // the start of the first span has not been moved to an item's edge yet
+      if (span < span_end) {
+        int off = pos.off;
+        auto cut_at = [&](int s) { return s >= n_spans ? total : span_cut(total, n_spans, s); };
+        for (int seq = pos.seq; seq < a.batch && span < span_end && ok; ++seq) {
+          if (seq >= q.base + 32) span_load(a, seq, q);
+          const int l = seq - q.base;
+          const int P = __shfl_sync(0xffffffffu, q.P, l), row0 = __shfl_sync(0xffffffffu, q.row0, l);
+          const int rows = __shfl_sync(0xffffffffu, q.rows, l), pairs = span_pairs(rows, lg);
+          int kvh = seq == pos.seq ? pos.kvh : 0, tp = seq == pos.seq ? pos.tp : 0;
+          for (; kvh < Hkv && pairs > 0 && span < span_end && ok; ++kvh, tp = 0) {
+            for (; tp < pairs && span < span_end && ok; ++tp) {
+              const int n = span_steps(P, rows, tp, lg);
+              const int tok_1 = (tp * 256 + 128) >> lg;  // first token of the second tile
+              const int hi0 = min(rows, tok_1), hi1 = tok_1 < rows ? min(rows, ((tp + 1) * 256) >> lg) : 0;
+              const int n0 = (P + hi0 + 127) >> 7, n1 = hi1 > 0 ? (P + hi1 + 127) >> 7 : 0;
+              auto put_cut = [&]() {
+                if (lane == 0) {
+                  a.span.desc[3 * span] = make_int4(off > 0 && off < n ? pos.at : -1, off, kvh, tp);
+                  a.span.desc[3 * span + 1] = make_int4(rows, row0, n0, n1);
+                }
+              };
+              if (fresh) {
+                fresh = false;
+                off = span_snap(a.span, off, n);
+                put_cut();
+              }
+              // the chunks of this item, one per span
+              while (off < n && span < span_end && ok) {
+                const int raw = cut_at(span + 1) - pos.at;  // where the span ends, counted from the item's first step
+                const int end = raw >= n ? n : raw <= 0 ? 0 : span_snap(a.span, raw, n);
+                if (end > off) {
+                  const int part = off > 0 ? 2 * span : end < n ? 2 * span + 1 : -1;
+                  announce(SpanRec{seq, kvh, tp, P - off * 128, rows, row0, max(0, min(n0, end) - off), max(0, min(n1, end) - off),
+                                   P + max(hi0, hi1) - off * 128, off, part});
+                  off = end;
+                }
+                if (raw <= n && (raw < n || off == n)) {  // the span ends in (or with) this item
+                  ++span;
+                  if (span < span_end) put_cut();
+                }
+              }
+              pos.at += n;
+              off = 0;
+            }
+          }
+        }
+      }
+      for (int s = span + (fresh ? 0 : 1); s < span_end; ++s)  // empty spans at the end of the line
+        if (lane == 0) a.span.desc[3 * s] = make_int4(-1, 0, 0, 0);
+      announce(SpanRec{-1, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0});
+    }
   } else if (warp >= kWarpEpilogue) {
     // =============================== epilogue warpgroup ====================================
     // One thread per row (= TMEM lane), both tiles in turn: O / l -> bf16 -> global.
@@ -746,26 +1106,28 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
     const int m = w4 * 32 + lane;
     const uint32_t lane_base = tmem + ((uint32_t)(w4 * 32) << 16);
     const int G = a.group, lg = a.lg_group, Hq = a.n_q_heads;
-    uint32_t done[2] = {0, 0};  // items finished per tile (phase of o_full / l_full, parity of inv_l)
+    uint32_t done0 = 0, done1 = 0;  // items finished per tile (phase of o_full / l_full, parity of inv_l)
     bool ok = true;
     Item it;
-    for (int round = 0; ok && fetch_item<FAN>(a, sched_get(round), n_total, it); ++round) {
+    for (int round = 0; ok && fetch(round, it); ++round) {
       sched_release(round);
+      if (CLUSTER && a.cl_splits > 1) continue;  // the softmax warps hand the partial results over
       if (it.ld_tiles == 0) continue;
-#pragma unroll
+#pragma unroll 1
       for (int t = 0; t < 2; ++t) {
-        if (it.n_kv[t] == 0 || !ok) continue;
+        if ((t ? it.n_kv[1] : it.n_kv[0]) == 0 || !ok) continue;
         const int rg = it.tp * 256 + t * 128 + m;
         const int tok = rg >> lg;
         const bool valid = tok < it.E;
         const int64_t orow_idx = (int64_t)(it.row0 + tok) * Hq + it.kvh * G + (rg & (G - 1));
-        ok = mbar_wait(smem_u32(&sm.l_full[t]), done[t] & 1, abortp);
-        if (ok) ok = mbar_wait(smem_u32(&sm.o_full[t]), done[t] & 1, abortp);
+        const uint32_t par = (t ? done1 : done0) & 1;
+        ok = mbar_wait(smem_u32(&sm.l_full[t]), par, abortp);
+        if (ok) ok = mbar_wait(smem_u32(&sm.o_full[t]), par, abortp);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         tc_fence_after_sync();
-        const float inv = sm.inv_l[t][done[t] & 1][m];
-        ++done[t];
+        const float inv = sm.inv_l[t][par][m];
+        if (t) ++done1; else ++done0;
         const uint32_t o_addr = lane_base + 256 + t * 128;
         // A row is 2 * D contiguous bytes, but a warp holds 32 different rows: 16-byte stores from the thread
         // that owns the row touch 32 cache lines per instruction and half a sector each.  Instead two
@@ -778,7 +1140,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
         const uint32_t n_hi = __shfl_xor_sync(0xffffffffu, (uint32_t)(reinterpret_cast<uintptr_t>(row_ptr) >> 32), 1);
         char* nb_ptr = reinterpret_cast<char*>(((uint64_t)n_hi << 32) | n_lo);
         const bool nb_valid = __shfl_xor_sync(0xffffffffu, (int)valid, 1) != 0;
-#pragma unroll
+#pragma unroll 1
         for (int c = 0; c < D / 32; ++c) {
           uint32_t orow[32];
           tmem_ld32(o_addr + c * 32, orow);
@@ -786,6 +1148,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
           if (c == D / 32 - 1) {  // all of the row has been read: the next item's PV may overwrite O
             tc_fence_before_sync();
             mbar_arrive(smem_u32(&sm.o_empty[t]));
+          }
+          if (SPAN && it.part >= 0) {  // a chunk of a cut item: its rows stay in fp32 until the chunks are merged
+            if (valid) {
+              store_part8x4(a.span.part_o + (((int64_t)it.part * (D / 8) + c * 4) * 256 + t * 128 + m) * 8, orow, inv);
+            }
+            continue;
           }
           uint32_t pk[16];  // columns [32c, 32c + 32) as bf16 pairs: two pieces of eight words
 #pragma unroll
@@ -831,11 +1199,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
     const int G = a.group, lg = a.lg_group, Hq = a.n_q_heads;
     uint32_t steps = 0, items_done = 0;            // phase of s_full / p_full; items finished (parity of inv_l)
     bool ok = true;
+    float cl_m = -INFINITY, cl_l = 0.f;            // cluster: the row's maximum and sum over this CTA's part
 
     // The item records are read where they are needed (they stay in L1) instead of being carried in registers
     // through the softmax loop, which needs the registers for the score row.
     for (int round = 0; ok; ++round) {
-      int n_t, limit;
+      int n_t, limit, part = -1;
       bool valid;
       int64_t orow_idx;
       // fan-out mode: the steps from n_own on walk the children's own keys; tok_s is this row's token among the
@@ -844,7 +1213,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
       ChildCur cc{0, 0, 0, 0};
       {
         Item it;
-        const bool more_items = fetch_item<FAN>(a, sched_get(round), n_total, it);
+        const bool more_items = fetch(round, it);
         if (!more_items) break;
         sched_release(round);
         if (it.ld_tiles == 0) continue;
@@ -855,6 +1224,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
         valid = tok < it.E;
         limit = valid && a.mode == 0 ? it.P + tok + 1 : it.kv_end;  // keys this row sees (rows past the end: any)
         orow_idx = (int64_t)(it.row0 + tok) * Hq + it.kvh * G + (rg & (G - 1));  // row of the LSE
+        if (SPAN) part = it.part;
         n_own = FAN ? (it.P + 127) >> 7 : n_t;
         if (FAN) {
           tok_s = valid ? tok : -1;
@@ -1018,6 +1388,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
       }
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
+      if (CLUSTER && a.cl_splits > 1) {  // O is final once the last PV is done
+        ok = mbar_wait(smem_u32(&sm.o_full[t]), 0, abortp);
+        ok = __all_sync(0xffffffffu, ok);
+        cl_m = m_run;
+        cl_l = l_run;
+        continue;
+      }
       // ---- hand the row to the epilogue warps: 1 / row sum through shared memory; the LSE is written here.
       // The softmax of an item needs only S, so with one-step items it could finish two items before the
       // epilogue warps have looked at the first: a barrier must not get two phases ahead of its waiters, so
@@ -1027,11 +1404,53 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
       }
-      sm.inv_l[t][items_done & 1][m] = 1.f / l_run;
+      // (a row may see no key of its chunk of a cut item: weight 0)
+      sm.inv_l[t][items_done & 1][m] = SPAN && !(l_run > 0.f) ? 0.f : 1.f / l_run;
       mbar_arrive(bar_l_full);
       ++items_done;
-      if (valid) a.lse[orow_idx] = (m_run + log2f(l_run)) * 0.6931471805599453f;
+      if (SPAN && part >= 0) {
+        if (valid) a.span.part_lse[part * 256 + t * 128 + m] = l_run > 0.f ? m_run + log2f(l_run) : -INFINITY;
+      } else if (valid) {
+        a.lse[orow_idx] = (m_run + log2f(l_run)) * 0.6931471805599453f;
+      }
     }
+    if (CLUSTER && a.cl_splits > 1) {
+      // The CTAs of the cluster hold partial results of the same rows.  Each writes its own out, then finishes an equal
+      // share of the rows from everybody's.  Through L2: read from the partners' shared memory, 148 rows on 8 CTAs took
+      // 8800 cycles (about 8 bytes a cycle and SM), this way 2500.
+      const int splits = a.cl_splits, unit = (int)blockIdx.x / splits, rank = (int)blockIdx.x - unit * splits;
+      const int4 u = sm.cl_unit;
+      const int row = t * 128 + m;
+      if (__any_sync(0xffffffffu, cl_l > 0.f)) {
+        tc_fence_after_sync();
+        const float inv = cl_l > 0.f ? 1.f / cl_l : 0.f;
+#pragma unroll 1
+        for (int c = 0; c < D / 32; ++c) {
+          uint32_t orow[32];
+          tmem_ld32(o_addr + c * 32, orow);
+          tmem_wait_ld();
+          if (row < u.x) store_part8x4(a.span.part_o + (((int64_t)blockIdx.x * (D / 8) + c * 4) * 256 + row) * 8, orow, inv);
+        }
+      }
+      a.span.part_lse[blockIdx.x * 256 + row] = cl_l > 0.f ? cl_m + log2f(cl_l) : -INFINITY;
+      cluster_arrive();
+      cluster_wait();
+      const int r_begin = u.x * rank / splits, cnt = u.x * (rank + 1) / splits - r_begin;
+      for (int i = tid; i < cnt * (D / 8); i += 256) {
+        const int g = i / cnt, r = r_begin + (i - g * cnt);  // eight dims of a row; neighbouring lanes take neighbouring rows
+        float lse2;
+        const uint4 o = merge_part8<D, kMaxClusterSplits>(a.span, splits, r, g, [&](int k) { return unit * splits + k; }, [](int) { return true; }, lse2);
+        const int rg = u.z * 256 + r;
+        const int64_t orow = (int64_t)(u.y + (rg >> lg)) * Hq + u.w * G + (rg & (G - 1));
+        reinterpret_cast<uint4*>(a.out + orow * D)[g] = o;
+        if (g == 0) a.lse[orow] = lse2 * 0.6931471805599453f;
+      }
+    }
+  }
+  if (CLUSTER && a.cl_splits > 1 && warp >= kWarpEpilogue) {  // the other warps' part in the cluster barrier
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
   }
 
   tc_fence_before_sync();
@@ -1040,7 +1459,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
   if (warp == kWarpProducer) tmem_dealloc(tmem, 512);
   // The last CTA to finish puts the work counter back where the plan left it, so that the same plan can serve
   // another launch (a model runs every layer of a step over the same lengths).  a.next_item + 1 counts the CTAs done.
-  if (tid == 0) {
+  if (!REC && tid == 0) {
     __threadfence();
     if (atomicAdd(a.next_item + 1, 1) == (int)gridDim.x - 1) {
       a.next_item[0] = (int)gridDim.x;
@@ -1048,6 +1467,70 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
       __threadfence();
     }
   }
+}
+
+// Merges the chunks of the items that the cuts between the spans went through.  Block (s - 1) * kCombineSlices + slice:
+// the item of which cut s is the first, 256 / kCombineSlices of its rows in turns of 32; warp w takes the dims 8w .. 8w + 7,
+// its lanes the rows.  Bound by latency and launch (a few MB through L2), so the blocks, most of which have nothing to do,
+// are to be resident at once: 40 registers.
+constexpr int kCombineSlices = 4;
+template <int D>
+__global__ void __launch_bounds__(D * 4, 384 / D) span_combine_kernel(const SpanArgs a, int n_q_heads, int group, int lg,
+                                                                      __nv_bfloat16* out, float* lse) {
+  launch_dependents();
+  dependency_wait();
+  constexpr int kRowWords = D / 2 + 4;  // a row of the result in shared memory, padded
+  __shared__ int first_tile[256];
+  __shared__ __align__(16) uint32_t rows[32 * kRowWords];
+  const int s = 1 + (int)blockIdx.x / kCombineSlices, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // (all loads of the cuts in flight at once)
+  const int mine = s + (int)threadIdx.x;
+  int dk_at = -1, dk_off = 0;
+  if (mine < a.n_spans && threadIdx.x < 255) {
+    const int4 dk = __ldcg(a.desc + 3 * mine);
+    dk_at = dk.x;
+    dk_off = dk.y;
+  }
+  const int4 d0 = __ldcg(a.desc + 3 * s), d1 = __ldcg(a.desc + 3 * s + 1);
+  const int before = __ldcg(a.desc + 3 * (s - 1)).x;
+  if (d0.x < 0 || before == d0.x) return;  // no cut, or not the first one of its item
+  // chunk 0 is the last of span s - 1, chunk k > 0 the first of span s + k - 1
+  const bool same = dk_at == d0.x;
+  if (same) first_tile[threadIdx.x + 1] = dk_off;
+  if (threadIdx.x == 0) first_tile[0] = 0;
+  const int chunks = 1 + __syncthreads_count(same);
+  const int kvh = d0.z, tp = d0.w, E = d1.x, row0 = d1.y;
+  auto row_of = [&](int mm) {  // row of the result
+    const int rg = tp * 256 + mm;
+    return (int64_t)(row0 + (rg >> lg)) * n_q_heads + kvh * group + (rg & (group - 1));
+  };
+  constexpr int kRows = 256 / kCombineSlices;
+  for (int m_slice = (int)(blockIdx.x % kCombineSlices) * kRows, turn = 0; turn < kRows / 32; ++turn, m_slice += 32) {
+    if (((tp * 256 + m_slice) >> lg) >= E) return;
+    const int m = m_slice + lane;
+    const int n_t = m < 128 ? d1.z : d1.w;
+    const bool valid = ((tp * 256 + m) >> lg) < E;
+    float lse2 = 0.f;
+    uint4 o = make_uint4(0, 0, 0, 0);
+    if (valid)
+      o = merge_part8<D, 2>(a, chunks, m, warp, [&](int k) { return k == 0 ? 2 * s - 1 : 2 * (s + k - 1); },
+                            [&](int k) { return first_tile[min(k, 255)] < n_t; }, lse2);
+    *reinterpret_cast<uint4*>(&rows[lane * kRowWords + warp * 4]) = o;
+    if (warp == 0 && valid) lse[row_of(m)] = lse2 * 0.6931471805599453f;
+    __syncthreads();
+    constexpr int kPieces = D / 8;  // 16-byte pieces of a row
+    const int r = (int)threadIdx.x / kPieces, piece = (int)threadIdx.x % kPieces;  // (32 * kPieces threads)
+    if (((tp * 256 + m_slice + r) >> lg) < E)
+      reinterpret_cast<uint4*>(out + row_of(m_slice + r) * D)[piece] = *reinterpret_cast<const uint4*>(&rows[r * kRowWords + piece * 4]);
+    __syncthreads();
+  }
+}
+
+// The suffix append in front of a span-scheduled attention kernel (which is launched early and waits for it inside).
+__global__ void __launch_bounds__(1024) append_prologue_kernel(const PoolView pool, const AppendArgs ap) {
+  launch_dependents();
+  const int warps_per_block = blockDim.x >> 5;
+  append_tokens<4>(pool, ap, blockIdx.x * warps_per_block + (threadIdx.x >> 5), gridDim.x * warps_per_block);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1058,12 +1541,40 @@ static int64_t item_capacity(int n_q_heads, int n_kv_heads, int batch, int total
   return (int64_t)total_q * G / 256 + batch + 1;
 }
 
-size_t extend_tc_workspace_bytes(int n_q_heads, int head_dim, int batch, int total_q, int max_total_len) {
-  (void)head_dim; (void)max_total_len;
-  if (batch <= 0 || total_q <= 0) return 0;
-  // n_kv_heads is not known here: G <= 8 bounds the list
+struct SpanLayout {
+  int n_spans;
+  bool cuts;              // may an item be cut?
+  size_t lse, o, total;   // behind the cuts
+};
+static int64_t items_at_most(const kv_pool_t* p, int n_q_heads, int batch, int total_q) {
+  return ((int64_t)total_q * (n_q_heads / p->n_kv_heads) / 256 + batch) * p->n_kv_heads;
+}
+static SpanLayout span_layout(const kv_pool_t* p, int n_q_heads, int batch, int total_q, int max_total_len) {
+  const int64_t steps = ((int64_t)max_total_len + 127) / 128, sms = sm_count_of(p->device);
+  const int64_t spans = (items_at_most(p, n_q_heads, batch, total_q) * steps + kSpanMinSteps - 1) / kSpanMinSteps;
+  SpanLayout l;
+  l.n_spans = (int)(spans < 1 ? 1 : spans < sms ? spans : sms);
+  l.cuts = steps > 2 * kSpanSnap + 1;  // (an item of up to that many steps is never cut)
+  const size_t rows = l.cuts ? (size_t)sms * 2 * 256 : 0;  // (two per span, or one per CTA of the clusters)
+  l.lse = align256((size_t)l.n_spans * 3 * sizeof(int4));
+  l.o = l.lse + align256(rows * sizeof(float));
+  l.total = l.o + rows * p->head_dim * sizeof(float);
+  return l;
+}
+static size_t list_bytes(int batch, int total_q) {
   return 256 + align256(2 * sizeof(int4) * (size_t)((int64_t)total_q * 8 / 256 + batch + 1));
 }
+
+// The item list of the plan, or what span scheduling keeps, whichever is larger whatever the batch turns out to be (a
+// workspace that is large enough for a batch is large enough for every smaller one); 256 bytes more to align the
+// caller's pointer.
+size_t extend_tc_workspace_bytes(const kv_pool_t* p, int n_q_heads, int batch, int total_q, int max_total_len) {
+  if (batch <= 0 || total_q <= 0 || n_q_heads < p->n_kv_heads) return 0;
+  const size_t list = list_bytes(batch, total_q), spans = span_layout(p, n_q_heads, batch, total_q, max_total_len).total;
+  return 256 + (list > spans ? list : spans);
+}
+// The least the extend kernel runs with (without span scheduling).
+size_t extend_tc_min_workspace_bytes(int batch, int total_q) { return 256 + list_bytes(batch, total_q); }
 
 bool extend_tc_supported(const kv_pool_t* p, int n_q_heads) {
   if (p->head_dim != 64 && p->head_dim != 128) return false;
@@ -1106,29 +1617,162 @@ static kv_status_t tc_grid(const kv_pool_t* p, int n_items_bound, int cta_cap, i
   return KV_OK;
 }
 
-template <int D, bool OPT, bool FAN>
-static kv_status_t launch_tc(const TcArgs& a, const CUtensorMap& q_map, int grid, int device, bool early_start, cudaStream_t st) {
+template <int D, bool OPT, bool FAN, int SCHED>
+static kv_status_t setup_tc(int device) {
   const size_t smem = sizeof(TcSmem<D>);
   static std::atomic<bool> configured[kMaxDevices];  // the attribute belongs to the function on one device
   if (device < 0 || device >= kMaxDevices) return KV_ERR_INVALID;
   if (!configured[device].load(std::memory_order_acquire)) {
-    KV_CUDA_OK(cudaFuncSetAttribute(attn_extend_tc_kernel<D, OPT, FAN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    KV_CUDA_OK(cudaFuncSetAttribute(attn_extend_tc_kernel<D, OPT, FAN, SCHED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (SCHED == kSchedCluster)
+      KV_CUDA_OK(cudaFuncSetAttribute(attn_extend_tc_kernel<D, OPT, FAN, SCHED>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     configured[device].store(true, std::memory_order_release);
   }
+  return KV_OK;
+}
+
+template <int D, bool OPT, bool FAN, int SCHED>
+static kv_status_t launch_tc(const TcArgs& a, const CUtensorMap& q_map, int grid, int device, bool early_start, cudaStream_t st) {
+  const kv_status_t ss = setup_tc<D, OPT, FAN, SCHED>(device);
+  if (ss != KV_OK) return ss;
   // early_start: launched so that it may start while the plan kernel in front of it still runs (it waits for it
   // inside).  Not wanted when another kernel is meant to take the SMs first (the mixed step's decode kernel): CTAs
   // that sit on an SM waiting for the plan keep that kernel's blocks away.
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(kTcThreads);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = sizeof(TcSmem<D>);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (early_start) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (SCHED == kSchedCluster && a.cl_splits > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = (unsigned)a.cl_splits;
+    attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = n;
+  KV_CUDA_OK(cudaLaunchKernelEx(&cfg, attn_extend_tc_kernel<D, OPT, FAN, SCHED>, a, q_map));
+  count_launch();
+  return KV_OK;
+}
+
+static constexpr int kSplitChoices[] = {1, 2, 3, 4, 6, 8};
+
+// How many clusters of c CTAs are on the device at a time (asked once per device and head size).
+template <int D>
+static kv_status_t resident_clusters(int device, int c, int* n) {
+  static std::atomic<int> cached[kMaxDevices][kMaxClusterSplits + 1];  // value + 1
+  const kv_status_t s = setup_tc<D, false, false, kSchedCluster>(device);
+  if (s != KV_OK) return s;
+  int v = cached[device][c].load(std::memory_order_relaxed);
+  if (v == 0) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)c);
+    cfg.blockDim = dim3(kTcThreads);
+    cfg.dynamicSmemBytes = sizeof(TcSmem<D>);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)c;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, attn_extend_tc_kernel<D, false, false, kSchedCluster>, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      clusters = 0;
+    }
+    v = clusters + 1;
+    cached[device][c].store(v, std::memory_order_relaxed);
+  }
+  *n = v - 1;
+  return KV_OK;
+}
+
+// Who takes which items, from the host-side bounds (and the workspace) alone; splits: CTAs per item for kSchedCluster.
+//  - Items that are on the device at once go to a cluster each, as large as fits, one KV step per CTA at least: no plan
+//    kernel, and the steps of an item run side by side.  Suffix append + extend of 1 / 4 / 8 / 16 sequences of 30-60 tokens
+//    behind 1000-2000 (32/8 heads of 128): 32.1 / 38.2 / 42.2 / 43.7 us through the list, 16.8 / 24.2 / 33.3 / 42.4 this
+//    way with 6 / 4 / 2 / 1 CTAs per item.
+//  - Few and long items: spans.  They cost a merge kernel behind the attention kernel (about 12 us, 8 steps) and win what
+//    the other two leave idle, the part of a cluster that no SM group holds or the last items of the list: 8 / 16
+//    sequences of 9000-16000 keys 219 / 225 us through the list, 121 / 242 with clusters, 102 / 181 with spans; 11 of up
+//    to 10700 (16/8 heads of 64) 260 and 197.  More than three items per SM, or short ones: the list (3 prefills of up to
+//    1950 tokens, 4.2 items per SM: 85 against 98; 64 sequences, 12 per SM: 263 against 298).
+static kv_status_t choose_schedule(const kv_pool_t* p, int n_q_heads, int batch, int total_q, int max_extend_len, int max_total_len,
+                                   size_t workspace_bytes, int* sched, int* splits) {
+  *sched = kSchedList;
+  *splits = 1;
+  const int G = n_q_heads / p->n_kv_heads, sms = sm_count_of(p->device);
+  const int64_t units = (int64_t)batch * (((int64_t)max_extend_len * G + 255) / 256) * p->n_kv_heads;
+  const int64_t steps = ((int64_t)max_total_len + 127) / 128;
+  const SpanLayout l = span_layout(p, n_q_heads, batch, total_q, max_total_len);
+  const bool room = workspace_bytes >= 256 + l.total;  // (else: nothing that leaves partial results)
+  if (units <= sms) {
+    *sched = kSchedCluster;
+    if (!room || !l.cuts) return KV_OK;
+    for (int c : kSplitChoices) {
+      if (c > steps) break;
+      int resident = 0;
+      const kv_status_t s = p->head_dim == 128 ? resident_clusters<128>(p->device, c, &resident) : resident_clusters<64>(p->device, c, &resident);
+      if (s != KV_OK) return s;
+      if (units <= resident) *splits = c;
+    }
+    // (steps of the longest item on its CTAs, against those of all items spread evenly, which are somewhat shorter)
+    if ((double)steps / *splits - 0.85 * (double)steps * units / sms > 12.0) *sched = kSchedSpans;
+  } else if (room && steps >= 32 && items_at_most(p, n_q_heads, batch, total_q) <= 3ll * sms) {
+    *sched = kSchedSpans;
+  }
+  return KV_OK;
+}
+
+static SpanArgs span_args(const SpanLayout& l, char* ws, int max_tp, int total_q, int cta_cap) {
+  SpanArgs a{};
+  a.n_spans = l.n_spans;  // (not the number of CTAs: the cuts, and with them the bits, are the same beside a decode kernel)
+  a.per_cta = cta_cap > 0 ? (l.n_spans + cta_cap - 1) / cta_cap : 1;
+  a.max_tp = max_tp;
+  a.total_q = total_q;
+  a.desc = reinterpret_cast<int4*>(ws);
+  a.part_lse = l.cuts ? reinterpret_cast<float*>(ws + l.lse) : nullptr;
+  a.part_o = l.cuts ? reinterpret_cast<float*>(ws + l.o) : nullptr;
+  return a;
+}
+static char* align_workspace(void* ws) {
+  return reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(ws) + 255) & ~(uintptr_t)255);
+}
+
+// Merges the chunks of cut items behind a span-scheduled attention kernel; nothing to do for other batches.  early: that
+// kernel is the one queued last.
+kv_status_t launch_extend_combine(kv_pool_t* p, int n_q_heads, int batch, int total_q, int max_extend_len, int max_total_len, void* out, float* lse,
+                                  void* workspace, size_t workspace_bytes, bool early, cudaStream_t st) {
+  int sched, splits;
+  const kv_status_t cs = choose_schedule(p, n_q_heads, batch, total_q, max_extend_len, max_total_len, workspace_bytes, &sched, &splits);
+  if (cs != KV_OK) return cs;
+  if (sched != kSchedSpans) return KV_OK;
+  const SpanLayout l = span_layout(p, n_q_heads, batch, total_q, max_total_len);
+  if (!l.cuts || l.n_spans < 2) return KV_OK;
+  const int G = n_q_heads / p->n_kv_heads;
+  int lg = 0;
+  while ((1 << lg) < G) ++lg;
+  const SpanArgs a = span_args(l, align_workspace(workspace), 0, total_q, 0);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)((a.n_spans - 1) * kCombineSlices));
+  cfg.blockDim = dim3((unsigned)p->head_dim * 4);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = early_start ? 1 : 0;
-  KV_CUDA_OK(cudaLaunchKernelEx(&cfg, attn_extend_tc_kernel<D, OPT, FAN>, a, q_map));
+  cfg.numAttrs = early ? 1 : 0;
+  if (p->head_dim == 128)
+    KV_CUDA_OK(cudaLaunchKernelEx(&cfg, span_combine_kernel<128>, a, n_q_heads, G, lg, (__nv_bfloat16*)out, lse));
+  else
+    KV_CUDA_OK(cudaLaunchKernelEx(&cfg, span_combine_kernel<64>, a, n_q_heads, G, lg, (__nv_bfloat16*)out, lse));
   count_launch();
   return KV_OK;
 }
@@ -1140,7 +1784,7 @@ kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const i
                              const AppendArgs* app, int phase, cudaStream_t st) {
   // phase 0: plan (with the suffix append, if any) and attention; 1: the plan only; 2: attention over the plan that a
   // phase-1 call with the same arguments left in the workspace
-  const size_t need = extend_tc_workspace_bytes(n_q_heads, p->head_dim, batch, total_q, max_total_len);
+  const size_t need = extend_tc_min_workspace_bytes(batch, total_q);
   if (workspace == nullptr || workspace_bytes < need) return KV_ERR_WORKSPACE;
   const int G = n_q_heads / p->n_kv_heads;
   // Q is read through a tensor map (16-byte base), O is written with 32-byte stores
@@ -1152,8 +1796,9 @@ kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const i
   }
   int lg = 0;
   while ((1 << lg) < G) ++lg;
-  int* n_items = reinterpret_cast<int*>(workspace);
-  int4* items = reinterpret_cast<int4*>(reinterpret_cast<char*>(workspace) + 256);
+  char* ws = align_workspace(workspace);
+  int* n_items = reinterpret_cast<int*>(ws);
+  int4* items = reinterpret_cast<int4*>(ws + 256);
   const int64_t capacity = item_capacity(n_q_heads, p->n_kv_heads, batch, total_q);
   const int max_tp = (int)(((int64_t)max_extend_len * G + 255) / 256);
   const int max_steps = 2 * ((max_total_len + 127) / 128);
@@ -1171,9 +1816,24 @@ kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const i
   groups = groups < 1 ? 1 : groups;
   groups = groups > batch ? batch : groups;
   groups = groups > kPlanBuckets / 16 ? kPlanBuckets / 16 : groups;
+  int sched = kSchedList, splits = 1;
+  if (mode == 0) {
+    const kv_status_t cs = choose_schedule(p, n_q_heads, batch, total_q, max_extend_len, max_total_len, workspace_bytes, &sched, &splits);
+    if (cs != KV_OK) return cs;
+  }
   const PlanArgs pa{prefix_lens, extend_lens, cu_q, batch, max_tp, lg, max_steps, (int)capacity, max_pages, mode,
                     fan != nullptr ? *fan : FanArgs{}, groups, p->d_status, items, n_items, n_items + 1, grid};
-  if (phase == 2) {
+  if (sched != kSchedList) {
+    // no plan: the attention kernel's CTAs find their work themselves
+    if (phase == 1) return KV_OK;
+    if (app != nullptr && app->total_new > 0) {
+      const int64_t want = ((int64_t)app->total_new + 31) / 32;
+      const int64_t cap = 2 * (int64_t)sm_count_of(p->device);
+      append_prologue_kernel<<<(int)(want < cap ? want : cap), 1024, 0, st>>>(p->view(), *app);
+      count_launch();
+      KV_CUDA_OK(cudaGetLastError());
+    }
+  } else if (phase == 2) {
     // the plan is in the workspace already
   } else if (app != nullptr && app->total_new > 0) {
     // plan block + append blocks (32 warps each, one warp per token, all blocks resident at once)
@@ -1184,7 +1844,7 @@ kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const i
   } else {
     extend_tc_plan_kernel<<<1, 1024, 0, st>>>(pa);
   }
-  if (phase != 2) {
+  if (phase != 2 && sched == kSchedList) {
     count_launch();
     KV_CUDA_OK(cudaGetLastError());
   }
@@ -1213,19 +1873,38 @@ kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const i
   // Skipping the search for the row maximum pays where items have many KV steps (measured: +2 % on the
   // long-document shapes, -1 % on the 8B extend batch whose items have a dozen steps)
   const bool opt = max_total_len >= kOptimisticMinLen;
-  const bool early = cta_cap >= 0;
+  bool early = cta_cap >= 0;
+  if (sched != kSchedList) {
+    a.span = span_args(span_layout(p, n_q_heads, batch, total_q, max_total_len), ws, max_tp, total_q, sched == kSchedSpans ? cta_cap : 0);
+    a.span.plan_early = app != nullptr && app->total_new > 0;
+    a.cl_splits = splits;
+    grid = sched == kSchedSpans ? (a.span.n_spans + a.span.per_cta - 1) / a.span.per_cta : batch * max_tp * p->n_kv_heads * splits;
+    // (beside a decode kernel that waits for nothing, this kernel has to start behind all that was queued before it)
+    if (cta_cap > 0) early = false;
+  }
   auto go = [&](auto d, auto o, auto f) {
-    return launch_tc<decltype(d)::value, decltype(o)::value, decltype(f)::value>(a, q_map, grid, p->device, early, st);
+    constexpr int DD = decltype(d)::value;
+    constexpr bool OO = decltype(o)::value, FF = decltype(f)::value;
+    if constexpr (!FF) {
+      if (sched == kSchedSpans) return launch_tc<DD, OO, false, kSchedSpans>(a, q_map, grid, p->device, early, st);
+      if (sched == kSchedCluster) return launch_tc<DD, OO, false, kSchedCluster>(a, q_map, grid, p->device, early, st);
+    }
+    return launch_tc<DD, OO, FF, kSchedList>(a, q_map, grid, p->device, early, st);
   };
   using I128 = std::integral_constant<int, 128>;
   using I64 = std::integral_constant<int, 64>;
   const bool fan_mode = mode == 2;
+  kv_status_t ls;
   if (p->head_dim == 128) {
-    if (fan_mode) return opt ? go(I128{}, std::true_type{}, std::true_type{}) : go(I128{}, std::false_type{}, std::true_type{});
-    return opt ? go(I128{}, std::true_type{}, std::false_type{}) : go(I128{}, std::false_type{}, std::false_type{});
+    if (fan_mode) ls = opt ? go(I128{}, std::true_type{}, std::true_type{}) : go(I128{}, std::false_type{}, std::true_type{});
+    else ls = opt ? go(I128{}, std::true_type{}, std::false_type{}) : go(I128{}, std::false_type{}, std::false_type{});
+  } else if (fan_mode) {
+    ls = opt ? go(I64{}, std::true_type{}, std::true_type{}) : go(I64{}, std::false_type{}, std::true_type{});
+  } else {
+    ls = opt ? go(I64{}, std::true_type{}, std::false_type{}) : go(I64{}, std::false_type{}, std::false_type{});
   }
-  if (fan_mode) return opt ? go(I64{}, std::true_type{}, std::true_type{}) : go(I64{}, std::false_type{}, std::true_type{});
-  return opt ? go(I64{}, std::true_type{}, std::false_type{}) : go(I64{}, std::false_type{}, std::false_type{});
+  if (ls != KV_OK || sched != kSchedSpans || cta_cap > 0) return ls;
+  return launch_extend_combine(p, n_q_heads, batch, total_q, max_extend_len, max_total_len, out, lse, workspace, workspace_bytes, true, st);
 }
 
 }  // namespace kvattn

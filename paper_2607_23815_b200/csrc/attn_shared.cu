@@ -17,7 +17,7 @@
 
 namespace kvattn {
 
-size_t extend_tc_workspace_bytes(int n_q_heads, int head_dim, int batch, int total_q, int max_total_len);
+size_t extend_tc_min_workspace_bytes(int batch, int total_q);
 bool extend_tc_supported(const kv_pool_t* p, int n_q_heads);
 kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const int* cu_q, const int* block_tables,
                              int max_pages, const int* prefix_lens, const int* extend_lens, int batch, int total_q,
@@ -107,12 +107,11 @@ __global__ void __launch_bounds__(256) shared_merge_kernel(const __nv_bfloat16* 
 
 size_t extend_shared_workspace_bytes(const kv_pool_t* p, int n_q_heads, int n_parents, int n_children, int total_q,
                                      int max_parent_len) {
+  (void)max_parent_len;
   if (n_parents <= 0 || n_children <= 0 || total_q <= 0) return 0;
   return align256(sizeof(int) * (size_t)(2 * n_parents + 1 + n_children)) +
          align256((size_t)total_q * n_q_heads * p->head_dim * 2) + align256((size_t)total_q * n_q_heads * 4) +
-         align256(extend_tc_workspace_bytes(n_q_heads, p->head_dim, n_children > n_parents ? n_children : n_parents, total_q,
-                                            max_parent_len)) +
-         256;
+         align256(extend_tc_min_workspace_bytes(n_children > n_parents ? n_children : n_parents, total_q)) + 256;
 }
 
 kv_status_t launch_extend_shared(kv_pool_t* p, const void* q, int n_q_heads, const int* cu_q, const int* cu_children,
@@ -133,8 +132,7 @@ kv_status_t launch_extend_shared(kv_pool_t* p, const void* q, int n_q_heads, con
   ws += align256((size_t)total_q * n_q_heads * p->head_dim * 2);
   float* lse_a = reinterpret_cast<float*>(ws);
   ws += align256((size_t)total_q * n_q_heads * 4);
-  const size_t tc_bytes = extend_tc_workspace_bytes(n_q_heads, p->head_dim, n_children > n_parents ? n_children : n_parents,
-                                                    total_q, max_parent_len);
+  const size_t tc_bytes = extend_tc_min_workspace_bytes(n_children > n_parents ? n_children : n_parents, total_q);
 
   const int n_prep = (n_parents + 1 > n_children ? n_parents + 1 : n_children);
   shared_prep_kernel<<<(n_prep + 255) / 256, 256, 0, st>>>(cu_q, cu_children, n_parents, n_children, cu_q_parent, rows_parent,
