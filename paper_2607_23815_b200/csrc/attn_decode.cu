@@ -12,6 +12,8 @@
 // measured on 20 batch shapes: twelve warps on an SM beat eight everywhere (a slot is refilled as soon as its page is
 // in registers, so two are enough), and two CTAs of six beat one of twelve on short contexts (128 sequences of 200-700:
 // 40.5 against 47.8 us) because one starts while the other ends.
+#include <math.h>
+
 #include "common.cuh"
 #include "page_mma.cuh"
 #include "sm100_ptx.cuh"
@@ -349,22 +351,41 @@ static kv_status_t resident_clusters(int device, int i, int* n) {
 //  - As many as fit on the device at once: a second wave of clusters costs more than the shorter runs save (8 sequences
 //    of 1000-4000 tokens: 22.1 / 19.0 / 22.2 us with 2 / 4 / 8), but not more warps than about 3/2 of the sequence's
 //    pages (517 tokens: 4.6 / 4.2 / 4.4 us with 4 / 8 / 16).
-//  - Long sequences are split even when the batch fills the device many times over, so that the last CTAs to finish
-//    hold less: 64 x 1024-4096 tokens 100.7 -> 94.1 us with 2, 40 x 4000-16000 245 / 230 / 220 us with 1 / 2 / 4; below
-//    192 pages it costs (128 x 200-700: 40.5 against 54.4; 24 x 1000-3000, 64/8 heads: 39.0 against 42.8).
+//  - Where that leaves SMs idle, more, by what the last wave costs.  A wave of less than kFull of the CTAs the device
+//    holds is as slow as one of kFull (the memory is saturated with 0.65 of them at 128 dims, hardly with all at 64):
+//    32 x 5100 tokens, 64 dims: 49 / 51 / 42.6 us with 1 / 2 / 3, 64 x 3000: 77 / 70 / 69.6; 20 x 12000, 128 dims: 163 /
+//    179 / 151.  Every further CTA costs about 4 % at 192 pages.
+//  - Long sequences of different lengths are split even when the batch fills the device many times over, so that the last
+//    CTAs to finish hold less: 64 x 1024-4096 tokens 100.7 -> 94.1 us with 2, 32 x 3230-5100 88.6 -> 83.3; with runs below
+//    128 pages it costs (128 x 200-700: 40.5 against 54.4; 24 x 1000-3000, 64/8 heads: 39.0 against 42.8).
 template <int D>
 static kv_status_t decode_splits(const kv_pool_t* p, int batch, int max_ctx_len, int* splits) {
   const int64_t units = (int64_t)batch * p->n_kv_heads;
   const int pages = (int)(((int64_t)max_ctx_len + kPageSize - 1) / kPageSize);
-  const int by_length = pages >= 640 ? 4 : pages >= 192 ? 2 : 1;
+  constexpr int kChoices = (int)(sizeof(kSplitChoices) / sizeof(int));
+  int resident[kChoices];
   *splits = 1;
-  for (int i = 0; i < (int)(sizeof(kSplitChoices) / sizeof(int)); ++i) {
-    const int c = kSplitChoices[i];
-    if (2 * kWarps * c > 3 * pages) break;
-    int resident = 0;
-    const kv_status_t s = resident_clusters<D>(p->device, i, &resident);
+  for (int i = 0; i < kChoices; ++i) {
+    const kv_status_t s = resident_clusters<D>(p->device, i, &resident[i]);
     if (s != KV_OK) return s;
-    if (units <= resident || (c <= by_length && resident > 0)) *splits = c;
+    if (2 * kWarps * kSplitChoices[i] <= 3 * pages && units <= resident[i]) *splits = kSplitChoices[i];
+  }
+  constexpr double kFull = D == 128 ? 0.65 : 0.9;
+  auto score = [&](int c) {
+    const double waves = (double)units * c / (resident[0] > 0 ? resident[0] : 1), whole = floor(waves), last = waves - whole;
+    const double per_cta = 1.0 + 0.04 * (c - 1) * 192.0 / pages;
+    return waves / (whole + (last > 0 ? (last > kFull ? last : kFull) : 0.0)) / per_cta;
+  };
+  const int cap = pages >= 640 ? 4 : 3;
+  double best = score(*splits);
+  for (int i = 0; i < kChoices; ++i) {
+    const int c = kSplitChoices[i];
+    if (c <= *splits || c > cap || pages < 48 * c || resident[i] == 0) continue;
+    const double sc = score(c);
+    if (sc > best || (pages >= 128 * c && sc > 0.9 * best)) {
+      *splits = c;
+      best = sc > best ? sc : best;
+    }
   }
   return KV_OK;
 }

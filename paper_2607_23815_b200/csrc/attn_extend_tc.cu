@@ -25,6 +25,8 @@
 // The two query tiles ping-pong: while one tile's softmax runs, the tensor core works on the other.
 // All waits are bounded; on expiry the CTA records KV_ERR_TIMEOUT, drains its copies, frees its
 // tensor memory and returns.
+#include <math.h>
+
 #include <type_traits>
 
 #include <cuda.h>  // CUtensorMap and its enums (types only: the encoder is looked up at run time)
@@ -1700,10 +1702,10 @@ static kv_status_t resident_clusters(int device, int c, int* n) {
 //    behind 1000-2000 (32/8 heads of 128): 32.1 / 38.2 / 42.2 / 43.7 us through the list, 16.8 / 24.2 / 33.3 / 42.4 this
 //    way with 6 / 4 / 2 / 1 CTAs per item.
 //  - Few and long items: spans.  They cost a merge kernel behind the attention kernel (about 12 us, 8 steps) and win what
-//    the other two leave idle, the part of a cluster that no SM group holds or the last items of the list: 8 / 16
-//    sequences of 9000-16000 keys 219 / 225 us through the list, 121 / 242 with clusters, 102 / 181 with spans; 11 of up
-//    to 10700 (16/8 heads of 64) 260 and 197.  More than three items per SM, or short ones: the list (3 prefills of up to
-//    1950 tokens, 4.2 items per SM: 85 against 98; 64 sequences, 12 per SM: 263 against 298).
+//    the other two leave idle, the SMs without a cluster or the last round of items: 8 / 16 sequences of 9000-16000 keys
+//    219 / 225 us through the list, 121 / 242 with clusters, 102 / 181 with spans; 11 of up to 10700 (16/8 heads of 64)
+//    260 and 197; but 4 of 6900 with 128 items of equal length 112 and 120.  More than three items per SM, or short ones:
+//    the list (3 prefills of up to 1950 tokens, 4.2 items per SM: 85 against 98; 64 sequences, 12 per SM: 263 against 298).
 static kv_status_t choose_schedule(const kv_pool_t* p, int n_q_heads, int batch, int total_q, int max_extend_len, int max_total_len,
                                    size_t workspace_bytes, int* sched, int* splits) {
   *sched = kSchedList;
@@ -1713,7 +1715,10 @@ static kv_status_t choose_schedule(const kv_pool_t* p, int n_q_heads, int batch,
   const int64_t steps = ((int64_t)max_total_len + 127) / 128;
   const SpanLayout l = span_layout(p, n_q_heads, batch, total_q, max_total_len);
   const bool room = workspace_bytes >= 256 + l.total;  // (else: nothing that leaves partial results)
-  if (units <= sms) {
+  const int64_t most = items_at_most(p, n_q_heads, batch, total_q);
+  // (a sequence's last tile pair is half full on average, its keys somewhat fewer than the longest's)
+  const double rounds = ((double)total_q * G / 256 + 0.5 * batch) * p->n_kv_heads / sms, even = 0.85 * steps * rounds;
+  if (units <= sms || (most <= sms && units <= 2 * sms)) {
     *sched = kSchedCluster;
     if (!room || !l.cuts) return KV_OK;
     for (int c : kSplitChoices) {
@@ -1723,9 +1728,8 @@ static kv_status_t choose_schedule(const kv_pool_t* p, int n_q_heads, int batch,
       if (s != KV_OK) return s;
       if (units <= resident) *splits = c;
     }
-    // (steps of the longest item on its CTAs, against those of all items spread evenly, which are somewhat shorter)
-    if ((double)steps / *splits - 0.85 * (double)steps * units / sms > 12.0) *sched = kSchedSpans;
-  } else if (room && steps >= 32 && items_at_most(p, n_q_heads, batch, total_q) <= 3ll * sms) {
+    if ((double)steps / *splits - even > 12.0) *sched = kSchedSpans;
+  } else if (room && l.cuts && most <= 3ll * sms && 0.85 * steps * ceil(rounds) - even > 16.0) {
     *sched = kSchedSpans;
   }
   return KV_OK;
