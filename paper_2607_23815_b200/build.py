@@ -1,4 +1,4 @@
-"""Builds the CUDA shared library in-tree with nvcc for sm_100a.
+"""Builds the CUDA shared library in-tree with nvcc for sm_100a, and the native half of the Python binding with g++.
 
     python -m paper_2607_23815_b200.build          # (re)build if sources are newer
     python -m paper_2607_23815_b200.build --force
@@ -9,10 +9,12 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libkvattn.so")
+BINDING = os.path.join(HERE, "_kvattn_native.so")
 SOURCES = ["pool.cu", "attn_small.cu", "attn_decode.cu", "attn_extend_tc.cu", "attn_decode_static.cu", "attn_shared.cu", "selftest.cu", "api.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "--shared", "-Xcompiler", "-fPIC", "-Xptxas", "-v"]
@@ -25,23 +27,42 @@ def _nvcc() -> str:
     raise RuntimeError("nvcc not found: the CUDA toolkit is needed to build libkvattn.so")
 
 
-def _stale() -> bool:
-    if not os.path.exists(LIB):
+def _stale(target: str, suffixes) -> bool:
+    if not os.path.exists(target):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(HERE, "..", "include", "kvattn.h")]
+    t = os.path.getmtime(target)
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(suffixes)] + [os.path.join(HERE, "..", "include", "kvattn.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
-def build_library(force: bool = False, verbose: bool = False) -> str:
-    if not force and not _stale():
-        return LIB
-    cmd = [_nvcc()] + NVCC_FLAGS + ["-o", LIB] + [os.path.join(CSRC, s) for s in SOURCES]
+def _run(cmd, verbose: bool, what: str) -> None:
     res = subprocess.run(cmd, capture_output=True, text=True)
     if verbose or res.returncode != 0:
         sys.stderr.write(res.stdout + res.stderr)
     if res.returncode != 0:
-        raise RuntimeError("nvcc failed building libkvattn.so")
+        raise RuntimeError(f"building {what} failed")
+
+
+def build_binding(force: bool = False, verbose: bool = False) -> str:
+    """The extension module that unpacks torch tensors and calls libkvattn.so (which lies beside it)."""
+    if not force and not _stale(BINDING, (".cpp",)):
+        return BINDING
+    import torch
+    from torch.utils import cpp_extension as ext
+    libs = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cuda = os.path.dirname(os.path.dirname(_nvcc()))
+    inc = ext.include_paths() + [os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
+    _run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+         + [f"-I{d}" for d in inc] + [os.path.join(CSRC, "binding.cpp"), "-o", BINDING, LIB, "-Wl,-rpath,$ORIGIN", f"-L{libs}",
+                                      "-lc10", "-lc10_cuda", "-ltorch", "-ltorch_cpu", "-ltorch_python"], verbose, "_kvattn_native.so")
+    return BINDING
+
+
+def build_library(force: bool = False, verbose: bool = False) -> str:
+    if force or _stale(LIB, (".cu", ".cuh")):
+        _run([_nvcc()] + NVCC_FLAGS + ["-Xlinker", "-soname=libkvattn.so", "-o", LIB] + [os.path.join(CSRC, s) for s in SOURCES],
+             verbose, "libkvattn.so")
+    build_binding(force, verbose)
     return LIB
 
 

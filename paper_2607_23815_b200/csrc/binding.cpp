@@ -1,0 +1,241 @@
+// Native half of the Python binding: unpacks torch tensors and calls the C ABI.
+//
+// A call of the library is worth 3-7 us of host time (one to two kernel launches).  Marshalling the arguments of such a
+// call through ctypes cost as much again and more (attn_decode 11.1 us, of which 4.2 in the library; attn_extend_append
+// 15.6 and 7.2), which bounded every small call: the kernel behind a decode of one sequence takes 4.2 us.
+#include <Python.h>
+
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include "../../include/kvattn.h"
+
+namespace {
+
+// Thrown with a Python exception set.
+struct Raised {};
+
+[[noreturn]] void raise(PyObject* type, const char* what) {
+  PyErr_SetString(type, what);
+  throw Raised{};
+}
+
+const at::Tensor& tensor(PyObject* o) {
+  if (!THPVariable_Check(o)) raise(PyExc_TypeError, "expected a torch tensor");
+  const at::Tensor& t = THPVariable_Unpack(o);
+  if (!t.is_contiguous()) raise(PyExc_AssertionError, "tensors passed to the library must be contiguous");
+  if (!t.is_cuda()) raise(PyExc_AssertionError, "expected a CUDA tensor");
+  return t;
+}
+
+void* data(const at::Tensor& t) { return const_cast<void*>(t.const_data_ptr()); }
+template <typename T = void>
+T* ptr(PyObject* o) { return o == Py_None ? nullptr : static_cast<T*>(data(tensor(o))); }
+int size(const at::Tensor& t, int dim) {
+  if (dim >= t.dim()) raise(PyExc_IndexError, "tensor has too few dimensions");
+  return (int)t.size(dim);
+}
+
+int integer(PyObject* o) {
+  const long v = PyLong_AsLong(o);
+  if (v == -1 && PyErr_Occurred()) throw Raised{};
+  return (int)v;
+}
+float real(PyObject* o) {
+  const double v = PyFloat_AsDouble(o);
+  if (v == -1.0 && PyErr_Occurred()) throw Raised{};
+  return (float)v;
+}
+kv_pool_t* pool(PyObject* o) {
+  if (o == Py_None) return nullptr;
+  void* p = PyLong_AsVoidPtr(o);
+  if (p == nullptr && PyErr_Occurred()) throw Raised{};
+  return static_cast<kv_pool_t*>(p);
+}
+// None: torch's current stream; else a stream object or its handle.
+void* stream(PyObject* o) {
+  if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
+  if (PyLong_Check(o)) return PyLong_AsVoidPtr(o);
+  PyObject* h = PyObject_GetAttrString(o, "cuda_stream");
+  if (h == nullptr) throw Raised{};
+  void* p = PyLong_AsVoidPtr(h);
+  Py_DECREF(h);
+  if (p == nullptr && PyErr_Occurred()) throw Raised{};
+  return p;
+}
+struct Workspace {
+  void* p = nullptr;
+  size_t bytes = 0;
+  explicit Workspace(PyObject* o) {
+    if (o == Py_None) return;
+    const at::Tensor& t = tensor(o);
+    p = data(t);
+    bytes = t.nbytes();
+  }
+};
+// A ctypes structure (or None).
+struct Struct {
+  Py_buffer view{};
+  explicit Struct(PyObject* o) {
+    if (o != Py_None && PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) throw Raised{};
+  }
+  ~Struct() {
+    if (view.obj != nullptr) PyBuffer_Release(&view);
+  }
+  template <typename T>
+  const T* as() const {
+    if (view.buf == nullptr) return nullptr;
+    if (view.len != (Py_ssize_t)sizeof(T)) raise(PyExc_TypeError, "argument structure of the wrong size");
+    return static_cast<const T*>(view.buf);
+  }
+};
+
+// Runs body(args), which returns a function to be called without the interpreter lock, and returns its status.
+template <typename Body>
+PyObject* call(Py_ssize_t got, Py_ssize_t want, Body body) {
+  if (got != want) {
+    PyErr_SetString(PyExc_TypeError, "wrong number of arguments");
+    return nullptr;
+  }
+  try {
+    return PyLong_FromLong(body());
+  } catch (const Raised&) {
+    return nullptr;
+  } catch (const std::exception& e) {
+    PyErr_SetString(PyExc_RuntimeError, e.what());
+    return nullptr;
+  }
+}
+template <typename F>
+long unlocked(F f) {
+  long status;
+  Py_BEGIN_ALLOW_THREADS;
+  status = f();
+  Py_END_ALLOW_THREADS;
+  return status;
+}
+
+PyObject* append(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return call(n, 8, [&] {
+    kv_pool_t* p = pool(a[0]);
+    const at::Tensor &k = tensor(a[1]), &start = tensor(a[4]), &bt = tensor(a[6]);
+    void *v = ptr(a[2]), *st = stream(a[7]);
+    const int *cu = ptr<int>(a[3]), *row = ptr<int>(a[5]);
+    const int pages = size(bt, 1), segs = (int)start.numel(), total = size(k, 0);
+    return unlocked([&] {
+      return kv_append(p, data(k), v, cu, (const int*)data(start), row, (const int*)data(bt), pages, segs, total, st);
+    });
+  });
+}
+
+PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return call(n, 10, [&] {
+    kv_pool_t* p = pool(a[0]);
+    const at::Tensor &q = tensor(a[1]), &bt = tensor(a[2]);
+    const int* ctx = ptr<int>(a[3]);
+    const int max_ctx = integer(a[4]), hq = size(q, 1), pages = size(bt, 1), batch = size(q, 0);
+    const float scale = real(a[5]);
+    void *out = ptr(a[6]), *st = stream(a[9]);
+    float* lse = ptr<float>(a[7]);
+    const Workspace ws(a[8]);
+    return unlocked([&] {
+      return attn_decode(p, data(q), hq, (const int*)data(bt), pages, ctx, batch, max_ctx, scale, out, lse, ws.p, ws.bytes, st);
+    });
+  });
+}
+
+// what attn_extend, attn_extend_planned and attn_extend_append share
+template <typename F>
+PyObject* extend_like(PyObject* const* a, Py_ssize_t n, int lead, F f) {  // lead: arguments before cu_q
+  return call(n, lead + 11, [&] {
+    kv_pool_t* p = pool(a[0]);
+    const at::Tensor& q = tensor(a[1]);
+    PyObject* const* b = a + lead;
+    const at::Tensor &bt = tensor(b[1]), &pl = tensor(b[2]);
+    const int *cu = ptr<int>(b[0]), *el = ptr<int>(b[3]);
+    const int max_e = integer(b[4]), max_l = integer(b[5]), hq = size(q, 1), total = size(q, 0), pages = size(bt, 1);
+    const float scale = real(b[6]);
+    void *out = ptr(b[7]), *st = stream(b[10]);
+    float* lse = ptr<float>(b[8]);
+    const Workspace ws(b[9]);
+    void *k = lead == 4 ? ptr(a[2]) : nullptr, *v = lead == 4 ? ptr(a[3]) : nullptr;
+    return unlocked([&] {
+      return f(p, data(q), k, v, hq, cu, (const int*)data(bt), pages, (const int*)data(pl), el, (int)pl.numel(), total, max_e, max_l,
+               scale, out, lse, ws.p, ws.bytes, st);
+    });
+  });
+}
+PyObject* extend(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return extend_like(a, n, 2, [](kv_pool_t* p, const void* q, const void*, const void*, auto... rest) { return attn_extend(p, q, rest...); });
+}
+PyObject* extend_planned(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return extend_like(a, n, 2, [](kv_pool_t* p, const void* q, const void*, const void*, auto... rest) { return attn_extend_planned(p, q, rest...); });
+}
+PyObject* extend_append(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return extend_like(a, n, 4, [](auto... all) { return attn_extend_append(all...); });
+}
+
+PyObject* extend_plan(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return call(n, 11, [&] {
+    kv_pool_t* p = pool(a[0]);
+    const int hq = integer(a[1]), total = integer(a[6]), max_e = integer(a[7]), max_l = integer(a[8]);
+    const at::Tensor &bt = tensor(a[3]), &pl = tensor(a[4]);
+    const int *cu = ptr<int>(a[2]), *el = ptr<int>(a[5]);
+    const int pages = size(bt, 1);
+    const Workspace ws(a[9]);
+    void* st = stream(a[10]);
+    return unlocked([&] {
+      return attn_extend_plan(p, hq, cu, (const int*)data(bt), pages, (const int*)data(pl), el, (int)pl.numel(), total, max_e, max_l,
+                              ws.p, ws.bytes, st);
+    });
+  });
+}
+
+PyObject* extend_shared(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return call(n, 16, [&] {
+    kv_pool_t* p = pool(a[0]);
+    const at::Tensor &q = tensor(a[1]), &pt = tensor(a[4]), &pl = tensor(a[5]), &ct = tensor(a[6]), &cl = tensor(a[7]);
+    const int *cu = ptr<int>(a[2]), *cc = ptr<int>(a[3]);
+    const int max_c = integer(a[8]), max_rows = integer(a[9]), max_p = integer(a[10]);
+    const int hq = size(q, 1), total = size(q, 0), pages_p = size(pt, 1), pages_c = size(ct, 1);
+    const float scale = real(a[11]);
+    void *out = ptr(a[12]), *st = stream(a[15]);
+    float* lse = ptr<float>(a[13]);
+    const Workspace ws(a[14]);
+    return unlocked([&] {
+      return attn_extend_shared(p, data(q), hq, cu, cc, (const int*)data(pt), pages_p, (const int*)data(pl), (const int*)data(ct), pages_c,
+                                (const int*)data(cl), (int)pl.numel(), (int)cl.numel(), total, max_c, max_rows, max_p, scale, out, lse,
+                                ws.p, ws.bytes, st);
+    });
+  });
+}
+
+PyObject* mixed(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return call(n, 7, [&] {
+    kv_pool_t* p = pool(a[0]);
+    const int hq = integer(a[1]);
+    const float scale = real(a[2]);
+    const Struct ext(a[3]), dec(a[4]);
+    const auto* e = ext.as<attn_extend_args_t>();
+    const auto* d = dec.as<attn_decode_args_t>();
+    const Workspace ws(a[5]);
+    void* st = stream(a[6]);
+    return unlocked([&] { return attn_mixed(p, hq, scale, e, d, ws.p, ws.bytes, st); });
+  });
+}
+
+#define ENTRY(name, fn) {name, (PyCFunction)(void (*)(void))fn, METH_FASTCALL, nullptr}
+PyMethodDef methods[] = {ENTRY("kv_append", append),
+                         ENTRY("attn_decode", decode),
+                         ENTRY("attn_extend", extend),
+                         ENTRY("attn_extend_append", extend_append),
+                         ENTRY("attn_extend_plan", extend_plan),
+                         ENTRY("attn_extend_planned", extend_planned),
+                         ENTRY("attn_extend_shared", extend_shared),
+                         ENTRY("attn_mixed", mixed),
+                         {nullptr, nullptr, 0, nullptr}};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_kvattn_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__kvattn_native(void) { return PyModule_Create(&module); }

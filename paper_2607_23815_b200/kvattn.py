@@ -1,11 +1,13 @@
-"""Thin ctypes binding of include/kvattn.h: same names, argument marshalling only.
+"""Thin binding of include/kvattn.h: same names, argument marshalling only.
 
 Tensors are torch tensors used as device memory; every step of the path runs in the library's
-kernels.  There is no CPU fallback: if the shared library is missing the import fails.
+kernels.  The calls that launch work on tensors go through a native module (csrc/binding.cpp), the
+others through ctypes.  There is no CPU fallback: if the shared library is missing the import fails.
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib
 import os
 from typing import Optional, Sequence
 
@@ -99,6 +101,23 @@ def lib():
     return _lib
 
 
+class _NativeLoader:
+    """Stands in for the native module until its first use."""
+
+    def __getattr__(self, name):
+        global _native
+        lib()
+        try:
+            module = importlib.import_module("._kvattn_native", __package__)
+        except ImportError as e:
+            raise ImportError("the native binding is missing or stale: build it with `python -m paper_2607_23815_b200.build`") from e
+        _native = module
+        return getattr(module, name)
+
+
+_native = _NativeLoader()
+
+
 def _ptr(t: Optional[torch.Tensor]):
     if t is None:
         return None
@@ -141,11 +160,13 @@ class Pool:
             st = lib().kv_pool_create_ex(num_pages, page_size, n_kv_heads, head_dim, _dev_ptr(k_base),
                                          _dev_ptr(v_base), C.byref(self.handle))
         _check(st, "kv_pool_create")
+        self.ptr = self.handle.value                                 # the handle as the native module takes it
 
     def destroy(self):
         if self.handle:
             lib().kv_pool_destroy(self.handle)
             self.handle = C.c_void_p()
+            self.ptr = None
 
     def __del__(self):
         try:
@@ -235,10 +256,7 @@ def kv_page_info(pool: Pool, page: int):
 
 
 def kv_append(pool: Pool, k_new, v_new, cu_new, start_pos, seg_row, block_tables, stream=None):
-    n_seg = start_pos.numel()
-    _check(lib().kv_append(pool.handle, _dev_ptr(k_new), _dev_ptr(v_new), _dev_ptr(cu_new), _dev_ptr(start_pos),
-                           _dev_ptr(seg_row), _dev_ptr(block_tables), block_tables.shape[1], n_seg,
-                           k_new.shape[0], _stream(stream)), "kv_append")
+    _check(_native.kv_append(pool.ptr, k_new, v_new, cu_new, start_pos, seg_row, block_tables, stream), "kv_append")
 
 
 def kv_gather(pool: Pool, block_table_row, length, k_out, v_out, stream=None):
@@ -254,42 +272,29 @@ def attn_workspace_bytes(pool: Pool, n_q_heads, batch_ext=0, total_q=0, max_tota
 
 def attn_extend(pool: Pool, q, cu_q, block_tables, prefix_lens, extend_lens, max_extend_len, max_total_len, scale,
                 out, lse, workspace=None, stream=None):
-    _check(lib().attn_extend(pool.handle, _dev_ptr(q), q.shape[1], _dev_ptr(cu_q), _dev_ptr(block_tables),
-                             block_tables.shape[1], _dev_ptr(prefix_lens), _dev_ptr(extend_lens),
-                             prefix_lens.numel(), q.shape[0], max_extend_len, max_total_len, float(scale),
-                             _dev_ptr(out), _dev_ptr(lse), _dev_ptr(workspace),
-                             0 if workspace is None else workspace.numel() * workspace.element_size(),
-                             _stream(stream)), "attn_extend")
+    _check(_native.attn_extend(pool.ptr, q, cu_q, block_tables, prefix_lens, extend_lens, max_extend_len, max_total_len, scale,
+                               out, lse, workspace, stream), "attn_extend")
 
 
 def attn_extend_append(pool: Pool, q, k_new, v_new, cu_q, block_tables, prefix_lens, extend_lens, max_extend_len,
                        max_total_len, scale, out, lse, workspace=None, stream=None):
     """kv_append of the suffix rows (k_new, v_new, ragged by cu_q) at positions prefix_lens[i].. and attn_extend, one call."""
-    _check(lib().attn_extend_append(pool.handle, _dev_ptr(q), _dev_ptr(k_new), _dev_ptr(v_new), q.shape[1], _dev_ptr(cu_q),
-                                    _dev_ptr(block_tables), block_tables.shape[1], _dev_ptr(prefix_lens),
-                                    _dev_ptr(extend_lens), prefix_lens.numel(), q.shape[0], max_extend_len, max_total_len,
-                                    float(scale), _dev_ptr(out), _dev_ptr(lse), _dev_ptr(workspace),
-                                    0 if workspace is None else workspace.numel() * workspace.element_size(),
-                                    _stream(stream)), "attn_extend_append")
+    _check(_native.attn_extend_append(pool.ptr, q, k_new, v_new, cu_q, block_tables, prefix_lens, extend_lens, max_extend_len,
+                                      max_total_len, scale, out, lse, workspace, stream), "attn_extend_append")
 
 
 def attn_extend_plan(pool: Pool, n_q_heads, cu_q, block_tables, prefix_lens, extend_lens, total_q, max_extend_len,
                      max_total_len, workspace, stream=None):
     """Builds attn_extend's work list for these lengths into the workspace (once per step, reused by every layer)."""
-    _check(lib().attn_extend_plan(pool.handle, n_q_heads, _dev_ptr(cu_q), _dev_ptr(block_tables), block_tables.shape[1],
-                                  _dev_ptr(prefix_lens), _dev_ptr(extend_lens), prefix_lens.numel(), total_q,
-                                  max_extend_len, max_total_len, _dev_ptr(workspace),
-                                  workspace.numel() * workspace.element_size(), _stream(stream)), "attn_extend_plan")
+    _check(_native.attn_extend_plan(pool.ptr, n_q_heads, cu_q, block_tables, prefix_lens, extend_lens, total_q, max_extend_len,
+                                    max_total_len, workspace, stream), "attn_extend_plan")
 
 
 def attn_extend_planned(pool: Pool, q, cu_q, block_tables, prefix_lens, extend_lens, max_extend_len, max_total_len, scale,
                         out, lse, workspace, stream=None):
     """attn_extend over the plan that attn_extend_plan left in the workspace (same arguments)."""
-    _check(lib().attn_extend_planned(pool.handle, _dev_ptr(q), q.shape[1], _dev_ptr(cu_q), _dev_ptr(block_tables),
-                                     block_tables.shape[1], _dev_ptr(prefix_lens), _dev_ptr(extend_lens),
-                                     prefix_lens.numel(), q.shape[0], max_extend_len, max_total_len, float(scale),
-                                     _dev_ptr(out), _dev_ptr(lse), _dev_ptr(workspace),
-                                     workspace.numel() * workspace.element_size(), _stream(stream)), "attn_extend_planned")
+    _check(_native.attn_extend_planned(pool.ptr, q, cu_q, block_tables, prefix_lens, extend_lens, max_extend_len, max_total_len,
+                                       scale, out, lse, workspace, stream), "attn_extend_planned")
 
 
 def attn_extend_host_staging_bytes(pool: Pool, n_q_heads, batch, total_q, max_pages, max_total_len) -> int:
@@ -324,22 +329,13 @@ def attn_extend_shared_workspace_bytes(pool: Pool, n_q_heads, n_parents, n_child
 def attn_extend_shared(pool: Pool, q, cu_q, cu_children, parent_tables, parent_lens, child_tables, child_lens,
                        max_child_len, max_parent_rows, max_parent_len, scale, out, lse, workspace, stream=None):
     """Children that share their parent's prefix pages (see the header): the shared pages are read once per parent."""
-    _check(lib().attn_extend_shared(pool.handle, _dev_ptr(q), q.shape[1], _dev_ptr(cu_q), _dev_ptr(cu_children),
-                                    _dev_ptr(parent_tables), parent_tables.shape[1], _dev_ptr(parent_lens),
-                                    _dev_ptr(child_tables), child_tables.shape[1], _dev_ptr(child_lens),
-                                    parent_lens.numel(), child_lens.numel(), q.shape[0], max_child_len,
-                                    max_parent_rows, max_parent_len, float(scale), _dev_ptr(out), _dev_ptr(lse),
-                                    _dev_ptr(workspace),
-                                    0 if workspace is None else workspace.numel() * workspace.element_size(),
-                                    _stream(stream)), "attn_extend_shared")
+    _check(_native.attn_extend_shared(pool.ptr, q, cu_q, cu_children, parent_tables, parent_lens, child_tables, child_lens,
+                                      max_child_len, max_parent_rows, max_parent_len, scale, out, lse, workspace, stream),
+           "attn_extend_shared")
 
 
 def attn_decode(pool: Pool, q, block_tables, ctx_lens, max_ctx_len, scale, out, lse, workspace=None, stream=None):
-    _check(lib().attn_decode(pool.handle, _dev_ptr(q), q.shape[1], _dev_ptr(block_tables), block_tables.shape[1],
-                             _dev_ptr(ctx_lens), q.shape[0], max_ctx_len, float(scale), _dev_ptr(out),
-                             _dev_ptr(lse), _dev_ptr(workspace),
-                             0 if workspace is None else workspace.numel() * workspace.element_size(),
-                             _stream(stream)), "attn_decode")
+    _check(_native.attn_decode(pool.ptr, q, block_tables, ctx_lens, max_ctx_len, scale, out, lse, workspace, stream), "attn_decode")
 
 
 def attn_decode_static(pool: Pool, q, block_tables, ctx_lens, max_ctx_len, scale, out, lse, stream=None):
@@ -367,10 +363,7 @@ def decode_args(q, block_tables, ctx_lens, max_ctx_len, out, lse) -> DecodeArgs:
 
 def attn_mixed(pool: Pool, n_q_heads, scale, ext: Optional[ExtendArgs], dec: Optional[DecodeArgs], workspace,
                stream=None):
-    _check(lib().attn_mixed(pool.handle, n_q_heads, float(scale), C.byref(ext) if ext is not None else None,
-                            C.byref(dec) if dec is not None else None, _dev_ptr(workspace),
-                            0 if workspace is None else workspace.numel() * workspace.element_size(),
-                            _stream(stream)), "attn_mixed")
+    _check(_native.attn_mixed(pool.ptr, n_q_heads, scale, ext, dec, workspace, stream), "attn_mixed")
 
 
 def kv_check_batch(pool: Pool, block_tables, lens, stream=None) -> int:
