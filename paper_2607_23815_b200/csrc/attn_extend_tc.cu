@@ -88,8 +88,8 @@ struct TcArgs {
   // mode 1: every row sees the keys [0, P_i) only.
   // mode 2 (fan-out): a "sequence" is a parent, its rows are the suffix tokens of its children stacked one
   //         after the other; a row sees the parent's keys [0, P) and then its own child's keys up to itself.
-  //         The KV steps of an item are the parent's tiles followed by the tiles of every child that has a
-  //         row in the item, each from the child's own pages.
+  //         The KV steps of an item are eight pages each of the parent's pages followed by those of every child that
+  //         has a row in the item.
   int mode;
   FanArgs fan;
   float scale_log2;
@@ -111,7 +111,8 @@ struct TcArgs {
 struct ItemRec {
   int seq, tp, P, E;
   int row0, n_kv0, n_kv1, kv_end;  // first query row; KV tile steps of the two tiles; keys the item sees at most
-                                   // (fan-out mode: kv_end holds the first child that has a row in the item)
+                                   // (fan-out mode: kv_end holds the first child that has a row in the item, the upper
+                                   // bits of tp the pages of its last step)
 };
 
 __device__ __forceinline__ ItemRec make_item(int seq, int tp, int P, int E, int row0, int lg, int max_pages, int mode,
@@ -142,23 +143,23 @@ __device__ __forceinline__ ItemRec make_item(int seq, int tp, int P, int E, int 
     }
     const int c_first = lo;
     const int tok_hi_item = max(tok_hi_t[0], tok_hi_t[1]);
-    int extra0 = 0, extra = 0;
-    bool fits = true;
+    // The item's keys are a list of pages: the parent's, then those of every child with a row in the item (of the last
+    // child only what the item's rows see).  A KV step is eight pages of that list, so that short children share a step
+    // with each other and with the end of the parent.
+    int pages0 = 0, pages = 0;  // of the children, for the first tile's rows and for both tiles'
+    bool fits = P <= max_pages * kPageSize;
     for (int c = c_first; c < c1; ++c) {
       const int start = __ldg(fan.cu_q + c) - row0, len = __ldg(fan.cu_q + c + 1) - __ldg(fan.cu_q + c);
       if (start > tok_hi_item) break;
       if (len > fan.max_pages * kPageSize) fits = false;
-      const int st = (len + 127) >> 7;
-      extra += st;
-      if (start <= tok_hi_t[0]) extra0 += st;
+      if (start <= tok_hi_t[0]) pages0 = pages + ((min(len, tok_hi_t[0] - start + 1) + 15) >> 4);
+      pages += (min(len, tok_hi_item - start + 1) + 15) >> 4;
     }
+    const int own = (P + kPageSize - 1) / kPageSize, total = own + pages;
+    r.n_kv0 = fits ? (own + pages0 + 7) >> 3 : 0;
+    r.n_kv1 = fits && tok_hi_t[1] >= 0 ? (total + 7) >> 3 : 0;
     r.kv_end = c_first;
-    if (!fits) {
-      r.n_kv0 = r.n_kv1 = 0;
-    } else if (r.n_kv0 > 0 || P == 0) {
-      r.n_kv0 = ((P + 127) >> 7) + extra0;
-      r.n_kv1 = tok_hi_t[1] >= 0 ? ((P + 127) >> 7) + extra : 0;
-    }
+    r.tp |= ((total - 1) & 7) << 28;  // pages of the last step, less one
   }
   return r;
 }
@@ -385,42 +386,10 @@ struct Item {
   int seq, kvh, tp, P, E, row0;
   int n_kv[2];   // KV tile steps of the two query tiles (0 = tile has no rows)
   int ld_tiles;  // KV tiles the producer brings in
-  int kv_end;    // keys the item can see at most (fan-out mode: the parent's keys)
+  int kv_end;    // keys the item can see at most (fan-out mode: slots of all its pages)
   int c_first;   // fan-out mode: first child with a row in the item
   int first_tile, part;  // span scheduling: first KV tile of the chunk, slot of its partial result (-1: none)
 };
-
-// Fan-out mode: position in the children's part of an item's KV steps.
-struct ChildCur {
-  int c, jc;        // child and 128-key tile inside the child's suffix
-  int start, len;   // the child's first token among the parent's stacked rows, and its length
-};
-__device__ __forceinline__ void child_load(const TcArgs& a, int row0, ChildCur& k) {
-  // children without tokens contribute no step
-  int r0 = __ldg(a.fan.cu_q + k.c), r1 = __ldg(a.fan.cu_q + k.c + 1);
-  while (r1 == r0 && k.c + 1 < a.fan.n_children) {
-    ++k.c;
-    r0 = r1;
-    r1 = __ldg(a.fan.cu_q + k.c + 1);
-  }
-  k.start = r0 - row0;
-  k.len = r1 - r0;
-}
-__device__ __forceinline__ void child_first(const TcArgs& a, const Item& it, ChildCur& k) {
-  k.c = it.c_first;
-  k.jc = 0;
-  child_load(a, it.row0, k);
-}
-__device__ __forceinline__ void child_next(const TcArgs& a, const Item& it, ChildCur& k) {
-  if ((k.jc + 1) * 128 < k.len) {
-    ++k.jc;
-  } else if (k.c + 1 < a.fan.n_children) {
-    ++k.c;
-    k.jc = 0;
-    child_load(a, it.row0, k);
-  }
-}
-__device__ __forceinline__ int child_pages(const ChildCur& k) { return min(8, (k.len - k.jc * 128 + 15) >> 4); }
 
 // Item k of the global list: entry k / Hkv of the plan, KV head k % Hkv.  Returns false past the end.
 template <bool FAN>
@@ -432,12 +401,13 @@ __device__ __forceinline__ bool fetch_item(const TcArgs& a, int k, int n_total, 
   it.seq = r0.x; it.tp = r0.y; it.P = r0.z; it.E = r0.w;
   it.row0 = r1.x; it.n_kv[0] = r1.y; it.n_kv[1] = r1.z; it.kv_end = r1.w;
   it.c_first = 0;
-  if (FAN) {
-    it.c_first = r1.w;
-    it.kv_end = it.P;
-  }
   it.kvh = k - e * Hkv;
   it.ld_tiles = max(it.n_kv[0], it.n_kv[1]);
+  if (FAN) {
+    it.c_first = r1.w;
+    it.kv_end = ((it.ld_tiles - 1) * 8 + (int)((unsigned)r0.y >> 28) + 1) * kPageSize;  // slots of the item's pages
+    it.tp = r0.y & 0x0fffffff;
+  }
   return true;
 }
 
@@ -774,17 +744,22 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
       if (!ok) break;
       const int* bt = a.block_tables + (int64_t)it.seq * a.max_pages + (REC ? it.first_tile * 8 : 0);
       const size_t head_off = (size_t)it.kvh * Cfg::kBlockBytes;
-      const int n_own = FAN ? (it.P + 127) >> 7 : it.ld_tiles;  // tiles from the sequence's (parent's) own pages
-      ChildCur cc{0, 0, 0, 0};
+      const int n_own = FAN ? (it.P + kPageSize - 1) / kPageSize : 0;  // fan-out mode: the parent's pages
+      int child = it.c_first, child_at = n_own;                        // this lane's child and its first page in the list
       for (int j = 0; j < it.ld_tiles && ok; ++j) {
-        int np = min(8, (it.kv_end - j * 128 + 15) >> 4);
-        const int* src_bt = bt + j * 8;
-        if (FAN && j >= n_own) {  // fan-out mode: a tile of a child's own keys
-          if (j == n_own) child_first(a, it, cc); else child_next(a, it, cc);
-          np = child_pages(cc);
-          src_bt = a.fan.tables + (int64_t)cc.c * a.fan.max_pages + cc.jc * 8;
-        }
+        const int np = min(8, (it.kv_end - j * 128 + 15) >> 4);
         int page = 0;
+        const int* src_bt = bt + j * 8;
+        if (FAN && lane < np && j * 8 + lane >= n_own) {
+          const int g = j * 8 + lane;
+          while (true) {
+            const int pages = (__ldg(a.fan.cu_q + child + 1) - __ldg(a.fan.cu_q + child) + kPageSize - 1) / kPageSize;
+            if (g < child_at + pages || child + 1 >= a.fan.n_children) break;
+            child_at += pages;
+            ++child;
+          }
+          src_bt = a.fan.tables + (int64_t)child * a.fan.max_pages + (g - child_at) - lane;
+        }
         if (lane < np) {
           page = __ldg(src_bt + lane);
           if ((unsigned)page >= (unsigned)a.pool.num_pages) {
@@ -871,14 +846,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
         }
         if (ok && elect_one_sync()) mma_commit(smem_u32(&sm.kv_empty[stage]));
         __syncwarp();
-        const int n_own = FAN ? (it.P + 127) >> 7 : it.ld_tiles;
-        ChildCur cc{0, 0, 0, 0};
         for (int j = 0; j < it.ld_tiles && ok; ++j) {
-          int np = min(8, (it.kv_end - j * 128 + 15) >> 4);
-          if (FAN && j >= n_own) {  // fan-out mode: a tile of a child's own keys
-            if (j == n_own) child_first(a, it, cc); else child_next(a, it, cc);
-            np = child_pages(cc);
-          }
+          const int np = min(8, (it.kv_end - j * 128 + 15) >> 4);
           const uint32_t v_stage = loads % Cfg::kStages;
           ok = mbar_wait(smem_u32(&sm.kv_full[v_stage]), (loads / Cfg::kStages) & 1, abortp);
           ++loads;
@@ -1209,10 +1178,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
       int n_t, limit, part = -1;
       bool valid;
       int64_t orow_idx;
-      // fan-out mode: the steps from n_own on walk the children's own keys; tok_s is this row's token among the
-      // parent's stacked rows (-1: no such row) and (f_row0, f_child) start the walk
-      int n_own, tok_s = -1, f_row0 = 0;
-      ChildCur cc{0, 0, 0, 0};
+      int f_lo = 0, f_hi = 0;  // fan-out mode: this row's child's own keys that it sees, among the slots of the item's pages
       {
         Item it;
         const bool more_items = fetch(round, it);
@@ -1224,14 +1190,20 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
         const int rg = it.tp * 256 + t * 128 + m;
         const int tok = rg >> lg;
         valid = tok < it.E;
-        limit = valid && a.mode == 0 ? it.P + tok + 1 : it.kv_end;  // keys this row sees (rows past the end: any)
+        // keys this row sees (rows past the end: any); fan-out mode: the parent's
+        limit = FAN ? it.P : valid && a.mode == 0 ? it.P + tok + 1 : it.kv_end;
         orow_idx = (int64_t)(it.row0 + tok) * Hq + it.kvh * G + (rg & (G - 1));  // row of the LSE
         if (SPAN) part = it.part;
-        n_own = FAN ? (it.P + 127) >> 7 : n_t;
-        if (FAN) {
-          tok_s = valid ? tok : -1;
-          f_row0 = it.row0;
-          cc.c = it.c_first;
+        if (FAN && valid) {
+          int c = it.c_first, r0 = __ldg(a.fan.cu_q + c) - it.row0, r1 = __ldg(a.fan.cu_q + c + 1) - it.row0;
+          f_lo = (it.P + kPageSize - 1) / kPageSize * kPageSize;
+          while (tok >= r1 && c + 1 < a.fan.n_children) {
+            f_lo += (r1 - r0 + kPageSize - 1) / kPageSize * kPageSize;
+            ++c;
+            r0 = r1;
+            r1 = __ldg(a.fan.cu_q + c + 1) - it.row0;
+          }
+          f_hi = f_lo + tok - r0 + 1;
         }
       }
       float m_run = -INFINITY, l_run = 0.f;
@@ -1245,22 +1217,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
         // One trip to tensor memory: the row's 128 scores are read into registers, reduced to the row
         // maximum, exponentiated in place and written back as bf16 P.
         // vis: how many of the tile's 128 key columns this row sees (diagonal / last tile: keys past the row's
-        // limit are hidden; fan-out mode: only the row's own child, up to the row's own token)
-        int vis = limit - j * 128;
-        if (FAN && j >= n_own) {
-          if (j == n_own) {
-            cc.jc = 0;
-            child_load(a, f_row0, cc);
-          } else if ((cc.jc + 1) * 128 < cc.len) {
-            ++cc.jc;
-          } else if (cc.c + 1 < a.fan.n_children) {
-            ++cc.c;
-            cc.jc = 0;
-            child_load(a, f_row0, cc);
-          }
-          const int t_local = tok_s - cc.start;
-          vis = (tok_s >= 0 && t_local >= 0 && t_local < cc.len) ? t_local + 1 - cc.jc * 128 : 0;
-        }
+        // limit are hidden); fan-out mode: also the columns lo .. hi - 1, its own child's keys up to its own token
+        const int vis = limit - j * 128, lo = f_lo - j * 128, hi = f_hi - j * 128;
         const bool ragged = vis < 128;
         uint32_t sr[4][32];
 #pragma unroll
@@ -1271,7 +1229,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
           for (int c = 0; c < 4; ++c)
 #pragma unroll
             for (int i = 0; i < 32; ++i)
-              if (c * 32 + i >= vis) sr[c][i] = 0xff800000u;  // -inf by select: NaN-safe
+              if (c * 32 + i >= vis && (!FAN || c * 32 + i < lo || c * 32 + i >= hi)) sr[c][i] = 0xff800000u;  // -inf by select: NaN-safe
         }
         if constexpr (OPT) {
           // The row maximum is needed only to keep the exponentials in range, and after the first tile it rarely
