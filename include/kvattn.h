@@ -239,8 +239,7 @@ kv_status_t attn_extend_host(kv_pool_t* pool, const void* q, const void* k_new, 
  * than 64/128, scale <= 0), KV_ERR_WORKSPACE; a table entry or length outside the pool is skipped on
  * the device and recorded as KV_ERR_BOUNDS (kv_last_async_status).  Nothing is allocated or retained.
  * With kvattn_set_shared_impl(1) the two partial results of a row (shared part, own part) are each
- * rounded to bf16 before they are merged; the default for suffixes of 16 tokens and more on average
- * accumulates both in one fp32 accumulator. */
+ * rounded to bf16 before they are merged; the default accumulates both in one fp32 accumulator. */
 size_t attn_extend_shared_workspace_bytes(const kv_pool_t* pool, int n_q_heads, int n_parents, int n_children,
                                           int total_q, int max_parent_len);
 kv_status_t attn_extend_shared(kv_pool_t* pool, const void* q, int n_q_heads, const int* cu_q, const int* cu_children,
@@ -305,8 +304,8 @@ kv_status_t kv_last_async_status(kv_pool_t* pool);
 /* Selects the extend kernel: 0 = automatic, 1 = the small-tile kernel (rows of one KV head read K/V
  * straight from HBM), 2 = the tcgen05 tensor-core kernel.  Process-wide; for tests and benchmarks. */
 kv_status_t kvattn_set_extend_impl(int impl);
-/* Test/tuning hook for attn_extend_shared: 0 = choose by the mean suffix length (default), 1 = three kernels
- * (shared part, own part, merge), 2 = one kernel that walks the parent's and then the children's tiles. */
+/* Test/tuning hook for attn_extend_shared: 1 = three kernels (shared part, own part, merge), 2 = one kernel over
+ * the parent's and the children's pages, 0 = the default, which is 2. */
 kv_status_t kvattn_set_shared_impl(int impl);
 /* Selects how the decode kernel brings pages on chip: 1 = straight into registers (one page per warp in flight), 2 =
  * through a per-warp ring of page slots in shared memory filled by bulk copies (several pages per warp in flight);

@@ -198,10 +198,13 @@ __device__ __forceinline__ void plan_body(const PlanArgs& pa) {
   for (int i = threadIdx.x; i < kPlanBuckets; i += blockDim.x) hist[i] = 0;
   __syncthreads();
   const int64_t n = (int64_t)batch * max_tp;
+  // Fan-out mode: a sequence is a parent, its rows are those of its children, which follow one another in Q.
+  auto row_of = [&](int seq) { return mode == 2 ? __ldg(cu_q + __ldg(fan.cu_children + seq)) : __ldg(cu_q + seq); };
+  auto rows_of = [&](int seq) { return mode == 2 ? row_of(seq + 1) - row_of(seq) : __ldg(extend_lens + seq); };
   // A sequence with more suffix tokens than the host-side bound the grid was sized with would lose its last rows
   // without a trace: it is reported instead.
   for (int seq = threadIdx.x; seq < batch; seq += blockDim.x) {
-    const int E = __ldg(extend_lens + seq);
+    const int E = rows_of(seq);
     if (__ldg(prefix_lens + seq) >= 0 && (int64_t)E > (((int64_t)max_tp * 256) >> lg)) report(status, KV_ERR_BOUNDS);
   }
   // The sequences are put into groups longest first, so that the last groups, which decide how evenly the CTAs
@@ -219,7 +222,7 @@ __device__ __forceinline__ void plan_body(const PlanArgs& pa) {
       return (int)min((int64_t)(kPlanSeqBuckets - 1), (int64_t)(P + E) * kPlanSeqBuckets / span);
     };
     for (int seq = threadIdx.x; seq < batch; seq += blockDim.x) {
-      const int P = __ldg(prefix_lens + seq), E = __ldg(extend_lens + seq);
+      const int P = __ldg(prefix_lens + seq), E = rows_of(seq);
       if (P >= 0 && E > 0) atomicAdd(&seq_hist[bucket_of(P, E)], 1);
     }
     __syncthreads();
@@ -249,7 +252,7 @@ __device__ __forceinline__ void plan_body(const PlanArgs& pa) {
     }
     __syncthreads();
     for (int seq = threadIdx.x; seq < batch; seq += blockDim.x) {
-      const int P = __ldg(prefix_lens + seq), E = __ldg(extend_lens + seq);
+      const int P = __ldg(prefix_lens + seq), E = rows_of(seq);
       seq_rank[seq] = (P >= 0 && E > 0) ? (unsigned short)atomicAdd(&seq_hist[bucket_of(P, E)], 1) : 0;
     }
     __syncthreads();
@@ -265,10 +268,10 @@ __device__ __forceinline__ void plan_body(const PlanArgs& pa) {
   };
   for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
     const int seq = (int)(e / max_tp), tp = (int)(e % max_tp);
-    const int P = __ldg(prefix_lens + seq), E = __ldg(extend_lens + seq);
+    const int P = __ldg(prefix_lens + seq), E = rows_of(seq);
     if (P < 0 || E <= 0) continue;
     if (((tp * 256) >> lg) >= E) continue;
-    const ItemRec r = make_item(seq, tp, P, E, __ldg(cu_q + seq), lg, max_pages, mode, fan);
+    const ItemRec r = make_item(seq, tp, P, E, row_of(seq), lg, max_pages, mode, fan);
     const int steps = r.n_kv0 + r.n_kv1;
     if (steps > 0) atomicAdd(&hist[key_of(steps, seq)], 1);
   }
@@ -305,10 +308,10 @@ __device__ __forceinline__ void plan_body(const PlanArgs& pa) {
   __syncthreads();
   for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
     const int seq = (int)(e / max_tp), tp = (int)(e % max_tp);
-    const int P = __ldg(prefix_lens + seq), E = __ldg(extend_lens + seq);
+    const int P = __ldg(prefix_lens + seq), E = rows_of(seq);
     if (P < 0 || E <= 0) continue;
     if (((tp * 256) >> lg) >= E) continue;
-    const ItemRec r = make_item(seq, tp, P, E, __ldg(cu_q + seq), lg, max_pages, mode, fan);
+    const ItemRec r = make_item(seq, tp, P, E, row_of(seq), lg, max_pages, mode, fan);
     const int steps = r.n_kv0 + r.n_kv1;
     if (steps == 0 && (mode == 0 || P > 0 || mode == 2)) report(status, KV_ERR_BOUNDS);  // rows exist but the lengths do not fit the tables
     if (steps > 0) {
@@ -379,7 +382,8 @@ struct __align__(1024) TcSmem {
 struct SpanRec {
   int seq, kvh, tp, P;
   int E, row0, n_kv0, n_kv1;
-  int kv_end, first_tile, part;  // part: slot of the partial result, -1 for a whole item
+  int kv_end, first_tile, part;  // part: slot of the partial result, -1 for a whole item (fan-out mode: P counts from the
+                                 // parent's first key, and the first child of the item follows)
 };
 
 struct Item {
@@ -419,7 +423,8 @@ struct SpanPos {
 
 // Rows of the sequence that count: none if the lengths do not fit the tables, no row past the host-side bounds.
 __device__ __forceinline__ int span_rows(const TcArgs& a, int P, int E, int row0) {
-  if (P < 0 || E <= 0 || row0 < 0 || P + E > a.max_pages * kPageSize) return 0;
+  // (fan-out mode: the rows' own keys are not in the parent's table)
+  if (P < 0 || E <= 0 || row0 < 0 || (a.mode != 0 ? P : P + E) > a.max_pages * kPageSize) return 0;
   return min(min(E, (int)min((int64_t)0x7fffffff, ((int64_t)a.span.max_tp * 256) >> a.lg_group)), max(0, a.span.total_q - row0));
 }
 // KV steps of tile pair tp of a sequence with E rows behind P keys
@@ -664,8 +669,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
     const int seq = (int)blockIdx.x / a.cl_splits / a.pool.n_kv_heads / a.span.max_tp;
     if (!a.span.plan_early) dependency_wait();
     cl_P = __ldg(a.prefix_lens + seq);
-    cl_E = __ldg(a.extend_lens + seq);
-    cl_row0 = __ldg(a.cu_q + seq);
+    if (FAN) {  // a parent's rows are those of its children
+      cl_row0 = __ldg(a.fan.cu_q + __ldg(a.fan.cu_children + seq));
+      cl_E = __ldg(a.fan.cu_q + __ldg(a.fan.cu_children + seq + 1)) - cl_row0;
+    } else {
+      cl_E = __ldg(a.extend_lens + seq);
+      cl_row0 = __ldg(a.cu_q + seq);
+    }
     for (int b = lane * 32; b < a.max_pages; b += 1024) prefetch_l2(a.block_tables + (int64_t)seq * a.max_pages + b);
   }
   tc_fence_before_sync();
@@ -697,7 +707,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
       it.seq = r0.x; it.kvh = r0.y; it.tp = r0.z; it.P = r0.w;
       it.E = r1.x; it.row0 = r1.y; it.n_kv[0] = r1.z; it.n_kv[1] = r1.w;
       it.kv_end = r2.x; it.first_tile = r2.y; it.part = r2.z;
-      it.c_first = 0;
+      it.c_first = FAN ? r2.w : 0;
       it.ld_tiles = max(it.n_kv[0], it.n_kv[1]);
       return it.seq >= 0;
     } else {
@@ -750,8 +760,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
         const int np = min(8, (it.kv_end - j * 128 + 15) >> 4);
         int page = 0;
         const int* src_bt = bt + j * 8;
-        if (FAN && lane < np && j * 8 + lane >= n_own) {
-          const int g = j * 8 + lane;
+        const int g = (j + (REC ? it.first_tile : 0)) * 8 + lane;
+        if (FAN && lane < np && g >= n_own) {
           while (true) {
             const int pages = (__ldg(a.fan.cu_q + child + 1) - __ldg(a.fan.cu_q + child) + kPageSize - 1) / kPageSize;
             if (g < child_at + pages || child + 1 >= a.fan.n_children) break;
@@ -967,21 +977,23 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
       if (a.span.plan_early) dependency_wait();
       if (lane == 0) {
         if (tp == 0 && kvh == 0 && rank == 0 && P >= 0 && rows < E) report(a.pool.status, KV_ERR_BOUNDS);
-        int n = 0, n0 = 0, n1 = 0, hi = 0;
+        int n = 0, n0 = 0, n1 = 0, kv_end = 0, first_child = 0;
         if (tp < pairs) {
-          const int tok_1 = (tp * 256 + 128) >> lg;  // first token of the second tile
-          n0 = (P + min(rows, tok_1) + 127) >> 7;
-          hi = min(rows, ((tp + 1) * 256) >> lg);
-          n = (P + hi + 127) >> 7;
-          n1 = tok_1 < rows ? n : 0;
+          const ItemRec r = make_item(seq, tp, P, rows, row0, lg, a.max_pages, a.mode, a.fan);
+          n0 = r.n_kv0;
+          n1 = r.n_kv1;
+          n = max(n0, n1);
+          first_child = r.kv_end;
+          kv_end = FAN ? ((n - 1) * 8 + (int)((unsigned)r.tp >> 28) + 1) * kPageSize : r.kv_end;
+          if (n == 0) report(a.pool.status, KV_ERR_BOUNDS);
         }
         const int off = n * rank / splits, end = n * (rank + 1) / splits;
-        sm.cl_unit = make_int4(tp < pairs ? min(256, (rows << lg) - tp * 256) : 0, row0, tp, kvh);
+        sm.cl_unit = make_int4(n > 0 ? min(256, (rows << lg) - tp * 256) : 0, row0, tp, kvh);
         int round = 0;
         if (end > off) {
-          sm.sched_rec[0][0] = make_int4(seq, kvh, tp, P - off * 128);
+          sm.sched_rec[0][0] = make_int4(seq, kvh, tp, FAN ? P : P - off * 128);
           sm.sched_rec[0][1] = make_int4(rows, row0, max(0, min(n0, end) - off), max(0, min(n1, end) - off));
-          sm.sched_rec[0][2] = make_int4(P + hi - off * 128, off, -1, 0);
+          sm.sched_rec[0][2] = make_int4(kv_end - off * 128, off, -1, first_child);
           mbar_arrive(smem_u32(&sm.sched_full[0]));
           round = 1;
         }
@@ -1191,12 +1203,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
         const int tok = rg >> lg;
         valid = tok < it.E;
         // keys this row sees (rows past the end: any); fan-out mode: the parent's
-        limit = FAN ? it.P : valid && a.mode == 0 ? it.P + tok + 1 : it.kv_end;
+        limit = FAN ? it.P - it.first_tile * 128 : valid && a.mode == 0 ? it.P + tok + 1 : it.kv_end;
         orow_idx = (int64_t)(it.row0 + tok) * Hq + it.kvh * G + (rg & (G - 1));  // row of the LSE
         if (SPAN) part = it.part;
         if (FAN && valid) {
           int c = it.c_first, r0 = __ldg(a.fan.cu_q + c) - it.row0, r1 = __ldg(a.fan.cu_q + c + 1) - it.row0;
-          f_lo = (it.P + kPageSize - 1) / kPageSize * kPageSize;
+          f_lo = (it.P + kPageSize - 1) / kPageSize * kPageSize - it.first_tile * 128;
           while (tok >= r1 && c + 1 < a.fan.n_children) {
             f_lo += (r1 - r0 + kPageSize - 1) / kPageSize * kPageSize;
             ++c;
@@ -1665,7 +1677,7 @@ static kv_status_t resident_clusters(int device, int c, int* n) {
 //    260 and 197; but 4 of 6900 with 128 items of equal length 112 and 120.  More than three items per SM, or short ones:
 //    the list (3 prefills of up to 1950 tokens, 4.2 items per SM: 85 against 98; 64 sequences, 12 per SM: 263 against 298).
 static kv_status_t choose_schedule(const kv_pool_t* p, int n_q_heads, int batch, int total_q, int max_extend_len, int max_total_len,
-                                   size_t workspace_bytes, int* sched, int* splits) {
+                                   size_t workspace_bytes, int mode, int* sched, int* splits) {
   *sched = kSchedList;
   *splits = 1;
   const int G = n_q_heads / p->n_kv_heads, sms = sm_count_of(p->device);
@@ -1686,8 +1698,8 @@ static kv_status_t choose_schedule(const kv_pool_t* p, int n_q_heads, int batch,
       if (s != KV_OK) return s;
       if (units <= resident) *splits = c;
     }
-    if ((double)steps / *splits - even > 12.0) *sched = kSchedSpans;
-  } else if (room && l.cuts && most <= 3ll * sms && 0.85 * steps * ceil(rounds) - even > 16.0) {
+    if (mode == 0 && (double)steps / *splits - even > 12.0) *sched = kSchedSpans;
+  } else if (mode == 0 && room && l.cuts && most <= 3ll * sms && 0.85 * steps * ceil(rounds) - even > 16.0) {
     *sched = kSchedSpans;
   }
   return KV_OK;
@@ -1713,7 +1725,7 @@ static char* align_workspace(void* ws) {
 kv_status_t launch_extend_combine(kv_pool_t* p, int n_q_heads, int batch, int total_q, int max_extend_len, int max_total_len, void* out, float* lse,
                                   void* workspace, size_t workspace_bytes, bool early, cudaStream_t st) {
   int sched, splits;
-  const kv_status_t cs = choose_schedule(p, n_q_heads, batch, total_q, max_extend_len, max_total_len, workspace_bytes, &sched, &splits);
+  const kv_status_t cs = choose_schedule(p, n_q_heads, batch, total_q, max_extend_len, max_total_len, workspace_bytes, 0, &sched, &splits);
   if (cs != KV_OK) return cs;
   if (sched != kSchedSpans) return KV_OK;
   const SpanLayout l = span_layout(p, n_q_heads, batch, total_q, max_total_len);
@@ -1779,8 +1791,8 @@ kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const i
   groups = groups > batch ? batch : groups;
   groups = groups > kPlanBuckets / 16 ? kPlanBuckets / 16 : groups;
   int sched = kSchedList, splits = 1;
-  if (mode == 0) {
-    const kv_status_t cs = choose_schedule(p, n_q_heads, batch, total_q, max_extend_len, max_total_len, workspace_bytes, &sched, &splits);
+  if (mode != 1) {
+    const kv_status_t cs = choose_schedule(p, n_q_heads, batch, total_q, max_extend_len, max_total_len, workspace_bytes, mode, &sched, &splits);
     if (cs != KV_OK) return cs;
   }
   const PlanArgs pa{prefix_lens, extend_lens, cu_q, batch, max_tp, lg, max_steps, (int)capacity, max_pages, mode,
@@ -1847,10 +1859,9 @@ kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const i
   auto go = [&](auto d, auto o, auto f) {
     constexpr int DD = decltype(d)::value;
     constexpr bool OO = decltype(o)::value, FF = decltype(f)::value;
-    if constexpr (!FF) {
+    if constexpr (!FF)
       if (sched == kSchedSpans) return launch_tc<DD, OO, false, kSchedSpans>(a, q_map, grid, p->device, early, st);
-      if (sched == kSchedCluster) return launch_tc<DD, OO, false, kSchedCluster>(a, q_map, grid, p->device, early, st);
-    }
+    if (sched == kSchedCluster) return launch_tc<DD, OO, FF, kSchedCluster>(a, q_map, grid, p->device, early, st);
     return launch_tc<DD, OO, FF, kSchedList>(a, q_map, grid, p->device, early, st);
   };
   using I128 = std::integral_constant<int, 128>;

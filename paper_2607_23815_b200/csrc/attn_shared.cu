@@ -6,17 +6,18 @@
 // E_c tokens in its private pages.  All suffix queries of all children of a parent are stacked row
 // after row, so that the parent's pages are read once, with full query tiles, instead of once per
 // child with mostly empty tiles.  Two ways to add the children's own keys:
-//   fused   the tensor-core kernel's fan-out mode: after the parent's KV tiles an item walks the
-//           tiles of every child that has a row in it, with all other rows masked.  One kernel, no
-//           intermediate results.  Good when a child's suffix fills a fair part of a 128-row tile.
+//   fused   the tensor-core kernel's fan-out mode: an item's keys are the parent's pages followed by
+//           the pages of every child that has a row in it, other rows masked.  One attention kernel, no
+//           intermediate results of its own.
 //   split   part A: the stacked rows over the parent's keys only; part B: every child's suffix
 //           over its own pages; then the two partial results of a row are merged with the
-//           log-sum-exp rule.  For very short suffixes (many children per tile).
+//           log-sum-exp rule.  On request only (kvattn_set_shared_impl).
 #include "append.cuh"
 #include "common.cuh"
 
 namespace kvattn {
 
+size_t extend_tc_workspace_bytes(const kv_pool_t* p, int n_q_heads, int batch, int total_q, int max_total_len);
 size_t extend_tc_min_workspace_bytes(int batch, int total_q);
 bool extend_tc_supported(const kv_pool_t* p, int n_q_heads);
 kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const int* cu_q, const int* block_tables,
@@ -31,7 +32,7 @@ kv_status_t launch_extend_small(kv_pool_t* p, const void* q, int n_q_heads, cons
 
 static inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-std::atomic<int> g_shared_impl{0};  // 0: choose by the mean suffix length, 1: split, 2: fused
+std::atomic<int> g_shared_impl{0};  // 0: the default, fused; 1: split; 2: fused
 
 // Row ranges of the parents in Q (their children are consecutive) and a vector of zeros (the prefix
 // lengths of part B).
@@ -105,13 +106,18 @@ __global__ void __launch_bounds__(256) shared_merge_kernel(const __nv_bfloat16* 
   if (lane == 0) lse[w] = mx + __logf(wa + wb);
 }
 
-size_t extend_shared_workspace_bytes(const kv_pool_t* p, int n_q_heads, int n_parents, int n_children, int total_q,
-                                     int max_parent_len) {
-  (void)max_parent_len;
-  if (n_parents <= 0 || n_children <= 0 || total_q <= 0) return 0;
+static size_t shared_min_workspace_bytes(const kv_pool_t* p, int n_q_heads, int n_parents, int n_children, int total_q) {
   return align256(sizeof(int) * (size_t)(2 * n_parents + 1 + n_children)) +
          align256((size_t)total_q * n_q_heads * p->head_dim * 2) + align256((size_t)total_q * n_q_heads * 4) +
          align256(extend_tc_min_workspace_bytes(n_children > n_parents ? n_children : n_parents, total_q)) + 256;
+}
+
+size_t extend_shared_workspace_bytes(const kv_pool_t* p, int n_q_heads, int n_parents, int n_children, int total_q,
+                                     int max_parent_len) {
+  if (n_parents <= 0 || n_children <= 0 || total_q <= 0) return 0;
+  const size_t least = shared_min_workspace_bytes(p, n_q_heads, n_parents, n_children, total_q);
+  // (room for the partial results of small batches; the longest item holds a parent and one tile pair's children)
+  return least + extend_tc_workspace_bytes(p, n_q_heads, n_parents, total_q, max_parent_len + 16 * kPageSize * kPageSize);
 }
 
 kv_status_t launch_extend_shared(kv_pool_t* p, const void* q, int n_q_heads, const int* cu_q, const int* cu_children,
@@ -121,7 +127,7 @@ kv_status_t launch_extend_shared(kv_pool_t* p, const void* q, int n_q_heads, con
                                  float scale, void* out, float* lse, void* workspace, size_t workspace_bytes,
                                  cudaStream_t st) {
   if (workspace == nullptr ||
-      workspace_bytes < extend_shared_workspace_bytes(p, n_q_heads, n_parents, n_children, total_q, max_parent_len))
+      workspace_bytes < shared_min_workspace_bytes(p, n_q_heads, n_parents, n_children, total_q))
     return KV_ERR_WORKSPACE;
   char* ws = reinterpret_cast<char*>(workspace);
   int* cu_q_parent = reinterpret_cast<int*>(ws);
@@ -134,20 +140,23 @@ kv_status_t launch_extend_shared(kv_pool_t* p, const void* q, int n_q_heads, con
   ws += align256((size_t)total_q * n_q_heads * 4);
   const size_t tc_bytes = extend_tc_min_workspace_bytes(n_children > n_parents ? n_children : n_parents, total_q);
 
+  const int impl = g_shared_impl.load();
+  // One kernel, whatever the children's lengths: even with one token each, a page of its own in its item's list, a child
+  // costs less there than a row of the split form's two tiles (16 parents of 600-900 tokens x 17 children of 1 / 3-5 /
+  // 8-14 tokens, 32/8 heads of 128: 88.6 / 112.5 / 144.6 us split, 33.6 / 49.7 / 66.9 in one kernel).
+  const bool fused = impl != 1;
+  if (fused) {
+    FanArgs fan{cu_q, cu_children, child_tables, max_pages_child, n_children};
+    return launch_extend_tc(p, q, n_q_heads, cu_q, parent_tables, max_pages_parent, parent_lens, child_lens, n_parents, total_q,
+                            max_parent_rows, max_parent_len + max_parent_rows, scale, out, lse, ws,
+                            workspace_bytes - (size_t)(ws - (char*)workspace), 0, 2, &fan, nullptr, 0, st);
+  }
   const int n_prep = (n_parents + 1 > n_children ? n_parents + 1 : n_children);
   shared_prep_kernel<<<(n_prep + 255) / 256, 256, 0, st>>>(cu_q, cu_children, n_parents, n_children, cu_q_parent, rows_parent,
                                                            zeros);
   count_launch();
   KV_CUDA_OK(cudaGetLastError());
   kv_status_t s;
-  const int impl = g_shared_impl.load();
-  const bool fused = impl == 2 || (impl == 0 && (int64_t)total_q >= 16 * (int64_t)n_children);
-  if (fused) {
-    FanArgs fan{cu_q, cu_children, child_tables, max_pages_child, n_children};
-    return launch_extend_tc(p, q, n_q_heads, cu_q_parent, parent_tables, max_pages_parent, parent_lens, rows_parent,
-                            n_parents, total_q, max_parent_rows, max_parent_len + max_parent_rows, scale, out, lse, ws,
-                            tc_bytes, 0, 2, &fan, nullptr, 0, st);
-  }
   // part B first, straight into the caller's buffers: each child's suffix over its private pages
   if (!extend_tc_supported(p, n_q_heads))
     s = launch_extend_small(p, q, n_q_heads, cu_q, child_tables, max_pages_child, zeros, child_lens, n_children,
