@@ -327,7 +327,11 @@ __device__ __forceinline__ void plan_body(const PlanArgs& pa) {
 }
 
 __global__ void __launch_bounds__(1024) extend_tc_plan_kernel(const PlanArgs pa) {
-  launch_dependents();  // the attention kernel may set itself up meanwhile; it waits for this kernel before it reads the plan
+  dependency_wait();
+  // The attention kernel may set itself up meanwhile; it waits for this kernel before it reads the plan.  (Not before the
+  // wait: a decode kernel that runs beside the attention kernel waits for nothing, and what precedes this kernel has to be
+  // complete by then.)
+  launch_dependents();
   plan_body(pa);
 }
 
@@ -335,6 +339,7 @@ __global__ void __launch_bounds__(1024) extend_tc_plan_kernel(const PlanArgs pa)
 // rows into their pages (one warp per token), so the step has one small kernel in front of the attention kernel
 // instead of two in a row, and the attention kernel's launch and set-up overlap it.
 __global__ void __launch_bounds__(1024) extend_prologue_kernel(const PlanArgs pa, const PoolView pool, const AppendArgs ap) {
+  dependency_wait();
   launch_dependents();
   if (blockIdx.x == 0) {
     plan_body(pa);
@@ -1500,7 +1505,8 @@ __global__ void __launch_bounds__(D * 4, 384 / D) span_combine_kernel(const Span
 
 // The suffix append in front of a span-scheduled attention kernel (which is launched early and waits for it inside).
 __global__ void __launch_bounds__(1024) append_prologue_kernel(const PoolView pool, const AppendArgs ap) {
-  launch_dependents();
+  dependency_wait();
+  launch_dependents();  // (the attention kernel reads the lengths before it waits for this one: not before the wait)
   const int warps_per_block = blockDim.x >> 5;
   append_tokens<4>(pool, ap, blockIdx.x * warps_per_block + (threadIdx.x >> 5), gridDim.x * warps_per_block);
 }
@@ -1734,19 +1740,14 @@ kv_status_t launch_extend_combine(kv_pool_t* p, int n_q_heads, int batch, int to
   int lg = 0;
   while ((1 << lg) < G) ++lg;
   const SpanArgs a = span_args(l, align_workspace(workspace), 0, total_q, 0);
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)((a.n_spans - 1) * kCombineSlices));
-  cfg.blockDim = dim3((unsigned)p->head_dim * 4);
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = early ? 1 : 0;
-  if (p->head_dim == 128)
-    KV_CUDA_OK(cudaLaunchKernelEx(&cfg, span_combine_kernel<128>, a, n_q_heads, G, lg, (__nv_bfloat16*)out, lse));
-  else
-    KV_CUDA_OK(cudaLaunchKernelEx(&cfg, span_combine_kernel<64>, a, n_q_heads, G, lg, (__nv_bfloat16*)out, lse));
+  const auto kernel = p->head_dim == 128 ? span_combine_kernel<128> : span_combine_kernel<64>;
+  const unsigned blocks = (unsigned)((a.n_spans - 1) * kCombineSlices), threads = (unsigned)p->head_dim * 4;
+  if (early) {
+    KV_CUDA_OK(launch_early(kernel, blocks, threads, st, a, n_q_heads, G, lg, (__nv_bfloat16*)out, lse));
+  } else {
+    kernel<<<blocks, threads, 0, st>>>(a, n_q_heads, G, lg, (__nv_bfloat16*)out, lse);
+    KV_CUDA_OK(cudaGetLastError());
+  }
   count_launch();
   return KV_OK;
 }
@@ -1803,9 +1804,8 @@ kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const i
     if (app != nullptr && app->total_new > 0) {
       const int64_t want = ((int64_t)app->total_new + 31) / 32;
       const int64_t cap = 2 * (int64_t)sm_count_of(p->device);
-      append_prologue_kernel<<<(int)(want < cap ? want : cap), 1024, 0, st>>>(p->view(), *app);
+      KV_CUDA_OK(launch_early(append_prologue_kernel, (unsigned)(want < cap ? want : cap), 1024, st, p->view(), *app));
       count_launch();
-      KV_CUDA_OK(cudaGetLastError());
     }
   } else if (phase == 2) {
     // the plan is in the workspace already
@@ -1814,13 +1814,11 @@ kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const i
     const int64_t want = ((int64_t)app->total_new + 31) / 32;
     const int64_t cap = 2 * (int64_t)sm_count_of(p->device) - 1;
     const int blocks = (int)(want < cap ? want : cap);
-    extend_prologue_kernel<<<1 + blocks, 1024, 0, st>>>(pa, p->view(), *app);
-  } else {
-    extend_tc_plan_kernel<<<1, 1024, 0, st>>>(pa);
-  }
-  if (phase != 2 && sched == kSchedList) {
+    KV_CUDA_OK(launch_early(extend_prologue_kernel, (unsigned)(1 + blocks), 1024, st, pa, p->view(), *app));
     count_launch();
-    KV_CUDA_OK(cudaGetLastError());
+  } else {
+    KV_CUDA_OK(launch_early(extend_tc_plan_kernel, 1, 1024, st, pa));
+    count_launch();
   }
   if (phase == 1) return KV_OK;
 

@@ -51,6 +51,22 @@ struct FanArgs {
 extern std::atomic<int64_t> g_launches;
 inline void count_launch(int n = 1) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
+// Launches a kernel that may start while the kernel in front of it in the stream still runs (programmatic dependent
+// launch).  The kernel waits for that one itself (ptx::dependency_wait) before it touches anything.
+template <typename... Params, typename... Args>
+inline cudaError_t launch_early(void (*kernel)(Params...), unsigned blocks, unsigned threads, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
 constexpr int kMaxDevices = 64;
 // Multiprocessors of the given device (asked once per device).
 int sm_count_of(int device);

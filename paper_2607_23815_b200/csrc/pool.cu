@@ -4,6 +4,7 @@
 
 #include "common.cuh"
 #include "append.cuh"
+#include "sm100_ptx.cuh"
 
 namespace kvattn {
 
@@ -14,8 +15,14 @@ std::atomic<int64_t> g_launches{0};
 // rows (coalesced loads, all in flight before the first store); the eight chunks of a 64-dim half land,
 // permuted, in one 128-byte row of the page (full-line 16-byte stores).
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) append_kernel(PoolView pool, AppendArgs a) {
-  append_tokens<8>(pool, a, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5);
+// kMaxPerLane: 16-byte chunks of K (and of V) of a token per lane and pass; no more than a token has, because the registers
+// they take decide how many tokens are on an SM at a time (10207 tokens of 8 heads x 128: 20.2 us with 8, of which a token
+// uses 4, 17.3 with 4; 64 dims, 2 per lane: 16.4 and 11.0).
+template <int kMaxPerLane>
+__global__ void __launch_bounds__(256, kMaxPerLane == 8 ? 2 : 4) append_kernel(PoolView pool, AppendArgs a) {
+  ptx::launch_dependents();
+  ptx::dependency_wait();
+  append_tokens<kMaxPerLane>(pool, a, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5);
 }
 
 __global__ void __launch_bounds__(256) gather_kernel(PoolView pool, const int* __restrict__ block_row, int len,
@@ -382,9 +389,11 @@ kv_status_t kv_append(kv_pool_t* p, const void* k_new, const void* v_new, const 
   if (!on_pool_device(p)) return KV_ERR_INVALID;
   const AppendArgs a{(const uint4*)k_new, (const uint4*)v_new, cu_new, start_pos, seg_row, block_tables, max_pages, n_segments,
                      total_new};
-  append_kernel<<<grid_for(p, (int64_t)total_new * 32, 256), 256, 0, (cudaStream_t)stream>>>(p->view(), a);  // one warp per token
+  const unsigned blocks = (unsigned)grid_for(p, (int64_t)total_new * 32, 256);  // one warp per token
+  const int chunks = p->n_kv_heads * (p->head_dim >> 3);
+  const auto kernel = chunks <= 64 ? append_kernel<2> : chunks <= 128 ? append_kernel<4> : append_kernel<8>;
+  KV_CUDA_OK(launch_early(kernel, blocks, 256, (cudaStream_t)stream, p->view(), a));
   count_launch();
-  KV_CUDA_OK(cudaGetLastError());
   return KV_OK;
 }
 
