@@ -60,9 +60,11 @@ struct SpanArgs {
   int plan_early;        // the kernel in front is this call's own append: the lengths may be read before waiting for it
   int4* desc;            // [n_spans][3]: the cut at the start of a span: (first step of the item it goes through among all
                          // steps, or -1; step of the item; KV head; tile pair), (rows, first row, KV steps of the two tiles)
-  float* part_o;         // [n_spans][2][D / 8][256][8]: a cut item's rows, normalised within the chunk (nullptr: no item is
-                         // cut); eight dims of a row, then the next row, so that a warp's rows are contiguous
-  float* part_lse;       // [n_spans][2][256]: log2-domain log-sum-exp of the chunk
+  int rows;              // rows a slot of partial results holds (no item of the batch has more)
+  float* part_o;         // [slot][D / 8][rows][8]: a cut item's rows, normalised within the chunk (nullptr: no item is cut);
+                         // eight dims of a row, then the next row, so that a warp's rows are contiguous.  Slots: two per
+                         // span, or one per CTA of the clusters
+  float* part_lse;       // [slot][rows]: log2-domain log-sum-exp of the chunk
 };
 constexpr int kSpanMinSteps = 2;  // KV steps of a span at least
 constexpr int kSpanSnap = 1;      // a cut this close to the edge of an item moves to the edge
@@ -566,12 +568,12 @@ __device__ __forceinline__ void issue_pv_mmas(uint32_t o_tmem, uint32_t p_tmem, 
     if (p < np) mma_ts(o_tmem, p_tmem + p * 8, make_desc(kHiV, v_lo + p * (D * 2)), idesc, 1u);
 }
 
-// Partial results lie in pieces of eight dims: [slot][D / 8][256 rows][8].
+// Partial results lie in pieces of eight dims: [slot][D / 8][rows][8].
 // 32 dims of a row, scaled, from registers: four pieces (a warp's 32 rows are contiguous in each).
-__device__ __forceinline__ void store_part8x4(float* dst, const uint32_t (&o)[32], float inv) {
+__device__ __forceinline__ void store_part8x4(float* dst, int rows, const uint32_t (&o)[32], float inv) {
 #pragma unroll
   for (int i = 0; i < 4; ++i)
-    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(dst + 256 * 8 * i),
+    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(dst + (int64_t)rows * 8 * i),
                  "f"(__uint_as_float(o[8 * i]) * inv), "f"(__uint_as_float(o[8 * i + 1]) * inv),
                  "f"(__uint_as_float(o[8 * i + 2]) * inv), "f"(__uint_as_float(o[8 * i + 3]) * inv),
                  "f"(__uint_as_float(o[8 * i + 4]) * inv), "f"(__uint_as_float(o[8 * i + 5]) * inv),
@@ -594,8 +596,8 @@ __device__ __forceinline__ uint4 merge_part8(const SpanArgs& a, int chunks, int 
       l[u] = -INFINITY;
       if (k < chunks && has(k)) {
         const int sl = slot(k);
-        l[u] = __ldcg(a.part_lse + sl * 256 + r);
-        const float4* src = reinterpret_cast<const float4*>(a.part_o + (((int64_t)sl * (D / 8) + g) * 256 + r) * 8);
+        l[u] = __ldcg(a.part_lse + sl * a.rows + r);
+        const float4* src = reinterpret_cast<const float4*>(a.part_o + (((int64_t)sl * (D / 8) + g) * a.rows + r) * 8);
         const float4 v0 = __ldcg(src), v1 = __ldcg(src + 1);
         x[u][0] = v0.x; x[u][1] = v0.y; x[u][2] = v0.z; x[u][3] = v0.w;
         x[u][4] = v1.x; x[u][5] = v1.y; x[u][6] = v1.z; x[u][7] = v1.w;
@@ -1139,7 +1141,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
           }
           if (SPAN && it.part >= 0) {  // a chunk of a cut item: its rows stay in fp32 until the chunks are merged
             if (valid) {
-              store_part8x4(a.span.part_o + (((int64_t)it.part * (D / 8) + c * 4) * 256 + t * 128 + m) * 8, orow, inv);
+              store_part8x4(a.span.part_o + (((int64_t)it.part * (D / 8) + c * 4) * a.span.rows + t * 128 + m) * 8, a.span.rows, orow, inv);
             }
             continue;
           }
@@ -1386,7 +1388,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
       mbar_arrive(bar_l_full);
       ++items_done;
       if (SPAN && part >= 0) {
-        if (valid) a.span.part_lse[part * 256 + t * 128 + m] = l_run > 0.f ? m_run + log2f(l_run) : -INFINITY;
+        if (valid) a.span.part_lse[part * a.span.rows + t * 128 + m] = l_run > 0.f ? m_run + log2f(l_run) : -INFINITY;
       } else if (valid) {
         a.lse[orow_idx] = (m_run + log2f(l_run)) * 0.6931471805599453f;
       }
@@ -1406,10 +1408,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
           uint32_t orow[32];
           tmem_ld32(o_addr + c * 32, orow);
           tmem_wait_ld();
-          if (row < u.x) store_part8x4(a.span.part_o + (((int64_t)blockIdx.x * (D / 8) + c * 4) * 256 + row) * 8, orow, inv);
+          if (row < u.x) store_part8x4(a.span.part_o + (((int64_t)blockIdx.x * (D / 8) + c * 4) * a.span.rows + row) * 8, a.span.rows, orow, inv);
         }
       }
-      a.span.part_lse[blockIdx.x * 256 + row] = cl_l > 0.f ? cl_m + log2f(cl_l) : -INFINITY;
+      if (row < u.x) a.span.part_lse[blockIdx.x * a.span.rows + row] = cl_l > 0.f ? cl_m + log2f(cl_l) : -INFINITY;
       cluster_arrive();
       cluster_wait();
       const int r_begin = u.x * rank / splits, cnt = u.x * (rank + 1) / splits - r_begin;
@@ -1520,7 +1522,7 @@ static int64_t item_capacity(int n_q_heads, int n_kv_heads, int batch, int total
 }
 
 struct SpanLayout {
-  int n_spans;
+  int n_spans, slots, rows;
   bool cuts;              // may an item be cut?
   size_t lse, o, total;   // behind the cuts
 };
@@ -1533,10 +1535,12 @@ static SpanLayout span_layout(const kv_pool_t* p, int n_q_heads, int batch, int 
   SpanLayout l;
   l.n_spans = (int)(spans < 1 ? 1 : spans < sms ? spans : sms);
   l.cuts = steps > 2 * kSpanSnap + 1;  // (an item of up to that many steps is never cut)
-  const size_t rows = l.cuts ? (size_t)sms * 2 * 256 : 0;  // (two per span, or one per CTA of the clusters)
+  const int64_t rows = (int64_t)total_q * (n_q_heads / p->n_kv_heads);
+  l.slots = l.cuts ? 2 * l.n_spans : 0;
+  l.rows = (int)(rows < 256 ? (rows + 7) / 8 * 8 : 256);
   l.lse = align256((size_t)l.n_spans * 3 * sizeof(int4));
-  l.o = l.lse + align256(rows * sizeof(float));
-  l.total = l.o + rows * p->head_dim * sizeof(float);
+  l.o = l.lse + align256((size_t)l.slots * l.rows * sizeof(float));
+  l.total = l.o + (size_t)l.slots * l.rows * p->head_dim * sizeof(float);
   return l;
 }
 static size_t list_bytes(int batch, int total_q) {
@@ -1698,7 +1702,7 @@ static kv_status_t choose_schedule(const kv_pool_t* p, int n_q_heads, int batch,
     *sched = kSchedCluster;
     if (!room || !l.cuts) return KV_OK;
     for (int c : kSplitChoices) {
-      if (c > steps) break;
+      if (c > steps || units * c > l.slots) break;
       int resident = 0;
       const kv_status_t s = p->head_dim == 128 ? resident_clusters<128>(p->device, c, &resident) : resident_clusters<64>(p->device, c, &resident);
       if (s != KV_OK) return s;
@@ -1717,6 +1721,7 @@ static SpanArgs span_args(const SpanLayout& l, char* ws, int max_tp, int total_q
   a.per_cta = cta_cap > 0 ? (l.n_spans + cta_cap - 1) / cta_cap : 1;
   a.max_tp = max_tp;
   a.total_q = total_q;
+  a.rows = l.rows;
   a.desc = reinterpret_cast<int4*>(ws);
   a.part_lse = l.cuts ? reinterpret_cast<float*>(ws + l.lse) : nullptr;
   a.part_o = l.cuts ? reinterpret_cast<float*>(ws + l.o) : nullptr;
