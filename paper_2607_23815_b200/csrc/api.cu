@@ -178,6 +178,73 @@ kv_status_t attn_extend_shared(kv_pool_t* p, const void* q, int n_q_heads, const
 }
 
 // ---- one call from host buffers ---------------------------------------------------------------
+// Copies by a kernel between pinned host memory and the device: several arrays in one launch.  The copy engines take turns
+// at every start of a copy: 32 MB in and 21 MB out at the same time take 680 us with one copy each way and 800 with the
+// three large and four small ones that a step has in.  So the lengths and tables always go by a kernel (the 16-tuple step
+// 768 -> 697 us), the rows of a step up to the limits below as well; above, the engines are faster (rows out by a
+// kernel: the 2-tuple step of 0.35 MB of Q 40.8 -> 34.2 us, 4 tuples of 3.5 MB 163 -> 146, but 16 of 21.9 MB 697 -> 738,
+// because it holds an SM that the next step's attention kernel wants).
+namespace {
+constexpr int kMaxCopies = 7;
+constexpr size_t kKernelCopyIn = size_t(1) << 20;   // bytes of the rows in / out up to which a kernel copies them
+constexpr size_t kKernelCopyOut = size_t(4) << 20;
+struct Copies {
+  int n = 0;
+  const char* src[kMaxCopies];
+  char* dst[kMaxCopies];
+  size_t bytes[kMaxCopies];  // multiples of 4
+  void add(void* d, const void* s, size_t b) {
+    src[n] = (const char*)s;
+    dst[n] = (char*)d;
+    bytes[n++] = b;
+  }
+  size_t total() const {
+    size_t t = 0;
+    for (int i = 0; i < n; ++i) t += bytes[i];
+    return t;
+  }
+};
+
+__global__ void __launch_bounds__(512) copy_kernel(const Copies c) {
+  const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+  for (int k = 0; k < c.n; ++k) {
+    const char* __restrict__ src = c.src[k];
+    char* __restrict__ dst = c.dst[k];
+    const size_t whole = (((uintptr_t)src | (uintptr_t)dst) & 15) == 0 ? c.bytes[k] / 16 : 0;  // 16-byte pieces
+    for (size_t i = t; i < whole; i += 4 * step) {
+      uint4 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (i + u * step < whole) v[u] = __ldcs(reinterpret_cast<const uint4*>(src) + i + u * step);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (i + u * step < whole) __stcs(reinterpret_cast<uint4*>(dst) + i + u * step, v[u]);
+    }
+    for (size_t i = whole * 4 + t; i < c.bytes[k] / 4; i += step)
+      reinterpret_cast<unsigned*>(dst)[i] = reinterpret_cast<const unsigned*>(src)[i];
+  }
+}
+
+kv_status_t launch_copies(const Copies& c, size_t max_blocks, cudaStream_t st) {
+  if (c.n == 0) return KV_OK;
+  const size_t blocks = (c.total() + 65535) / 65536;
+  copy_kernel<<<(unsigned)(blocks < 1 ? 1 : blocks < max_blocks ? blocks : max_blocks), 512, 0, st>>>(c);
+  count_launch();
+  KV_CUDA_OK(cudaGetLastError());
+  return KV_OK;
+}
+
+// The address at which the device reaches a pinned host buffer, nullptr if it cannot (pageable memory).
+void* device_view(const void* host) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, host) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return a.type == cudaMemoryTypeHost && ((uintptr_t)a.devicePointer & 3) == 0 ? a.devicePointer : nullptr;
+}
+}  // namespace
+
 // Layout of the staging area: the device copies of the inputs and results, each 256-byte aligned, followed by the
 // attention workspace.
 namespace {
@@ -246,14 +313,24 @@ kv_status_t attn_extend_host(kv_pool_t* p, const void* q, const void* k_new, con
     }
   }
   KV_CUDA_OK(cudaStreamWaitEvent(p->h2d_stream, hs->ran, 0));  // (a never-recorded event counts as complete)
-  KV_CUDA_OK(cudaMemcpyAsync(d + L.k, k_new, kv_bytes, cudaMemcpyHostToDevice, p->h2d_stream));
-  KV_CUDA_OK(cudaMemcpyAsync(d + L.v, v_new, kv_bytes, cudaMemcpyHostToDevice, p->h2d_stream));
-  KV_CUDA_OK(cudaMemcpyAsync(d + L.q, q, q_bytes, cudaMemcpyHostToDevice, p->h2d_stream));
-  KV_CUDA_OK(cudaMemcpyAsync(d + L.cu, cu_q, sizeof(int) * ((size_t)batch + 1), cudaMemcpyHostToDevice, p->h2d_stream));
-  KV_CUDA_OK(cudaMemcpyAsync(d + L.bt, block_tables, sizeof(int) * (size_t)batch * max_pages, cudaMemcpyHostToDevice,
-                             p->h2d_stream));
-  KV_CUDA_OK(cudaMemcpyAsync(d + L.pl, prefix_lens, sizeof(int) * (size_t)batch, cudaMemcpyHostToDevice, p->h2d_stream));
-  KV_CUDA_OK(cudaMemcpyAsync(d + L.el, extend_lens, sizeof(int) * (size_t)batch, cudaMemcpyHostToDevice, p->h2d_stream));
+  {
+    // by a kernel: the lengths and tables, and the rows of a small step; by the copy engine: large rows, pageable buffers
+    const struct { size_t at; const void* src; size_t bytes; bool rows; } in[] = {
+        {L.k, k_new, kv_bytes, true}, {L.v, v_new, kv_bytes, true}, {L.q, q, q_bytes, true},
+        {L.cu, cu_q, sizeof(int) * ((size_t)batch + 1), false}, {L.bt, block_tables, sizeof(int) * (size_t)batch * max_pages, false},
+        {L.pl, prefix_lens, sizeof(int) * (size_t)batch, false}, {L.el, extend_lens, sizeof(int) * (size_t)batch, false}};
+    const bool small = 2 * kv_bytes + q_bytes <= kKernelCopyIn;
+    Copies c;
+    for (const auto& i : in) {
+      const void* view = i.rows && !small ? nullptr : device_view(i.src);
+      if (view != nullptr)
+        c.add(d + i.at, view, i.bytes);
+      else
+        KV_CUDA_OK(cudaMemcpyAsync(d + i.at, i.src, i.bytes, cudaMemcpyHostToDevice, p->h2d_stream));
+    }
+    const kv_status_t cs = launch_copies(c, 8, p->h2d_stream);
+    if (cs != KV_OK) return cs;
+  }
   KV_CUDA_OK(cudaEventRecord(hs->in, p->h2d_stream));
   KV_CUDA_OK(cudaStreamWaitEvent(st, hs->in, 0));
   const int* d_cu = reinterpret_cast<const int*>(d + L.cu);
@@ -267,8 +344,19 @@ kv_status_t attn_extend_host(kv_pool_t* p, const void* q, const void* k_new, con
   KV_CUDA_OK(cudaEventRecord(hs->ran, st));
   if (s != KV_OK) return s;
   KV_CUDA_OK(cudaStreamWaitEvent(p->d2h_stream, hs->ran, 0));
-  KV_CUDA_OK(cudaMemcpyAsync(out, d + L.out, q_bytes, cudaMemcpyDeviceToHost, p->d2h_stream));
-  KV_CUDA_OK(cudaMemcpyAsync(lse, d + L.lse, (size_t)total_q * n_q_heads * 4, cudaMemcpyDeviceToHost, p->d2h_stream));
+  {
+    Copies c;
+    const struct { void* dst; size_t at, bytes; } res[] = {{out, L.out, q_bytes}, {lse, L.lse, (size_t)total_q * n_q_heads * 4}};
+    for (const auto& r : res) {
+      void* view = q_bytes <= kKernelCopyOut ? device_view(r.dst) : nullptr;
+      if (view != nullptr)
+        c.add(view, d + r.at, r.bytes);
+      else
+        KV_CUDA_OK(cudaMemcpyAsync(r.dst, d + r.at, r.bytes, cudaMemcpyDeviceToHost, p->d2h_stream));
+    }
+    const kv_status_t cs = launch_copies(c, 4, p->d2h_stream);
+    if (cs != KV_OK) return cs;
+  }
   KV_CUDA_OK(cudaEventRecord(hs->out, p->d2h_stream));
   KV_CUDA_OK(cudaStreamWaitEvent(st, hs->out, 0));
   return KV_OK;

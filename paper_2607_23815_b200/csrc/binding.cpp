@@ -224,6 +224,29 @@ PyObject* mixed(PyObject*, PyObject* const* a, Py_ssize_t n) {
   });
 }
 
+const at::Tensor& host_tensor(PyObject* o) {
+  if (!THPVariable_Check(o)) raise(PyExc_TypeError, "expected a torch tensor");
+  const at::Tensor& t = THPVariable_Unpack(o);
+  if (t.is_cuda() || !t.is_contiguous()) raise(PyExc_ValueError, "attn_extend_host takes contiguous host tensors");
+  return t;
+}
+PyObject* extend_host(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return call(n, 15, [&] {
+    kv_pool_t* p = pool(a[0]);
+    const at::Tensor &q = host_tensor(a[1]), &k = host_tensor(a[2]), &v = host_tensor(a[3]), &cu = host_tensor(a[4]), &bt = host_tensor(a[5]),
+                     &pl = host_tensor(a[6]), &el = host_tensor(a[7]), &out = host_tensor(a[11]), &lse = host_tensor(a[12]);
+    const int max_e = integer(a[8]), max_l = integer(a[9]), hq = size(q, 1), total = size(q, 0), pages = size(bt, 1);
+    const float scale = real(a[10]);
+    const Workspace staging(a[13]);
+    void* st = stream(a[14]);
+    return unlocked([&] {
+      return attn_extend_host(p, data(q), data(k), data(v), hq, (const int*)data(cu), (const int*)data(bt), pages, (const int*)data(pl),
+                              (const int*)data(el), (int)pl.numel(), total, max_e, max_l, scale, data(out), (float*)data(lse), staging.p,
+                              staging.bytes, st);
+    });
+  });
+}
+
 #define ENTRY(name, fn) {name, (PyCFunction)(void (*)(void))fn, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {ENTRY("kv_append", append),
                          ENTRY("attn_decode", decode),
@@ -233,6 +256,7 @@ PyMethodDef methods[] = {ENTRY("kv_append", append),
                          ENTRY("attn_extend_planned", extend_planned),
                          ENTRY("attn_extend_shared", extend_shared),
                          ENTRY("attn_mixed", mixed),
+                         ENTRY("attn_extend_host", extend_host),
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_kvattn_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 

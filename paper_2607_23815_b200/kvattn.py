@@ -305,16 +305,8 @@ def attn_extend_host(pool: Pool, q, k_new, v_new, cu_q, block_tables, prefix_len
                      max_total_len, scale, out, lse, staging, stream=None):
     """One step from host tensors (pinned for asynchrony): copies in, kv_append of the suffix, attn_extend, copies out.
     `staging` is a device byte tensor of attn_extend_host_staging_bytes() bytes."""
-    for t in (q, k_new, v_new, cu_q, block_tables, prefix_lens, extend_lens, out, lse):
-        if t.is_cuda or not t.is_contiguous():
-            raise ValueError("attn_extend_host takes contiguous host tensors")
-    _check(lib().attn_extend_host(pool.handle, C.c_void_p(q.data_ptr()), C.c_void_p(k_new.data_ptr()),
-                                  C.c_void_p(v_new.data_ptr()), q.shape[1], C.c_void_p(cu_q.data_ptr()),
-                                  C.c_void_p(block_tables.data_ptr()), block_tables.shape[1],
-                                  C.c_void_p(prefix_lens.data_ptr()), C.c_void_p(extend_lens.data_ptr()),
-                                  prefix_lens.numel(), q.shape[0], max_extend_len, max_total_len, float(scale),
-                                  C.c_void_p(out.data_ptr()), C.c_void_p(lse.data_ptr()), _dev_ptr(staging),
-                                  staging.numel() * staging.element_size(), _stream(stream)), "attn_extend_host")
+    _check(_native.attn_extend_host(pool.ptr, q, k_new, v_new, cu_q, block_tables, prefix_lens, extend_lens, max_extend_len,
+                                    max_total_len, scale, out, lse, staging, stream), "attn_extend_host")
 
 
 def kvattn_set_shared_impl(impl: int):

@@ -1,0 +1,58 @@
+"""attn_extend_host from pinned and pageable buffers, in steps small enough for its copy kernel and larger ones, with
+addresses that are not 16-byte aligned, one staging area and two in turn: the bits of the call on device tensors."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2607_23815_b200 import kvattn, synth
+from harness import Batch, DualPool
+
+pytestmark = pytest.mark.gpu
+
+
+def _host(t, pinned, shift=0):
+    """A host copy of t; shift: elements by which it starts off its buffer's beginning."""
+    flat = torch.empty(t.numel() + shift, dtype=t.dtype, pin_memory=pinned)
+    view = flat[shift:shift + t.numel()].view(t.shape)
+    view.copy_(t)
+    return view
+
+
+@pytest.mark.parametrize("pinned", [True, False, "mixed"])
+@pytest.mark.parametrize("extend", [[5, 1], [60, 33], [600, 300, 1]])
+def test_host_step_gives_the_bits_of_the_device_call(extend, pinned):
+    geom = synth.Geometry(8, 2, 128)                       # the largest suffix set: 4.6 MB of rows, above the kernel's limit
+    P = [37, 250, 16][:len(extend)]
+    L = [p + e for p, e in zip(P, extend)]
+    outs = []
+    for way in ("device", "host"):
+        dp = DualPool(geom, 256, seed=71, with_oracle=False)
+        b = Batch(dp, L)
+        b.write([(i, 0, P[i]) for i in range(len(P))])
+        ks, vs = zip(*[b.kv(i, P[i], L[i]) for i in range(len(P))])
+        k, v = torch.cat(ks).contiguous(), torch.cat(vs).contiguous()
+        q = torch.cat([b.q(i, P[i], L[i]) for i in range(len(P))]).contiguous()
+        i32 = lambda x: torch.tensor(np.asarray(x), dtype=torch.int32)
+        cu, bt, pl, el = i32(np.concatenate([[0], np.cumsum(extend)])), torch.from_numpy(b.block_tables()), i32(P), i32(extend)
+        bounds = (max(extend), max(L), geom.scale)
+        if way == "device":
+            out, lse = torch.empty_like(q), torch.empty((q.shape[0], 8), device="cuda")
+            ws = torch.empty(kvattn.attn_workspace_bytes(dp.pool, 8, len(P), int(q.shape[0]), max(L)), dtype=torch.uint8, device="cuda")
+            kvattn.attn_extend_append(dp.pool, q, k, v, cu.cuda(), bt.cuda(), pl.cuda(), el.cuda(), *bounds, out, lse, ws)
+            outs.append((synth.bf16_bits(out), lse.cpu().numpy(), dp.device_image()))
+        else:
+            pin = lambda i: pinned if pinned != "mixed" else i % 2 == 0
+            h = [_host(t, pin(i), shift=1 if t.dtype == torch.int32 else 0) for i, t in enumerate((q, k, v, cu, bt, pl, el))]
+            size = kvattn.attn_extend_host_staging_bytes(dp.pool, 8, len(P), int(q.shape[0]), bt.shape[1], max(L))
+            areas = [torch.empty(size, dtype=torch.uint8, device="cuda") for _ in range(2)]
+            for step in range(5):                           # (an append of the same rows again changes nothing)
+                o = _host(torch.full(q.shape, float("nan"), dtype=torch.bfloat16), pin(0))
+                l = _host(torch.full((q.shape[0], 8), float("nan")), pin(1), shift=1)
+                kvattn.attn_extend_host(dp.pool, *h, *bounds, o, l, areas[step % 2])
+                torch.cuda.current_stream().synchronize()
+                outs.append((synth.bf16_bits(o), l.numpy().copy(), dp.device_image()))
+        assert kvattn.kv_last_async_status(dp.pool) == kvattn.KV_OK
+        dp.close()
+    for o in outs[1:]:
+        assert np.array_equal(o[0], outs[0][0]) and np.array_equal(o[1], outs[0][1])
+        assert np.array_equal(o[2][0], outs[0][2][0]) and np.array_equal(o[2][1], outs[0][2][1])
