@@ -234,14 +234,17 @@ kv_status_t launch_copies(const Copies& c, size_t max_blocks, cudaStream_t st) {
   return KV_OK;
 }
 
-// The address at which the device reaches a pinned host buffer, nullptr if it cannot (pageable memory).
-void* device_view(const void* host) {
-  cudaPointerAttributes a;
-  if (cudaPointerGetAttributes(&a, host) != cudaSuccess) {
+// The address at which the device reaches a host buffer that is pinned from its first byte to its last, else nullptr.
+void* device_view(const void* host, size_t bytes) {
+  cudaPointerAttributes a, z;
+  if (cudaPointerGetAttributes(&a, host) != cudaSuccess ||
+      cudaPointerGetAttributes(&z, (const char*)host + bytes - 1) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
   }
-  return a.type == cudaMemoryTypeHost && ((uintptr_t)a.devicePointer & 3) == 0 ? a.devicePointer : nullptr;
+  const bool pinned = a.type == cudaMemoryTypeHost && z.type == cudaMemoryTypeHost &&
+                      (const char*)z.devicePointer - (const char*)a.devicePointer == (ptrdiff_t)bytes - 1;
+  return pinned && ((uintptr_t)a.devicePointer & 3) == 0 ? a.devicePointer : nullptr;
 }
 }  // namespace
 
@@ -322,7 +325,7 @@ kv_status_t attn_extend_host(kv_pool_t* p, const void* q, const void* k_new, con
     const bool small = 2 * kv_bytes + q_bytes <= kKernelCopyIn;
     Copies c;
     for (const auto& i : in) {
-      const void* view = i.rows && !small ? nullptr : device_view(i.src);
+      const void* view = i.rows && !small ? nullptr : device_view(i.src, i.bytes);
       if (view != nullptr)
         c.add(d + i.at, view, i.bytes);
       else
@@ -348,13 +351,13 @@ kv_status_t attn_extend_host(kv_pool_t* p, const void* q, const void* k_new, con
     Copies c;
     const struct { void* dst; size_t at, bytes; } res[] = {{out, L.out, q_bytes}, {lse, L.lse, (size_t)total_q * n_q_heads * 4}};
     for (const auto& r : res) {
-      void* view = q_bytes <= kKernelCopyOut ? device_view(r.dst) : nullptr;
+      void* view = q_bytes <= kKernelCopyOut ? device_view(r.dst, r.bytes) : nullptr;
       if (view != nullptr)
         c.add(view, d + r.at, r.bytes);
       else
         KV_CUDA_OK(cudaMemcpyAsync(r.dst, d + r.at, r.bytes, cudaMemcpyDeviceToHost, p->d2h_stream));
     }
-    const kv_status_t cs = launch_copies(c, 4, p->d2h_stream);
+    const kv_status_t cs = launch_copies(c, 2, p->d2h_stream);
     if (cs != KV_OK) return cs;
   }
   KV_CUDA_OK(cudaEventRecord(hs->out, p->d2h_stream));
