@@ -311,8 +311,9 @@ kv_status_t kvattn_set_shared_impl(int impl);
  * through a per-warp ring of page slots in shared memory filled by bulk copies (several pages per warp in flight);
  * 0 = the default, which is 2.  Same arithmetic, same bits.  Process-wide; for tests and benchmarks. */
 kv_status_t kvattn_set_decode_impl(int impl);
-/* Tuning: inside attn_mixed (both sets present) the persistent extend kernel takes at most n SMs, so that the
- * HBM-bound decode kernel runs beside it on the others instead of after it.  0 = derived from the bounds of the two
+/* Tuning: inside attn_mixed (both sets present) the persistent extend kernel takes n SMs, so that the HBM-bound decode
+ * kernel runs beside it on the others instead of after it (an extend set cut into equal spans: as many spans per SM as
+ * come nearest to that; one with so few items that each has SMs of its own: those).  0 = derived from the bounds of the two
  * batches (the default).  Process-wide. */
 kv_status_t kvattn_set_mixed_extend_ctas(int n);
 /* Test surface (the paper has no counterpart): runs a one-CTA kernel whose warps wait, with the same bounded

@@ -434,14 +434,23 @@ kv_status_t attn_mixed(kv_pool_t* p, int n_q_heads, float scale, const attn_exte
     // SMs the extend CTAs give back.  It waits for nothing: it reads and writes nothing the extend kernel writes.
     int cap = g_mixed_extend_ctas.load();
     if (cap <= 0) {
-      // Share of the SMs by the two kinds of work, from the host-side bounds: extend costs its flops at the rate the
-      // kernel reaches per SM, decode its bytes at the rate at which about two thirds of the SMs saturate the memory.
-      const int sms = sm_count_of(p->device);
-      const double flops = 4.0 * p->head_dim * n_q_heads * (double)ext->total_q * 0.75 * ext->max_total_len;
+      // Share of the SMs by the two kinds of work, from the host-side bounds: the extend kernel costs its items, of so
+      // many KV steps each (what a step of two query tiles and an item's ends take, whatever the rows in the tiles), the
+      // decode kernel its bytes at the rate at which about two thirds of the SMs saturate the memory.  Batches of short
+      // suffixes fill few rows of a tile: by its flops at 800 TFLOP/s the extend kernel was given 43 of 148 SMs for 39
+      // sequences of 24 tokens (8/8 heads) beside 49 decodes, 84 us against 50 with 116 SMs; 46 of 17 tokens 61 and 31.
+      // Up to all SMs: 41 of 26-96 tokens beside 5 decodes 94 us with 116, 82 with 148; but 48 of up to 192 beside 192
+      // decodes of up to 4100 398 with 72 and 463 with 148.
+      const int sms = sm_count_of(p->device), G = n_q_heads / p->n_kv_heads;
+      const double pairs = ((int64_t)ext->max_extend_len * G + 255) / 256, n = ext->batch;
+      const double some = (double)ext->total_q * G / 256 + 0.5 * n;  // (a sequence's last tile pair is half full)
+      const double items = (pairs < 2 ? n : n * pairs < some ? n * pairs : some) * p->n_kv_heads;
+      const double steps = 0.8 * ((ext->max_total_len + 127) / 128);
+      const double item_us = (steps > 1 ? steps : 1) * (p->head_dim == 128 ? 1.75 : 1.4) + 2.5;
       const double bytes = (double)dec->batch * 0.62 * dec->max_ctx_len * 2.0 * p->n_kv_heads * p->head_dim * 2.0;
-      const double sm_s_ext = flops / 800e12 * sms, sm_s_dec = bytes / 6e12 * (sms * 0.68);
-      cap = (int)(sms * sm_s_ext / (sm_s_ext + sm_s_dec) + 0.5);
-      cap = cap < 16 ? 16 : (cap > sms - 32 ? sms - 32 : cap);
+      const double sm_us_ext = items * item_us, sm_us_dec = (bytes / 6e6 + 3.0) * (sms * 0.68);
+      cap = (int)(sms * sm_us_ext / (sm_us_ext + sm_us_dec) + 0.5);
+      cap = cap < 16 ? 16 : cap;
     }
     kv_status_t s = extend_impl(p, ext->q, n_q_heads, ext->cu_q, ext->block_tables, ext->max_pages, ext->prefix_lens,
                                 ext->extend_lens, ext->batch, ext->total_q, ext->max_extend_len, ext->max_total_len,

@@ -1718,7 +1718,9 @@ static kv_status_t choose_schedule(const kv_pool_t* p, int n_q_heads, int batch,
 static SpanArgs span_args(const SpanLayout& l, char* ws, int max_tp, int total_q, int cta_cap) {
   SpanArgs a{};
   a.n_spans = l.n_spans;  // (not the number of CTAs: the cuts, and with them the bits, are the same beside a decode kernel)
-  a.per_cta = cta_cap > 0 ? (l.n_spans + cta_cap - 1) / cta_cap : 1;
+  // Two spans a CTA pay where the decode kernel, on the SMs that this leaves, takes longer than the extend kernel on all of
+  // them; that is where the share is 0.6 of the SMs (three: 0.37).
+  a.per_cta = cta_cap > 0 ? max(1, (int)((double)l.n_spans / cta_cap + 0.32)) : 1;
   a.max_tp = max_tp;
   a.total_q = total_q;
   a.rows = l.rows;
