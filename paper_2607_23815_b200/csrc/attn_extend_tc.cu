@@ -64,7 +64,7 @@ struct SpanArgs {
   float* part_o;         // [slot][D / 8][rows][8]: a cut item's rows, normalised within the chunk (nullptr: no item is cut);
                          // eight dims of a row, then the next row, so that a warp's rows are contiguous.  Slots: two per
                          // span, or one per CTA of the clusters
-  float* part_lse;       // [slot][rows]: log2-domain log-sum-exp of the chunk
+  float* part_lse;       // [slot][rows]: log2-domain log-sum-exp of the chunk (clusters: the maximum and the sum)
 };
 constexpr int kSpanMinSteps = 2;  // KV steps of a span at least
 constexpr int kSpanSnap = 1;      // a cut this close to the edge of an item moves to the edge
@@ -580,6 +580,20 @@ __device__ __forceinline__ void store_part8x4(float* dst, int rows, const uint32
                  "f"(__uint_as_float(o[8 * i + 6]) * inv), "f"(__uint_as_float(o[8 * i + 7]) * inv)
                  : "memory");
 }
+__device__ __forceinline__ void store_part8x4(float* dst, int rows, const uint32_t (&o)[32]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(dst + (int64_t)rows * 8 * i), "r"(o[8 * i]), "r"(o[8 * i + 1]),
+                 "r"(o[8 * i + 2]), "r"(o[8 * i + 3]), "r"(o[8 * i + 4]), "r"(o[8 * i + 5]), "r"(o[8 * i + 6]), "r"(o[8 * i + 7])
+                 : "memory");
+}
+// A piece of a partial result: 32 bytes in one load (two of 16 bytes ask for every sector twice).
+__device__ __forceinline__ void load_part8(const float* src, float (&x)[8]) {
+  asm volatile("ld.global.L1::no_allocate.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7])
+               : "l"(src)
+               : "memory");
+}
 // Merges piece g of row r over its chunks, in chunk order, U chunks' loads in flight: eight dims as bf16, and the
 // log2-domain log-sum-exp.  slot(k): slot of chunk k; has(k): does chunk k hold a step of the row's tile (else its slot
 // was not written; a chunk without a key the row sees has weight 0).
@@ -597,10 +611,7 @@ __device__ __forceinline__ uint4 merge_part8(const SpanArgs& a, int chunks, int 
       if (k < chunks && has(k)) {
         const int sl = slot(k);
         l[u] = __ldcg(a.part_lse + sl * a.rows + r);
-        const float4* src = reinterpret_cast<const float4*>(a.part_o + (((int64_t)sl * (D / 8) + g) * a.rows + r) * 8);
-        const float4 v0 = __ldcg(src), v1 = __ldcg(src + 1);
-        x[u][0] = v0.x; x[u][1] = v0.y; x[u][2] = v0.z; x[u][3] = v0.w;
-        x[u][4] = v1.x; x[u][5] = v1.y; x[u][6] = v1.z; x[u][7] = v1.w;
+        load_part8(a.part_o + (((int64_t)sl * (D / 8) + g) * a.rows + r) * 8, x[u]);
       }
     }
 #pragma unroll
@@ -1395,34 +1406,86 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
     }
     if (CLUSTER && a.cl_splits > 1) {
       // The CTAs of the cluster hold partial results of the same rows.  Each writes its own out, then finishes an equal
-      // share of the rows from everybody's.  Through L2: read from the partners' shared memory, 148 rows on 8 CTAs took
-      // 8800 cycles (about 8 bytes a cycle and SM), this way 2500.
+      // share of the rows from everybody's, through L2.  One sequence of 37 tokens behind 1500, 64 CTAs of 76 KB each: 1.4 us
+      // to write, 1.1 for the barrier behind the stores, 2.4 to merge; 3.6 with two loads of 16 bytes for a piece and the items
+      // one after the other, 3.7 with the weights computed once per row in front (another wait for L2).
       const int splits = a.cl_splits, unit = (int)blockIdx.x / splits, rank = (int)blockIdx.x - unit * splits;
       const int4 u = sm.cl_unit;
       const int row = t * 128 + m;
       if (__any_sync(0xffffffffu, cl_l > 0.f)) {
         tc_fence_after_sync();
-        const float inv = cl_l > 0.f ? 1.f / cl_l : 0.f;
+        float* dst = a.span.part_o + ((int64_t)blockIdx.x * (D / 8) * a.span.rows + row) * 8;
 #pragma unroll 1
-        for (int c = 0; c < D / 32; ++c) {
+        for (int c = 0; c < D / 32; ++c, dst += (int64_t)a.span.rows * 32) {
           uint32_t orow[32];
           tmem_ld32(o_addr + c * 32, orow);
           tmem_wait_ld();
-          if (row < u.x) store_part8x4(a.span.part_o + (((int64_t)blockIdx.x * (D / 8) + c * 4) * a.span.rows + row) * 8, a.span.rows, orow, inv);
+          if (row < u.x) store_part8x4(dst, a.span.rows, orow);
         }
       }
-      if (row < u.x) a.span.part_lse[blockIdx.x * a.span.rows + row] = cl_l > 0.f ? cl_m + log2f(cl_l) : -INFINITY;
+      float2* part_ml = reinterpret_cast<float2*>(a.span.part_lse);  // [CTA][row]: maximum (log2 domain) and sum
+      if (row < u.x) part_ml[blockIdx.x * a.span.rows + row] = make_float2(cl_m, cl_l);
+      __syncwarp();
       cluster_arrive();
       cluster_wait();
       const int r_begin = u.x * rank / splits, cnt = u.x * (rank + 1) / splits - r_begin;
-      for (int i = tid; i < cnt * (D / 8); i += 256) {
-        const int g = i / cnt, r = r_begin + (i - g * cnt);  // eight dims of a row; neighbouring lanes take neighbouring rows
-        float lse2;
-        const uint4 o = merge_part8<D, kMaxClusterSplits>(a.span, splits, r, g, [&](int k) { return unit * splits + k; }, [](int) { return true; }, lse2);
-        const int rg = u.z * 256 + r;
-        const int64_t orow = (int64_t)(u.y + (rg >> lg)) * Hq + u.w * G + (rg & (G - 1));
-        reinterpret_cast<uint4*>(a.out + orow * D)[g] = o;
-        if (g == 0) a.lse[orow] = lse2 * 0.6931471805599453f;
+      auto finish = [&](auto n) {
+        // Item i: eight dims of a row; neighbouring lanes take neighbouring rows.  As many items of a thread at a time as make
+        // sixteen loads: the wait for L2 is paid once.
+        constexpr int N = decltype(n)::value, ITEMS = 16 / N;
+        const int items = cnt * (D / 8);
+        for (int base = tid; base < items; base += 256 * ITEMS) {
+          float2 ml[ITEMS][N];
+          float x[ITEMS][N][8];
+#pragma unroll
+          for (int k = 0; k < ITEMS; ++k) {
+            const int i = base + 256 * k;
+            if (i >= items) break;
+            const int g = i / cnt, r = r_begin + (i - g * cnt);
+            const float2* src_ml = part_ml + unit * N * a.span.rows + r;
+            const float* src = a.span.part_o + (((int64_t)unit * N * (D / 8) + g) * a.span.rows + r) * 8;
+#pragma unroll
+            for (int c = 0; c < N; ++c, src_ml += a.span.rows, src += (int64_t)a.span.rows * D) {
+              ml[k][c] = __ldcg(src_ml);
+              load_part8(src, x[k][c]);
+            }
+          }
+#pragma unroll
+          for (int k = 0; k < ITEMS; ++k) {
+            const int i = base + 256 * k;
+            if (i >= items) break;
+            const int g = i / cnt, r = r_begin + (i - g * cnt);
+            float mx = -INFINITY, sum = 0.f;
+#pragma unroll
+            for (int c = 0; c < N; ++c) mx = fmaxf(mx, ml[k][c].x);
+            float2 o[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[e] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int c = 0; c < N; ++c) {
+              if (!(ml[k][c].y > 0.f)) continue;  // (no step of the row's tile, or no key that the row sees: not written)
+              const float w = exp2f(ml[k][c].x - mx);
+              sum += w * ml[k][c].y;
+#pragma unroll
+              for (int e = 0; e < 4; ++e) o[e] = __ffma2_rn(make_float2(x[k][c][2 * e], x[k][c][2 * e + 1]), make_float2(w, w), o[e]);
+            }
+            const float inv = 1.f / sum;
+            uint32_t pk[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pk[e]) : "f"(o[e].y * inv), "f"(o[e].x * inv));
+            const int rg = u.z * 256 + r;
+            const int64_t orow = (int64_t)(u.y + (rg >> lg)) * Hq + u.w * G + (rg & (G - 1));
+            reinterpret_cast<uint4*>(a.out + orow * D)[g] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            if (g == 0) a.lse[orow] = (mx + log2f(sum)) * 0.6931471805599453f;
+          }
+        }
+      };
+      switch (splits) {
+        case 2: finish(std::integral_constant<int, 2>{}); break;
+        case 3: finish(std::integral_constant<int, 3>{}); break;
+        case 4: finish(std::integral_constant<int, 4>{}); break;
+        case 6: finish(std::integral_constant<int, 6>{}); break;
+        default: finish(std::integral_constant<int, 8>{});
       }
     }
   }
@@ -1539,7 +1602,7 @@ static SpanLayout span_layout(const kv_pool_t* p, int n_q_heads, int batch, int 
   l.slots = l.cuts ? 2 * l.n_spans : 0;
   l.rows = (int)(rows < 256 ? (rows + 7) / 8 * 8 : 256);
   l.lse = align256((size_t)l.n_spans * 3 * sizeof(int4));
-  l.o = l.lse + align256((size_t)l.slots * l.rows * sizeof(float));
+  l.o = l.lse + align256((size_t)l.slots * l.rows * 2 * sizeof(float));
   l.total = l.o + (size_t)l.slots * l.rows * p->head_dim * sizeof(float);
   return l;
 }
