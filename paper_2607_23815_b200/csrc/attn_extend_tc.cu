@@ -1744,23 +1744,26 @@ static kv_status_t resident_clusters(int device, int c, int* n) {
 //    kernel, and the steps of an item run side by side.  Suffix append + extend of 1 / 4 / 8 / 16 sequences of 30-60 tokens
 //    behind 1000-2000 (32/8 heads of 128): 32.1 / 38.2 / 42.2 / 43.7 us through the list, 16.8 / 24.2 / 33.3 / 42.4 this
 //    way with 6 / 4 / 2 / 1 CTAs per item.
-//  - Few and long items: spans.  They cost a merge kernel behind the attention kernel (about 12 us, 8 steps) and win what
-//    the other two leave idle, the SMs without a cluster or the last round of items: 8 / 16 sequences of 9000-16000 keys
-//    219 / 225 us through the list, 121 / 242 with clusters, 102 / 181 with spans; 11 of up to 10700 (16/8 heads of 64)
-//    260 and 197; but 4 of 6900 with 128 items of equal length 112 and 120.  More than three items per SM, or short ones:
-//    the list (3 prefills of up to 1950 tokens, 4.2 items per SM: 85 against 98; 64 sequences, 12 per SM: 263 against 298).
+//  - Items that leave SMs idle: spans.  They cost a merge kernel behind the attention kernel and the partial results, 5 to
+//    8 steps, and win what the other two leave idle, the SMs without a cluster or the last round of items.  8 / 16 sequences
+//    of 9000-16000 keys 219 / 225 us through the list, 121 / 242 with clusters, 102 / 181 with spans; 160 items of 25 steps
+//    (1.1 rounds) 93 and 70, 184 of 13 to 16 (1.2) 50 and 46, 68 and 61, but 160 of 10 40 and 40, 168 of 5 30 and 31.  The
+//    number of items is known if a sequence has one; if it is estimated, the line lies higher: 320 of 22 (2.2) 122 and 106,
+//    240 of 13 57 and 59.  More than four items per SM: the list (672 of 36 348 against 369).
 static kv_status_t choose_schedule(const kv_pool_t* p, int n_q_heads, int batch, int total_q, int max_extend_len, int max_total_len,
                                    size_t workspace_bytes, int mode, int* sched, int* splits) {
   *sched = kSchedList;
   *splits = 1;
   const int G = n_q_heads / p->n_kv_heads, sms = sm_count_of(p->device);
-  const int64_t units = (int64_t)batch * (((int64_t)max_extend_len * G + 255) / 256) * p->n_kv_heads;
+  const int64_t pairs = ((int64_t)max_extend_len * G + 255) / 256, units = (int64_t)batch * pairs * p->n_kv_heads;
   const int64_t steps = ((int64_t)max_total_len + 127) / 128;
   const SpanLayout l = span_layout(p, n_q_heads, batch, total_q, max_total_len);
   const bool room = workspace_bytes >= 256 + l.total;  // (else: nothing that leaves partial results)
   const int64_t most = items_at_most(p, n_q_heads, batch, total_q);
-  // (a sequence's last tile pair is half full on average, its keys somewhat fewer than the longest's)
-  const double rounds = ((double)total_q * G / 256 + 0.5 * batch) * p->n_kv_heads / sms, even = 0.85 * steps * rounds;
+  // (a sequence's last tile pair is half full on average, its keys somewhat fewer than the longest's; sequences of one pair
+  // each are as many items as there are)
+  const double rounds = (pairs == 1 ? (double)batch : (double)total_q * G / 256 + 0.5 * batch) * p->n_kv_heads / sms;
+  const double even = 0.85 * steps * rounds;
   if (units <= sms || (most <= sms && units <= 2 * sms)) {
     *sched = kSchedCluster;
     if (!room || !l.cuts) return KV_OK;
@@ -1772,7 +1775,7 @@ static kv_status_t choose_schedule(const kv_pool_t* p, int n_q_heads, int batch,
       if (units <= resident) *splits = c;
     }
     if (mode == 0 && (double)steps / *splits - even > 12.0) *sched = kSchedSpans;
-  } else if (mode == 0 && room && l.cuts && most <= 3ll * sms && 0.85 * steps * ceil(rounds) - even > 16.0) {
+  } else if (mode == 0 && room && l.cuts && most <= 4ll * sms && 0.85 * steps * ceil(rounds) - even > (pairs == 1 ? 7.5 : 11.5)) {
     *sched = kSchedSpans;
   }
   return KV_OK;
