@@ -309,7 +309,8 @@ kv_status_t kvattn_set_extend_impl(int impl);
 kv_status_t kvattn_set_shared_impl(int impl);
 /* Selects how the decode kernel brings pages on chip: 1 = straight into registers (one page per warp in flight), 2 =
  * through a per-warp ring of page slots in shared memory filled by bulk copies (several pages per warp in flight);
- * 0 = the default, which is 2.  Same arithmetic, same bits.  Process-wide; for tests and benchmarks. */
+ * 0 = the default, 1 where a warp has a page or two and 2 elsewhere.  Same arithmetic, same bits.  Process-wide; for
+ * tests and benchmarks. */
 kv_status_t kvattn_set_decode_impl(int impl);
 /* Tuning: inside attn_mixed (both sets present) the persistent extend kernel takes n SMs, so that the HBM-bound decode
  * kernel runs beside it on the others instead of after it (an extend set cut into equal spans: as many spans per SM as

@@ -7,7 +7,7 @@
 // What bounds it: full batches, HBM (256 sequences of 1024-4096 tokens, 32/8 heads of 128: 373 us; the kernel it replaced,
 // one warp per 1024-token chunk and a combine kernel behind it, took 418).  Small batches, the latency of a warp's
 // pages (about 0.7 us each, whatever the depth of its ring), so the sequence is spread over as many warps as are
-// resident: one sequence of 517 tokens 32.0 -> 4.3 us, of 16000 tokens 63 -> 15.6, 8 of 1000-4000 tokens 61.7 -> 18.8.
+// resident: one sequence of 517 tokens 32.0 -> 3.9 us, of 16000 tokens 63 -> 15.6, 8 of 1000-4000 tokens 61.7 -> 18.8.
 // kWarps x kStages: six warps with two page slots each, two CTAs per SM (D = 128).  4 x 3, 8 x 3, 12 x 2 and 4 x 6 were
 // measured on 20 batch shapes: twelve warps on an SM beat eight everywhere (a slot is refilled as soon as its page is
 // in registers, so two are enough), and two CTAs of six beat one of twelve on short contexts (128 sequences of 200-700:
@@ -185,21 +185,12 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
           ptx::mbar_wait_limit(bars + (used % kStages) * 8, (used / kStages) & 1, &never, 100000000ull);
       }
     } else {
-      // two register sets alternate: the next page's loads are in flight while this one is consumed
-      auto fetch = [&](PageRegs<D>& pr, int p) {
-        const int pg = page_id(p);
-        load_page<D>(pr, kbase + (size_t)pg * page_stride, vbase + (size_t)pg * page_stride, r, c);
-      };
-      PageRegs<D> ra, rb;
-      if (p_begin < p_end) fetch(ra, p_begin);
-      for (int p = p_begin; p < p_end; p += 2) {
+      for (int p = p_begin; p < p_end; ++p) {
         advance(p);
-        if (p + 1 < p_end) fetch(rb, p + 1);
-        page_step<D>(st, ra, qf, p * kPageSize, limit0, limit1, L, a.scale_log2, r, c);
-        if (p + 1 < p_end) {
-          if (p + 2 < p_end) fetch(ra, p + 2);
-          page_step<D>(st, rb, qf, (p + 1) * kPageSize, limit0, limit1, L, a.scale_log2, r, c);
-        }
+        const int pg = page_id(p);
+        PageRegs<D> pr;
+        load_page<D>(pr, kbase + (size_t)pg * page_stride, vbase + (size_t)pg * page_stride, r, c);
+        page_step<D>(st, pr, qf, p * kPageSize, limit0, limit1, L, a.scale_log2, r, c);
       }
     }
   }
@@ -287,7 +278,7 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
   if (a.wait_mode == kWaitLast && blockIdx.x == gridDim.x - 1) ptx::dependency_wait();
 }
 
-std::atomic<int> g_decode_impl{0};  // 0: default (the ring), 1: pages stream through registers, 2: pages go through a shared-memory ring
+std::atomic<int> g_decode_impl{0};  // 0: by the pages per warp, 1: pages stream through registers, 2: pages go through a shared-memory ring
 
 // Prepares the kernel for a device (once).
 template <int D, bool RING>
@@ -390,6 +381,16 @@ static kv_status_t decode_splits(const kv_pool_t* p, int batch, int max_ctx_len,
   return KV_OK;
 }
 
+// Whether a warp has so few pages that it should load them straight into registers: a copy into a slot, its barrier and the
+// read back cost 0.4 to 0.7 us more than a load, and with a page or two per warp there is nothing to overlap them with.
+// Ring / registers at so many pages per warp: 128 dims 4.7 / 4.2 us (1.0), 5.7 / 5.5 (1.8), 6.0 / 5.3 (1.95), 7.2 / 7.3 (2.1),
+// 7.3 / 8.0 (3.1), with more CTAs than are resident 24.2 / 23.3 (1.0), 17.4 / 17.8 (1.3); 64 dims 4.6 / 4.1 (0.8), 8.1 / 6.9
+// (1.3), 6.5 / 5.9 (2.75), 14.9 / 16.0 (3.7).
+static bool few_pages(const kv_pool_t* p, int64_t blocks, int splits, int max_ctx_len) {
+  const double pages = (double)(max_ctx_len + kPageSize - 1) / kPageSize / (kWarps * splits);
+  return pages <= (p->head_dim == 64 ? 2.75 : blocks <= 2 * sm_count_of(p->device) ? 2.0 : 1.0);
+}
+
 template <int D, bool RING>
 static kv_status_t launch_decode_kernel(const kv_pool_t* p, const DecodeArgs& a, int64_t blocks, cudaStream_t st) {
   const kv_status_t s = decode_setup<D, RING>(p->device);
@@ -437,7 +438,8 @@ kv_status_t launch_decode(kv_pool_t* p, const void* q, int n_q_heads, const int*
   a.lse = lse;
   const int64_t blocks = (int64_t)batch * p->n_kv_heads * a.splits;
   if (blocks > 0x7fffffffLL) return KV_ERR_UNSUPPORTED;
-  const bool ring = g_decode_impl.load() != 1;
+  const int impl = g_decode_impl.load();
+  const bool ring = impl == 0 ? !few_pages(p, blocks, a.splits, max_ctx_len) : impl != 1;
   if (p->head_dim == 128)
     return ring ? launch_decode_kernel<128, true>(p, a, blocks, st) : launch_decode_kernel<128, false>(p, a, blocks, st);
   return ring ? launch_decode_kernel<64, true>(p, a, blocks, st) : launch_decode_kernel<64, false>(p, a, blocks, st);

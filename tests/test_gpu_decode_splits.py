@@ -44,6 +44,27 @@ def test_more_clusters_than_the_device_holds(max_ctx, batch):
     _check(synth.Geometry(32, 8, 128), lens, seed=800)
 
 
+@pytest.mark.parametrize("d,batch,pages", [(128, 1, 192), (128, 1, 193), (64, 1, 264), (64, 1, 265), (128, 320, 6), (128, 320, 7)])
+def test_where_the_default_goes_from_registers_to_the_ring(d, batch, pages):
+    # two (64 dims: 2.75) pages per warp of 16 CTAs; a batch of more CTAs than are resident: one page per warp of one
+    geom = synth.Geometry(8, 1, d)
+    lens = [16 * pages] + [16 * (i % pages) + 1 for i in range(batch - 1)]
+    dp = DualPool(geom, sum(synth.pages_needed(L, 16) for L in lens) + 2, seed=pages)
+    b = Batch(dp, lens)
+    b.write([(i, 0, L) for i, L in enumerate(lens)])
+    outs = []
+    for impl in (0, 1, 2):
+        kvattn.kvattn_set_decode_impl(impl)
+        try:
+            outs.append(run_decode(dp, b, lens, oracle=(impl == 0)))
+        finally:
+            kvattn.kvattn_set_decode_impl(0)
+    assert_close(outs[0], f"decode of {batch} sequences, {pages} pages")
+    for o in outs[1:]:
+        assert np.array_equal(outs[0]["o_bits"], o["o_bits"]) and np.array_equal(outs[0]["lse_raw"], o["lse_raw"])
+    dp.close()
+
+
 def test_back_to_back_calls_that_depend_on_each_other():
     # The kernel is launched early behind whatever runs before it on the stream: an append, another decode, a fill.
     geom = synth.Geometry(8, 2, 128)
