@@ -3,6 +3,7 @@
 // A cluster of `splits` CTAs owns one (sequence, KV head); its splits * kWarps warps take equal runs of the sequence's
 // pages.  Every warp streams its run (page_mma.cuh), the warps of a CTA are merged through shared memory and the CTAs of
 // the cluster through distributed shared memory: one kernel, no partial result in global memory, no combine kernel.
+// Where there are many short sequences instead, a CTA takes several pairs (pairs_per_cta).
 //
 // What bounds it: full batches, HBM (256 sequences of 1024-4096 tokens, 32/8 heads of 128: 373 us; the kernel it replaced,
 // one warp per 1024-token chunk and a combine kernel behind it, took 418).  Small batches, the latency of a warp's
@@ -29,6 +30,8 @@ struct DecodeArgs {
   const int* ctx_lens;
   int n_q_heads, group;
   int splits;        // CTAs of a cluster
+  int units;         // (sequence, KV head) pairs
+  int per_cta;       // pairs a CTA takes, kWarps / per_cta warps each (1 where splits > 1)
   int len_bound;     // host-side bound on ctx_lens, up to a multiple of kDecodeChunkTokens (a longer sequence is reported and skipped)
   int wait_mode;     // kWaitFirst / kWaitLast
   float scale_log2;  // scale * log2(e)
@@ -59,6 +62,7 @@ struct DecodeShared {
   float ml[kWarps][8][2];         // [warp][row]: maximum, sum
   float in_ml[kMaxSplits][8][2];  // [CTA][row]
   int abort_flag;
+  int fits[kWarps];               // [pair of the CTA]: its sequence is as long as the host said or shorter
 };
 
 template <int D, bool RING>
@@ -78,8 +82,12 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int r = lane >> 2, c = lane & 3;
   const int splits = a.splits;
-  const int unit = blockIdx.x / splits, rank = blockIdx.x - unit * splits;
+  const int cluster = blockIdx.x / splits, rank = blockIdx.x - cluster * splits;
   const int Hkv = a.pool.n_kv_heads, G = a.group, Hq = a.n_q_heads;
+  const int team = kWarps / a.per_cta, mine = warp / team;  // warps of a pair; the pair of this warp
+  const int first_unit = cluster * a.per_cta, n_units = min(a.per_cta, a.units - first_unit);
+  const bool idle = mine >= n_units;
+  const int unit = idle ? first_unit : first_unit + mine;
   const int seq = unit / Hkv, kvh = unit - seq * Hkv;
 
   ptx::launch_dependents();
@@ -97,10 +105,11 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
 
   const int L = __ldg(a.ctx_lens + seq);
   const bool fits = L <= a.max_pages * kPageSize && L <= a.len_bound;
-  if (!fits && rank == 0 && tid == 0) report(a.pool.status, KV_ERR_BOUNDS);  // left unwritten
-  const int n_pages = fits && L > 0 ? (L + kPageSize - 1) / kPageSize : 0;
-  const int runs = kWarps * splits;
-  const int run = rank * kWarps + warp;
+  if (!fits && rank == 0 && lane == 0) report(a.pool.status, KV_ERR_BOUNDS);  // left unwritten
+  if (lane == 0 && warp == mine * team) sh.fits[mine] = fits;
+  const int n_pages = fits && L > 0 && !idle ? (L + kPageSize - 1) / kPageSize : 0;
+  const int runs = team * splits;
+  const int run = rank * team + warp - mine * team;
   const int p_begin = (int)((int64_t)n_pages * run / runs), p_end = (int)((int64_t)n_pages * (run + 1) / runs);
 
   // query rows: lane loads row r's chunks; rows past the group are zero
@@ -220,34 +229,38 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
   }
   __syncthreads();
 
-  // ---- merge.  Element i (four dims of a row) = row i / (D/4), dims 4 (i % (D/4)) ..
+  // ---- merge.  Element i (four dims of a row) of a pair = row i / (D/4), dims 4 (i % (D/4)) ..
   constexpr int kVec = D / 4;
   const int n_elem = G * kVec;
-  auto store = [&](int i, float4 o, float m, float l) {
+  auto store = [&](int u, int i, float4 o, float m, float l) {
     const int row = i / kVec, dv = i % kVec;
     const float inv = l > 0.f ? 1.f / l : 0.f;
-    const int64_t orow = (int64_t)seq * Hq + kvh * G + row;
+    const int s_u = u / Hkv, h_u = u - s_u * Hkv;
+    const int64_t orow = (int64_t)s_u * Hq + h_u * G + row;
     *reinterpret_cast<uint2*>(a.out + orow * D + dv * 4) = make_uint2(pack_bf16x2(o.x * inv, o.y * inv), pack_bf16x2(o.z * inv, o.w * inv));
     if (dv == 0) a.lse[orow] = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
   };
   const int slice = (n_elem + splits - 1) / splits;  // elements of the result each CTA finishes (the last ones: what is left)
   if (splits > 1) cluster_wait();                    // the partners run: their shared memory may be written
-  for (int i = tid; i < n_elem; i += kWarps * 32) {
+  for (int e = tid; e < n_units * n_elem; e += kWarps * 32) {
+    const int pair = e / n_elem, i = e - pair * n_elem, w0 = pair * team;
     const int row = i / kVec, dv = i % kVec;
     float m = -INFINITY, l = 0.f;
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) m = fmaxf(m, sh.ml[w][row][0]);
+    for (int w = 0; w < kWarps; ++w)
+      if (w < team) m = fmaxf(m, sh.ml[w0 + w][row][0]);
     const float mu = m == -INFINITY ? 0.f : m;
     float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int w = 0; w < kWarps; ++w) {
-      const float wt = fast_exp2(sh.ml[w][row][0] - mu);
-      l += wt * sh.ml[w][row][1];
-      const float4 x = *reinterpret_cast<const float4*>(part + (w * 8 + row) * SM::kRowFloats + dv * 4);
+      if (w >= team) break;
+      const float wt = fast_exp2(sh.ml[w0 + w][row][0] - mu);
+      l += wt * sh.ml[w0 + w][row][1];
+      const float4 x = *reinterpret_cast<const float4*>(part + ((w0 + w) * 8 + row) * SM::kRowFloats + dv * 4);
       o.x += wt * x.x; o.y += wt * x.y; o.z += wt * x.z; o.w += wt * x.w;
     }
     if (splits == 1) {
-      if (fits) store(i, o, m, l);
+      if (sh.fits[pair]) store(first_unit + pair, i, o, m, l);
     } else {
       const int dest = i / slice, at = i - dest * slice;
       st_cluster(cluster_addr(ptx::smem_u32(in_o + ((rank * slice + at) << 2)), dest), o);
@@ -270,7 +283,7 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
         const float4 x = *reinterpret_cast<const float4*>(in_o + ((s * slice + at) << 2));
         o.x += wt * x.x; o.y += wt * x.y; o.z += wt * x.z; o.w += wt * x.w;
       }
-      if (fits) store(i, o, m, l);
+      if (fits) store(unit, i, o, m, l);
     }
   }
   // Beside another kernel: this grid must not be complete before that one is, or work queued behind this grid with an
@@ -381,13 +394,32 @@ static kv_status_t decode_splits(const kv_pool_t* p, int batch, int max_ctx_len,
   return KV_OK;
 }
 
+// (sequence, KV head) pairs per CTA where no pair is spread over a cluster: many short sequences are bound by the starts,
+// barriers and merges of their CTAs, so a CTA takes as many pairs as bring them all on the device at once, one to three
+// warps for a pair, while a warp's run stays short: 16 pages, 8 where there is a second wave all the same.  Us with 1 / 2 /
+// 3 / 6 pairs (128 dims, 296 CTAs resident): 72 x 8 pairs of up to 6 pages 9.4 / 6.7 / 8.0 / 10.2, 103 x 8 of 7 15.4 / 13.9 /
+// 10.0 / 11.9, 222 x 8 of 8 32.1 / 25.1 / 23.0 / 20.3, 75 x 8 of 32 32.4 / 33.8 / 29.9 / 35.8; second waves: 251 x 8 of 12
+// 44.7 / 36.3 / 35.7 / 39.3, 149 x 8 of 37 60.4 / 62.5 / 60.6 / 63.5; 64 dims (444 resident): 101 x 8 of 18 13.5 / 10.6 / 12.4 /
+// 16.8, 230 x 8 of 48 60.4 / 62.6 / 62.3 / 60.6.
+template <int D>
+static kv_status_t pairs_per_cta(const kv_pool_t* p, int64_t units, int max_ctx_len, int* n) {
+  int resident;
+  const kv_status_t s = resident_clusters<D>(p->device, 0, &resident);
+  if (s != KV_OK) return s;
+  const int pages = (int)(((int64_t)max_ctx_len + kPageSize - 1) / kPageSize);
+  *n = 1;
+  for (int u : {2, 3, 6})
+    if (units > (int64_t)*n * resident && pages * u <= kWarps * (units <= (int64_t)u * resident ? 16 : 8)) *n = u;
+  return KV_OK;
+}
+
 // Whether a warp has so few pages that it should load them straight into registers: a copy into a slot, its barrier and the
 // read back cost 0.4 to 0.7 us more than a load, and with a page or two per warp there is nothing to overlap them with.
 // Ring / registers at so many pages per warp: 128 dims 4.7 / 4.2 us (1.0), 5.7 / 5.5 (1.8), 6.0 / 5.3 (1.95), 7.2 / 7.3 (2.1),
 // 7.3 / 8.0 (3.1), with more CTAs than are resident 24.2 / 23.3 (1.0), 17.4 / 17.8 (1.3); 64 dims 4.6 / 4.1 (0.8), 8.1 / 6.9
 // (1.3), 6.5 / 5.9 (2.75), 14.9 / 16.0 (3.7).
-static bool few_pages(const kv_pool_t* p, int64_t blocks, int splits, int max_ctx_len) {
-  const double pages = (double)(max_ctx_len + kPageSize - 1) / kPageSize / (kWarps * splits);
+static bool few_pages(const kv_pool_t* p, int64_t blocks, int warps, int max_ctx_len) {
+  const double pages = (double)(max_ctx_len + kPageSize - 1) / kPageSize / warps;
   return pages <= (p->head_dim == 64 ? 2.75 : blocks <= 2 * sm_count_of(p->device) ? 2.0 : 1.0);
 }
 
@@ -436,10 +468,18 @@ kv_status_t launch_decode(kv_pool_t* p, const void* q, int n_q_heads, const int*
   a.scale_log2 = scale * 1.4426950408889634f;
   a.out = (__nv_bfloat16*)out;
   a.lse = lse;
-  const int64_t blocks = (int64_t)batch * p->n_kv_heads * a.splits;
-  if (blocks > 0x7fffffffLL) return KV_ERR_UNSUPPORTED;
+  const int64_t units = (int64_t)batch * p->n_kv_heads;
+  if (units * a.splits > 0x7fffffffLL) return KV_ERR_UNSUPPORTED;
+  a.units = (int)units;
+  a.per_cta = 1;
+  if (a.splits == 1) {
+    const kv_status_t us = p->head_dim == 128 ? pairs_per_cta<128>(p, units, max_ctx_len, &a.per_cta)
+                                              : pairs_per_cta<64>(p, units, max_ctx_len, &a.per_cta);
+    if (us != KV_OK) return us;
+  }
+  const int64_t blocks = (units + a.per_cta - 1) / a.per_cta * a.splits;
   const int impl = g_decode_impl.load();
-  const bool ring = impl == 0 ? !few_pages(p, blocks, a.splits, max_ctx_len) : impl != 1;
+  const bool ring = impl == 0 ? !few_pages(p, blocks, kWarps / a.per_cta * a.splits, max_ctx_len) : impl != 1;
   if (p->head_dim == 128)
     return ring ? launch_decode_kernel<128, true>(p, a, blocks, st) : launch_decode_kernel<128, false>(p, a, blocks, st);
   return ring ? launch_decode_kernel<64, true>(p, a, blocks, st) : launch_decode_kernel<64, false>(p, a, blocks, st);

@@ -65,6 +65,14 @@ def test_where_the_default_goes_from_registers_to_the_ring(d, batch, pages):
     dp.close()
 
 
+@pytest.mark.parametrize("hq,hkv,d,batch", [(4, 1, 128, 297), (32, 8, 128, 75), (8, 8, 128, 113), (8, 4, 64, 333), (2, 1, 64, 2000)])
+def test_ctas_with_several_short_sequences(hq, hkv, d, batch):
+    # two, three and six (sequence, KV head) pairs per CTA, the last CTA not full, runs from none to several pages
+    rng = np.random.default_rng(batch)
+    lens = [0, 1, 16, 17, 80] + [int(x) for x in rng.integers(1, 80, size=batch - 5)]
+    _check(synth.Geometry(hq, hkv, d), lens, seed=batch)
+
+
 def test_back_to_back_calls_that_depend_on_each_other():
     # The kernel is launched early behind whatever runs before it on the stream: an append, another decode, a fill.
     geom = synth.Geometry(8, 2, 128)
