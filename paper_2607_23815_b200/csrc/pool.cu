@@ -17,7 +17,9 @@ std::atomic<int64_t> g_launches{0};
 // ------------------------------------------------------------------------------------------
 // kMaxPerLane: 16-byte chunks of K (and of V) of a token per lane and pass; no more than a token has, because the registers
 // they take decide how many tokens are on an SM at a time (10207 tokens of 8 heads x 128: 20.2 us with 8, of which a token
-// uses 4, 17.3 with 4; 64 dims, 2 per lane: 16.4 and 11.0).
+// uses 4, 17.3 with 4; 64 dims, 2 per lane: 16.4 and 11.0).  Rows of several hundred MB are the exception: with twice the
+// tokens in flight the reads and writes get in each other's way in DRAM (8 heads x 128: 20000 tokens 28.9 with 8 and 27.0
+// with 4, 80000 106.6 and 107.5, 160000 208.8 and 217.7, 640000 829 and 893; at 64 dims 2 per lane stay ahead, 519 and 442).
 template <int kMaxPerLane>
 __global__ void __launch_bounds__(256, kMaxPerLane == 8 ? 2 : 4) append_kernel(PoolView pool, AppendArgs a) {
   ptx::launch_dependents();
@@ -391,7 +393,9 @@ kv_status_t kv_append(kv_pool_t* p, const void* k_new, const void* v_new, const 
                      total_new};
   const unsigned blocks = (unsigned)grid_for(p, (int64_t)total_new * 32, 256);  // one warp per token
   const int chunks = p->n_kv_heads * (p->head_dim >> 3);
-  const auto kernel = chunks <= 64 ? append_kernel<2> : chunks <= 128 ? append_kernel<4> : append_kernel<8>;
+  // (rows of many times the L2: fewer tokens on an SM at a time, see append_kernel)
+  const bool bulk = (int64_t)total_new * chunks * 32 >= 320000000;
+  const auto kernel = chunks <= 64 ? append_kernel<2> : chunks <= 128 && !bulk ? append_kernel<4> : append_kernel<8>;
   KV_CUDA_OK(launch_early(kernel, blocks, 256, (cudaStream_t)stream, p->view(), a));
   count_launch();
   return KV_OK;
