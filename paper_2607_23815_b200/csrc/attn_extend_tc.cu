@@ -57,7 +57,7 @@ constexpr float kOptimisticSum = 65536.0f;  // a row sum of one tile beyond this
 struct SpanArgs {
   int n_spans, per_cta;  // spans at most; neighbouring spans one CTA takes
   int max_tp, total_q;   // host-side bounds: tile pairs of a sequence, rows of Q
-  int plan_early;        // the kernel in front is this call's own append: the lengths may be read before waiting for it
+  int plan_early;        // the kernel in front is this call's own append: lengths, tables and Q may be read before it is done
   int4* desc;            // [n_spans][3]: the cut at the start of a span: (first step of the item it goes through among all
                          // steps, or -1; step of the item; KV head; tile pair), (rows, first row, KV steps of the two tiles)
   int rows;              // rows a slot of partial results holds (no item of the batch has more)
@@ -702,8 +702,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
   const uint32_t tmem = sm.tmem_base;
   // Everything up to here touched only this CTA's own shared and tensor memory and may have run while the kernel in
   // front of this one (the plan, or the plan and the suffix append) was still at work; its results are needed now.
-  // (the scheduler warp reads the lengths first where it may)
-  if (!REC || warp != kWarpSched || !a.span.plan_early) dependency_wait();
+  // (Behind this call's own append, which has waited for all that came before it: lengths, tables and Q may be read at
+  // once, so the scheduler, the Q loader and the producer do not wait here; the producer does before its first K/V copy.)
+  const bool reads_early = REC && a.span.plan_early;
+  if (!reads_early || (warp != kWarpSched && warp != kWarpQ && warp != kWarpProducer)) dependency_wait();
   const int n_total = REC ? 0 : __ldcg(a.n_items) * a.pool.n_kv_heads;
   const int Hkv = a.pool.n_kv_heads;
   // Round r of this CTA works on item sched_get(r) of the global list (>= n_total: no more work).  A warp
@@ -741,7 +743,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
     const char* kpool = reinterpret_cast<const char*>(a.pool.k);
     const char* vpool = reinterpret_cast<const char*>(a.pool.v);
     uint32_t loads = 0;  // stage loads issued so far (ring position)
-    bool ok = true;
+    bool ok = true, wait_first = reads_early;
     // Announces item idx as round r (waits until every reader is done with the slot's previous round).
     auto announce = [&](int r, int idx) {
       if (lane == 0) {
@@ -796,6 +798,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
           }
         }
         const size_t src_off = ((size_t)page * Hkv) * Cfg::kBlockBytes + head_off;
+        if (REC && wait_first) {
+          dependency_wait();
+          wait_first = false;
+        }
 #pragma unroll
         for (int which = 0; which < 2; ++which) {  // 0: K tile, 1: V tile
           const uint32_t s = loads % Cfg::kStages, par = (loads / Cfg::kStages) & 1;
@@ -992,7 +998,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
       const int rest = unit / Hkv, kvh = unit - rest * Hkv, seq = rest / a.span.max_tp, tp = rest - seq * a.span.max_tp;
       const int P = cl_P, E = cl_E, row0 = cl_row0;
       const int rows = span_rows(a, P, E, row0), pairs = span_pairs(rows, lg);
-      if (a.span.plan_early) dependency_wait();
       if (lane == 0) {
         if (tp == 0 && kvh == 0 && rank == 0 && P >= 0 && rows < E) report(a.pool.status, KV_ERR_BOUNDS);
         int n = 0, n0 = 0, n1 = 0, kv_end = 0, first_child = 0;
@@ -1030,7 +1035,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
       SpanSeqs q;
       span_locate(a, span, pos, total, q);
       const int n_spans = span_count(a.span, total);
-      if (a.span.plan_early) dependency_wait();
       const int span_end = min(span + a.span.per_cta, n_spans);
       bool ok = true;
       auto announce = [&](const SpanRec& r) {
