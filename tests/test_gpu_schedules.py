@@ -78,3 +78,54 @@ def test_spans_cut_long_items(batch, long, hq, hkv, d):
     E = [int(x) for x in rng.integers(0, 60, size=batch)]
     P[0], E[0], P[batch // 2], E[batch // 2], P[-1], E[-1] = long - 50, 50, long - 61, 61, long // 2, 64
     _check(synth.Geometry(hq, hkv, d), P, E, 960 + batch, f"spans {batch}")
+
+
+@pytest.mark.parametrize("long,batch", [(1500, 3), (3000, 40)])
+def test_append_and_extend_right_behind_what_writes_their_inputs(long, batch):
+    # clusters and spans read lengths, tables and Q while the call's own append runs: everything queued before that is final.
+    # Each step's query, keys, lengths and table come from the kernels just in front of it; with and without waiting between.
+    hq, hkv, d, e, steps = 8, 2, 128, 24, 4
+    rng = np.random.default_rng(batch)
+    P = [long] + [int(x) for x in rng.integers(0, 200, size=batch - 1)]
+    need = [-(-(p + e * steps) // 16) for p in P]
+    width, total = max(need), sum(need)
+    table = np.full((batch, width), -1, dtype=np.int32)
+    ids = rng.permutation(total).astype(np.int32)
+    for i, k in enumerate(need):
+        table[i, :k], ids = ids[:k], ids[k:]
+    pages = [torch.zeros((total, hkv, 16, d), dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    pool = kvattn.kv_pool_create_ex(total, 16, hkv, d, *pages)
+    ids_all = kvattn.kv_alloc(pool, total)
+    assert sorted(ids_all) == list(range(total))
+    gen = torch.Generator(device="cuda").manual_seed(batch)
+    randn = lambda *s: torch.randn(s, generator=gen, device="cuda", dtype=torch.bfloat16)
+    k0, v0, q0 = randn(sum(P), hkv, d), randn(sum(P), hkv, d), randn(batch * e, hq, d)
+    cu_p, cu = _i32(np.concatenate([[0], np.cumsum(P)])), _i32(np.arange(batch + 1) * e)
+    bt_all, el, scale, ml = _i32(table), _i32([e] * batch), float(np.float32(d ** -0.5)), max(P) + e * steps
+    ws = torch.empty(kvattn.attn_workspace_bytes(pool, hq, batch, batch * e, ml, 0, 0), dtype=torch.uint8, device="cuda")
+    runs = []
+    for wait in (True, False, False):
+        for t in pages:
+            t.zero_()
+        kvattn.kv_append(pool, k0, v0, cu_p, _i32([0] * batch), None, bt_all)
+        q, pl, bt, outs = q0.clone(), _i32(P), torch.full_like(bt_all, -1), []
+        out, lse = torch.empty_like(q), torch.empty((batch * e, hq), device="cuda")
+        for _ in range(steps):
+            bt.copy_(bt_all)                       # (the table of the step is written in front of the call)
+            kn, vn = q[:, :hkv].contiguous(), q[:, hkv:2 * hkv].contiguous()
+            if wait:
+                torch.cuda.synchronize()
+            kvattn.attn_extend_append(pool, q, kn, vn, cu, bt, pl, el, e, ml, scale, out, lse, ws)
+            if wait:
+                torch.cuda.synchronize()
+            outs.append((out.clone(), lse.clone()))
+            pl += el
+            q = (out * 4).contiguous()
+            bt.fill_(-1)
+        torch.cuda.synchronize()
+        runs.append(outs)
+    assert kvattn.kv_last_async_status(pool) == kvattn.KV_OK
+    for other in runs[1:]:
+        for (o1, l1), (o2, l2) in zip(runs[0], other):
+            assert torch.equal(o1.view(torch.int16), o2.view(torch.int16)) and torch.equal(l1, l2)
+    kvattn.kv_pool_destroy(pool)
