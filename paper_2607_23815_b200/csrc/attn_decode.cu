@@ -8,7 +8,7 @@
 // What bounds it: full batches, HBM (256 sequences of 1024-4096 tokens, 32/8 heads of 128: 373 us; the kernel it replaced,
 // one warp per 1024-token chunk and a combine kernel behind it, took 418).  Small batches, the latency of a warp's
 // pages (about 0.7 us each, whatever the depth of its ring), so the sequence is spread over as many warps as are
-// resident: one sequence of 517 tokens 32.0 -> 3.9 us, of 16000 tokens 63 -> 15.6, 8 of 1000-4000 tokens 61.7 -> 18.8.
+// resident: one sequence of 517 tokens 32.0 -> 3.8 us, of 16000 tokens 63 -> 15.6, 8 of 1000-4000 tokens 61.7 -> 18.8.
 // kWarps x kStages: six warps with two page slots each, two CTAs per SM (D = 128).  4 x 3, 8 x 3, 12 x 2 and 4 x 6 were
 // measured on 20 batch shapes: twelve warps on an SM beat eight everywhere (a slot is refilled as soon as its page is
 // in registers, so two are enough), and two CTAs of six beat one of twelve on short contexts (128 sequences of 200-700:
@@ -70,7 +70,9 @@ constexpr int decode_smem_bytes() {
   return (RING ? DecodeSmem<D>::kRing : DecodeSmem<D>::kPart) + DecodeSmem<D>::kIn + (int)sizeof(DecodeShared);
 }
 
-template <int D, bool RING>
+// MULTI: several pairs per CTA (a.per_cta > 1).  An instantiation of its own: with the pair as a run-time value everywhere the
+// others lost 0.3 us (13 sequences of 200-3000 tokens, 64 dims, 13.2 -> 13.5; one of 517 4.25 -> 4.5).
+template <int D, bool RING, bool MULTI>
 __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeArgs a) {
   using SM = DecodeSmem<D>;
   constexpr int NJ = D / 32, NU = D / 64;
@@ -84,9 +86,9 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
   const int splits = a.splits;
   const int cluster = blockIdx.x / splits, rank = blockIdx.x - cluster * splits;
   const int Hkv = a.pool.n_kv_heads, G = a.group, Hq = a.n_q_heads;
-  const int team = kWarps / a.per_cta, mine = warp / team;  // warps of a pair; the pair of this warp
-  const int first_unit = cluster * a.per_cta, n_units = min(a.per_cta, a.units - first_unit);
-  const bool idle = mine >= n_units;
+  const int team = MULTI ? kWarps / a.per_cta : kWarps, mine = MULTI ? warp / team : 0;  // warps of a pair; the pair of this warp
+  const int first_unit = MULTI ? cluster * a.per_cta : cluster, n_units = MULTI ? min(a.per_cta, a.units - first_unit) : 1;
+  const bool idle = MULTI && mine >= n_units;
   const int unit = idle ? first_unit : first_unit + mine;
   const int seq = unit / Hkv, kvh = unit - seq * Hkv;
 
@@ -106,7 +108,7 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
   const int L = __ldg(a.ctx_lens + seq);
   const bool fits = L <= a.max_pages * kPageSize && L <= a.len_bound;
   if (!fits && rank == 0 && lane == 0) report(a.pool.status, KV_ERR_BOUNDS);  // left unwritten
-  if (lane == 0 && warp == mine * team) sh.fits[mine] = fits;
+  if (MULTI && lane == 0 && warp == mine * team) sh.fits[mine] = fits;
   const int n_pages = fits && L > 0 && !idle ? (L + kPageSize - 1) / kPageSize : 0;
   const int runs = team * splits;
   const int run = rank * team + warp - mine * team;
@@ -235,7 +237,7 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
   auto store = [&](int u, int i, float4 o, float m, float l) {
     const int row = i / kVec, dv = i % kVec;
     const float inv = l > 0.f ? 1.f / l : 0.f;
-    const int s_u = u / Hkv, h_u = u - s_u * Hkv;
+    const int s_u = MULTI ? u / Hkv : seq, h_u = MULTI ? u - s_u * Hkv : kvh;
     const int64_t orow = (int64_t)s_u * Hq + h_u * G + row;
     *reinterpret_cast<uint2*>(a.out + orow * D + dv * 4) = make_uint2(pack_bf16x2(o.x * inv, o.y * inv), pack_bf16x2(o.z * inv, o.w * inv));
     if (dv == 0) a.lse[orow] = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
@@ -243,7 +245,7 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
   const int slice = (n_elem + splits - 1) / splits;  // elements of the result each CTA finishes (the last ones: what is left)
   if (splits > 1) cluster_wait();                    // the partners run: their shared memory may be written
   for (int e = tid; e < n_units * n_elem; e += kWarps * 32) {
-    const int pair = e / n_elem, i = e - pair * n_elem, w0 = pair * team;
+    const int pair = MULTI ? e / n_elem : 0, i = e - pair * n_elem, w0 = pair * team;
     const int row = i / kVec, dv = i % kVec;
     float m = -INFINITY, l = 0.f;
 #pragma unroll
@@ -260,7 +262,7 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
       o.x += wt * x.x; o.y += wt * x.y; o.z += wt * x.z; o.w += wt * x.w;
     }
     if (splits == 1) {
-      if (sh.fits[pair]) store(first_unit + pair, i, o, m, l);
+      if (MULTI ? sh.fits[pair] != 0 : fits) store(first_unit + pair, i, o, m, l);
     } else {
       const int dest = i / slice, at = i - dest * slice;
       st_cluster(cluster_addr(ptx::smem_u32(in_o + ((rank * slice + at) << 2)), dest), o);
@@ -294,14 +296,14 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
 std::atomic<int> g_decode_impl{0};  // 0: by the pages per warp, 1: pages stream through registers, 2: pages go through a shared-memory ring
 
 // Prepares the kernel for a device (once).
-template <int D, bool RING>
+template <int D, bool RING, bool MULTI>
 static kv_status_t decode_setup(int device) {
   static std::atomic<bool> configured[kMaxDevices];
   if (device < 0 || device >= kMaxDevices) return KV_ERR_INVALID;
   if (!configured[device].load(std::memory_order_acquire)) {
-    KV_CUDA_OK(cudaFuncSetAttribute(attn_decode_kernel<D, RING>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    KV_CUDA_OK(cudaFuncSetAttribute(attn_decode_kernel<D, RING, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     decode_smem_bytes<D, RING>()));
-    KV_CUDA_OK(cudaFuncSetAttribute(attn_decode_kernel<D, RING>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    KV_CUDA_OK(cudaFuncSetAttribute(attn_decode_kernel<D, RING, MULTI>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     configured[device].store(true, std::memory_order_release);
   }
   return KV_OK;
@@ -330,7 +332,7 @@ static constexpr int kSplitChoices[] = {1, 2, 3, 4, 6, 8, 16};
 template <int D>
 static kv_status_t resident_clusters(int device, int i, int* n) {
   static std::atomic<int> cached[kMaxDevices][sizeof(kSplitChoices) / sizeof(int)];  // value + 1
-  const kv_status_t s = decode_setup<D, true>(device);
+  const kv_status_t s = decode_setup<D, true, false>(device);
   if (s != KV_OK) return s;
   int v = cached[device][i].load(std::memory_order_relaxed);
   if (v == 0) {
@@ -340,7 +342,7 @@ static kv_status_t resident_clusters(int device, int i, int* n) {
     cfg.attrs = attr + 1;
     cfg.numAttrs = 1;
     int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, attn_decode_kernel<D, true>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&clusters, attn_decode_kernel<D, true, false>, &cfg) != cudaSuccess) {
       cudaGetLastError();
       clusters = 0;
     }
@@ -423,16 +425,20 @@ static bool few_pages(const kv_pool_t* p, int64_t blocks, int warps, int max_ctx
   return pages <= (p->head_dim == 64 ? 2.75 : blocks <= 2 * sm_count_of(p->device) ? 2.0 : 1.0);
 }
 
-template <int D, bool RING>
-static kv_status_t launch_decode_kernel(const kv_pool_t* p, const DecodeArgs& a, int64_t blocks, cudaStream_t st) {
-  const kv_status_t s = decode_setup<D, RING>(p->device);
+template <int D, bool RING, bool MULTI>
+static kv_status_t launch_decode_variant(const kv_pool_t* p, const DecodeArgs& a, int64_t blocks, cudaStream_t st) {
+  const kv_status_t s = decode_setup<D, RING, MULTI>(p->device);
   if (s != KV_OK) return s;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
   decode_config(cfg, attr, a.splits, blocks, decode_smem_bytes<D, RING>(), st);
-  KV_CUDA_OK(cudaLaunchKernelEx(&cfg, attn_decode_kernel<D, RING>, a));
+  KV_CUDA_OK(cudaLaunchKernelEx(&cfg, attn_decode_kernel<D, RING, MULTI>, a));
   count_launch();
   return KV_OK;
+}
+template <int D, bool RING>
+static kv_status_t launch_decode_kernel(const kv_pool_t* p, const DecodeArgs& a, int64_t blocks, cudaStream_t st) {
+  return a.per_cta > 1 ? launch_decode_variant<D, RING, true>(p, a, blocks, st) : launch_decode_variant<D, RING, false>(p, a, blocks, st);
 }
 
 // What the entry points ask their callers for.  The kernel keeps its partial results on chip and uses none of it; the
