@@ -73,7 +73,7 @@ constexpr int kSpanSnap = 1;      // a cut this close to the edge of an item mov
 //  kSchedList: the plan's list, through a work counter (any number of items).
 //  kSchedSpans: equal spans of KV steps (see SpanArgs).
 //  kSchedCluster: one item per cluster of cl_splits CTAs, each with an equal part of its KV steps; their results are merged
-//  through distributed shared memory.  For batches whose items, that many CTAs each, are on the device at once.
+//  through L2 behind a cluster barrier.  For batches whose items, that many CTAs each, are on the device at once.
 constexpr int kSchedList = 0, kSchedSpans = 1, kSchedCluster = 2;
 constexpr int kMaxClusterSplits = 8;
 
@@ -1746,7 +1746,7 @@ static kv_status_t resident_clusters(int device, int c, int* n) {
 // Who takes which items, from the host-side bounds (and the workspace) alone; splits: CTAs per item for kSchedCluster.
 //  - Items that are on the device at once go to a cluster each, as large as fits, one KV step per CTA at least: no plan
 //    kernel, and the steps of an item run side by side.  Suffix append + extend of 1 / 4 / 8 / 16 sequences of 30-60 tokens
-//    behind 1000-2000 (32/8 heads of 128): 32.1 / 38.2 / 42.2 / 43.7 us through the list, 16.8 / 24.2 / 33.3 / 42.4 this
+//    behind 1000-2000 (32/8 heads of 128): 32.1 / 38.2 / 42.2 / 43.7 us through the list, 15.7 / 24.4 / 31.8 / 41.0 this
 //    way with 6 / 4 / 2 / 1 CTAs per item.
 //  - Items that leave SMs idle: spans.  They cost a merge kernel behind the attention kernel and the partial results, 5 to
 //    8 steps, and win what the other two leave idle, the SMs without a cluster or the last round of items.  8 / 16 sequences
