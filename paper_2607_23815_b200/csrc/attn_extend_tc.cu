@@ -1398,12 +1398,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
       }
-      // (a row may see no key of its chunk of a cut item: weight 0)
-      sm.inv_l[t][items_done & 1][m] = SPAN && !(l_run > 0.f) ? 0.f : 1.f / l_run;
+      // (A row may see no key of its chunk of a cut item: its sum is exactly 0 and the chunk has weight 0.  A sum that is not a
+      // number must reach the result: dropping the chunk would hide a broken key behind plausible values of the others.)
+      const bool unseen = SPAN && part >= 0 && l_run == 0.f;
+      sm.inv_l[t][items_done & 1][m] = unseen ? 0.f : 1.f / l_run;
       mbar_arrive(bar_l_full);
       ++items_done;
       if (SPAN && part >= 0) {
-        if (valid) a.span.part_lse[part * a.span.rows + t * 128 + m] = l_run > 0.f ? m_run + log2f(l_run) : -INFINITY;
+        if (valid) a.span.part_lse[part * a.span.rows + t * 128 + m] = unseen ? -INFINITY : m_run + log2f(l_run);
       } else if (valid) {
         a.lse[orow_idx] = (m_run + log2f(l_run)) * 0.6931471805599453f;
       }
@@ -1416,7 +1418,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
       const int splits = a.cl_splits, unit = (int)blockIdx.x / splits, rank = (int)blockIdx.x - unit * splits;
       const int4 u = sm.cl_unit;
       const int row = t * 128 + m;
-      if (__any_sync(0xffffffffu, cl_l > 0.f)) {
+      if (__any_sync(0xffffffffu, cl_l != 0.f)) {  // (a sum that is not a number is handed over like any other)
         tc_fence_after_sync();
         float* dst = a.span.part_o + ((int64_t)blockIdx.x * (D / 8) * a.span.rows + row) * 8;
 #pragma unroll 1
@@ -1467,7 +1469,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
             for (int e = 0; e < 4; ++e) o[e] = make_float2(0.f, 0.f);
 #pragma unroll
             for (int c = 0; c < N; ++c) {
-              if (!(ml[k][c].y > 0.f)) continue;  // (no step of the row's tile, or no key that the row sees: not written)
+              if (ml[k][c].y == 0.f) continue;  // (no step of the row's tile, or no key that the row sees: not written)
               const float w = exp2f(ml[k][c].x - mx);
               sum += w * ml[k][c].y;
 #pragma unroll

@@ -194,3 +194,15 @@ def assert_close(res, what=""):
     assert d_l <= LSE_TOL, f"{what}: max|dLSE| = {d_l:.3e} > {LSE_TOL}"
     assert t <= 1.0, f"{what}: element-wise gate exceeded by {t:.2f}x (max|dO| {d_o:.3e})"
     return d_o, d_l, t
+
+
+def extend_schedule(pool, hq, q, cu, bt, pl, el, max_e, max_l, scale, ws):
+    """Which of the extend kernel's three schedules serves this call, by the kernels that planning and the planned call
+    launch: the list has a plan kernel, spans have a merge kernel behind the attention kernel, clusters have neither."""
+    out, lse = torch.empty_like(q), torch.empty((q.shape[0], hq), dtype=torch.float32, device=q.device)
+    n0 = kvattn.kvattn_launch_count()
+    kvattn.attn_extend_plan(pool, hq, cu, bt, pl, el, int(q.shape[0]), max_e, max_l, ws)
+    n1 = kvattn.kvattn_launch_count()
+    kvattn.attn_extend_planned(pool, q, cu, bt, pl, el, max_e, max_l, scale, out, lse, ws)
+    n2 = kvattn.kvattn_launch_count()
+    return {(1, 1): "list", (0, 1): "clusters", (0, 2): "spans"}[(n1 - n0, n2 - n1)]
