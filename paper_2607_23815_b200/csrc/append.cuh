@@ -3,6 +3,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "sm100_ptx.cuh"
 
 namespace kvattn {
 
@@ -44,8 +45,8 @@ __device__ __forceinline__ void append_tokens(const PoolView& pool, const Append
     for (int i = 0; i < kMaxPerLane; ++i) {
       const int c = i * 32 + lane;
       if (c < chunks_per_token) {
-        kk[i] = __ldg(ksrc + c);
-        vv[i] = __ldg(vsrc + c);
+        kk[i] = ptx::ld_plain(ksrc + c);
+        vv[i] = ptx::ld_plain(vsrc + c);
       }
     }
     // segment of this token: last s with cu_new[s] <= token.  The lanes probe 32 evenly spaced entries at a time, so
@@ -55,20 +56,20 @@ __device__ __forceinline__ void append_tokens(const PoolView& pool, const Append
     while (span > 1) {
       const int step = (span + 31) >> 5;
       const int idx = lo + lane * step;
-      const bool le = idx < lo + span && __ldg(cu_new + idx) <= token;
+      const bool le = idx < lo + span && ptx::ld_plain(cu_new + idx) <= token;
       const int k = __popc(__ballot_sync(0xffffffffu, le)) - 1;   // >= 0: cu_new[lo] <= token
       const int end = lo + span;
       lo += max(k, 0) * step;
       span = min(step, end - lo);
     }
     const int seg = lo;
-    const int seg_begin = __ldg(cu_new + seg), seg_end = __ldg(cu_new + seg + 1);
+    const int seg_begin = ptx::ld_plain(cu_new + seg), seg_end = ptx::ld_plain(cu_new + seg + 1);
     if (token >= seg_end) continue;                            // cu_new not covering this row: skip
-    const int pos = __ldg(start_pos + seg) + (token - seg_begin);
-    const int row = seg_row ? __ldg(seg_row + seg) : seg;
+    const int pos = ptx::ld_plain(start_pos + seg) + (token - seg_begin);
+    const int row = seg_row ? ptx::ld_plain(seg_row + seg) : seg;
     const int blk_idx = pos >> 4;
     if (pos < 0 || blk_idx >= max_pages) { report(pool.status, KV_ERR_BOUNDS); continue; }
-    const int page = __ldg(block_tables + (int64_t)row * max_pages + blk_idx);
+    const int page = ptx::ld_plain(block_tables + (int64_t)row * max_pages + blk_idx);
     if (page < 0 || page >= pool.num_pages) { report(pool.status, KV_ERR_BOUNDS); continue; }
     const size_t page_off = (size_t)page * pool.n_kv_heads * blk;
     const bool last = token + 1 == seg_end;
@@ -78,8 +79,8 @@ __device__ __forceinline__ void append_tokens(const PoolView& pool, const Append
         for (int i = 0; i < kMaxPerLane; ++i) {
           const int c = c0 + i * 32 + lane;
           if (c < chunks_per_token) {
-            kk[i] = __ldg(ksrc + c);
-            vv[i] = __ldg(vsrc + c);
+            kk[i] = ptx::ld_plain(ksrc + c);
+            vv[i] = ptx::ld_plain(vsrc + c);
           }
         }
       }

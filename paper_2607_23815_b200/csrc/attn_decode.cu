@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
   if (splits > 1) cluster_arrive();
   if (a.wait_mode == kWaitFirst) ptx::dependency_wait();
 
-  const int L = __ldg(a.ctx_lens + seq);
+  const int L = ptx::ld_plain(a.ctx_lens + seq);
   const bool fits = L <= a.max_pages * kPageSize && L <= a.len_bound;
   if (!fits && rank == 0 && lane == 0) report(a.pool.status, KV_ERR_BOUNDS);  // left unwritten
   if (MULTI && lane == 0 && warp == mine * team) sh.fits[mine] = fits;
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
     const __nv_bfloat16* qp = a.q + ((int64_t)seq * Hq + kvh * G + r) * D;
 #pragma unroll
     for (int j = 0; j < NJ; ++j)
-      qf[j] = r < G ? __ldg(reinterpret_cast<const uint4*>(qp) + 4 * j + c) : make_uint4(0, 0, 0, 0);
+      qf[j] = r < G ? ptx::ld_plain(reinterpret_cast<const uint4*>(qp) + 4 * j + c) : make_uint4(0, 0, 0, 0);
   }
   const int limit0 = 2 * c < G ? L : 0, limit1 = 2 * c + 1 < G ? L : 0;
 
@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
     auto table_entry = [&](int p) {
       int pg = 0;
       if (p < p_end) {
-        pg = __ldg(bt_row + p);
+        pg = ptx::ld_plain(bt_row + p);
         if ((unsigned)pg >= (unsigned)a.pool.num_pages) {
           report(a.pool.status, KV_ERR_BOUNDS);
           pg = 0;  // stay inside the pool; the result of this row is flagged, not trusted

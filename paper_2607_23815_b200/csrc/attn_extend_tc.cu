@@ -136,12 +136,12 @@ __device__ __forceinline__ ItemRec make_item(int seq, int tp, int P, int E, int 
   if (mode == 2 && tok_hi_t[0] >= 0) {
     // children with a row in this item: the first one whose last token lies at or after the item's first token,
     // then on until a child starts after the item's last token
-    const int c0 = __ldg(fan.cu_children + seq), c1 = __ldg(fan.cu_children + seq + 1);
+    const int c0 = ptx::ld_plain(fan.cu_children + seq), c1 = ptx::ld_plain(fan.cu_children + seq + 1);
     const int tok_lo = (tp * 256) >> lg;
     int lo = c0, hi = c1;
     while (lo < hi) {
       const int mid = (lo + hi) >> 1;
-      if (__ldg(fan.cu_q + mid + 1) - row0 > tok_lo) hi = mid; else lo = mid + 1;
+      if (ptx::ld_plain(fan.cu_q + mid + 1) - row0 > tok_lo) hi = mid; else lo = mid + 1;
     }
     const int c_first = lo;
     const int tok_hi_item = max(tok_hi_t[0], tok_hi_t[1]);
@@ -151,7 +151,7 @@ __device__ __forceinline__ ItemRec make_item(int seq, int tp, int P, int E, int 
     int pages0 = 0, pages = 0;  // of the children, for the first tile's rows and for both tiles'
     bool fits = P <= max_pages * kPageSize;
     for (int c = c_first; c < c1; ++c) {
-      const int start = __ldg(fan.cu_q + c) - row0, len = __ldg(fan.cu_q + c + 1) - __ldg(fan.cu_q + c);
+      const int start = ptx::ld_plain(fan.cu_q + c) - row0, len = ptx::ld_plain(fan.cu_q + c + 1) - ptx::ld_plain(fan.cu_q + c);
       if (start > tok_hi_item) break;
       if (len > fan.max_pages * kPageSize) fits = false;
       if (start <= tok_hi_t[0]) pages0 = pages + ((min(len, tok_hi_t[0] - start + 1) + 15) >> 4);
@@ -201,13 +201,13 @@ __device__ __forceinline__ void plan_body(const PlanArgs& pa) {
   __syncthreads();
   const int64_t n = (int64_t)batch * max_tp;
   // Fan-out mode: a sequence is a parent, its rows are those of its children, which follow one another in Q.
-  auto row_of = [&](int seq) { return mode == 2 ? __ldg(cu_q + __ldg(fan.cu_children + seq)) : __ldg(cu_q + seq); };
-  auto rows_of = [&](int seq) { return mode == 2 ? row_of(seq + 1) - row_of(seq) : __ldg(extend_lens + seq); };
+  auto row_of = [&](int seq) { return mode == 2 ? ptx::ld_plain(cu_q + ptx::ld_plain(fan.cu_children + seq)) : ptx::ld_plain(cu_q + seq); };
+  auto rows_of = [&](int seq) { return mode == 2 ? row_of(seq + 1) - row_of(seq) : ptx::ld_plain(extend_lens + seq); };
   // A sequence with more suffix tokens than the host-side bound the grid was sized with would lose its last rows
   // without a trace: it is reported instead.
   for (int seq = threadIdx.x; seq < batch; seq += blockDim.x) {
     const int E = rows_of(seq);
-    if (__ldg(prefix_lens + seq) >= 0 && (int64_t)E > (((int64_t)max_tp * 256) >> lg)) report(status, KV_ERR_BOUNDS);
+    if (ptx::ld_plain(prefix_lens + seq) >= 0 && (int64_t)E > (((int64_t)max_tp * 256) >> lg)) report(status, KV_ERR_BOUNDS);
   }
   // The sequences are put into groups longest first, so that the last groups, which decide how evenly the CTAs
   // finish, hold the cheapest items: a counting sort of the sequences on their length (ties in arrival order: only
@@ -224,7 +224,7 @@ __device__ __forceinline__ void plan_body(const PlanArgs& pa) {
       return (int)min((int64_t)(kPlanSeqBuckets - 1), (int64_t)(P + E) * kPlanSeqBuckets / span);
     };
     for (int seq = threadIdx.x; seq < batch; seq += blockDim.x) {
-      const int P = __ldg(prefix_lens + seq), E = rows_of(seq);
+      const int P = ptx::ld_plain(prefix_lens + seq), E = rows_of(seq);
       if (P >= 0 && E > 0) atomicAdd(&seq_hist[bucket_of(P, E)], 1);
     }
     __syncthreads();
@@ -254,7 +254,7 @@ __device__ __forceinline__ void plan_body(const PlanArgs& pa) {
     }
     __syncthreads();
     for (int seq = threadIdx.x; seq < batch; seq += blockDim.x) {
-      const int P = __ldg(prefix_lens + seq), E = rows_of(seq);
+      const int P = ptx::ld_plain(prefix_lens + seq), E = rows_of(seq);
       seq_rank[seq] = (P >= 0 && E > 0) ? (unsigned short)atomicAdd(&seq_hist[bucket_of(P, E)], 1) : 0;
     }
     __syncthreads();
@@ -270,7 +270,7 @@ __device__ __forceinline__ void plan_body(const PlanArgs& pa) {
   };
   for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
     const int seq = (int)(e / max_tp), tp = (int)(e % max_tp);
-    const int P = __ldg(prefix_lens + seq), E = rows_of(seq);
+    const int P = ptx::ld_plain(prefix_lens + seq), E = rows_of(seq);
     if (P < 0 || E <= 0) continue;
     if (((tp * 256) >> lg) >= E) continue;
     const ItemRec r = make_item(seq, tp, P, E, row_of(seq), lg, max_pages, mode, fan);
@@ -310,7 +310,7 @@ __device__ __forceinline__ void plan_body(const PlanArgs& pa) {
   __syncthreads();
   for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
     const int seq = (int)(e / max_tp), tp = (int)(e % max_tp);
-    const int P = __ldg(prefix_lens + seq), E = rows_of(seq);
+    const int P = ptx::ld_plain(prefix_lens + seq), E = rows_of(seq);
     if (P < 0 || E <= 0) continue;
     if (((tp * 256) >> lg) >= E) continue;
     const ItemRec r = make_item(seq, tp, P, E, row_of(seq), lg, max_pages, mode, fan);
@@ -479,8 +479,8 @@ __device__ __forceinline__ void span_load(const TcArgs& a, int base, SpanSeqs& q
   q.base = base;
   q.P = q.rows = q.row0 = 0;
   if (seq < a.batch) {
-    const int P = __ldg(a.prefix_lens + seq), E = __ldg(a.extend_lens + seq);
-    q.row0 = __ldg(a.cu_q + seq);
+    const int P = ptx::ld_plain(a.prefix_lens + seq), E = ptx::ld_plain(a.extend_lens + seq);
+    q.row0 = ptx::ld_plain(a.cu_q + seq);
     q.P = P;
     q.rows = span_rows(a, P, E, q.row0);
     if (blockIdx.x == 0 && P >= 0 && q.rows < E) report(a.pool.status, KV_ERR_BOUNDS);
@@ -686,13 +686,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
   if (CLUSTER && warp == kWarpSched) {  // the item's lengths are asked for while the CTA is set up
     const int seq = (int)blockIdx.x / a.cl_splits / a.pool.n_kv_heads / a.span.max_tp;
     if (!a.span.plan_early) dependency_wait();
-    cl_P = __ldg(a.prefix_lens + seq);
+    cl_P = ptx::ld_plain(a.prefix_lens + seq);
     if (FAN) {  // a parent's rows are those of its children
-      cl_row0 = __ldg(a.fan.cu_q + __ldg(a.fan.cu_children + seq));
-      cl_E = __ldg(a.fan.cu_q + __ldg(a.fan.cu_children + seq + 1)) - cl_row0;
+      cl_row0 = ptx::ld_plain(a.fan.cu_q + ptx::ld_plain(a.fan.cu_children + seq));
+      cl_E = ptx::ld_plain(a.fan.cu_q + ptx::ld_plain(a.fan.cu_children + seq + 1)) - cl_row0;
     } else {
-      cl_E = __ldg(a.extend_lens + seq);
-      cl_row0 = __ldg(a.cu_q + seq);
+      cl_E = ptx::ld_plain(a.extend_lens + seq);
+      cl_row0 = ptx::ld_plain(a.cu_q + seq);
     }
     for (int b = lane * 32; b < a.max_pages; b += 1024) prefetch_l2(a.block_tables + (int64_t)seq * a.max_pages + b);
   }
@@ -783,7 +783,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
         const int g = (j + (REC ? it.first_tile : 0)) * 8 + lane;
         if (FAN && lane < np && g >= n_own) {
           while (true) {
-            const int pages = (__ldg(a.fan.cu_q + child + 1) - __ldg(a.fan.cu_q + child) + kPageSize - 1) / kPageSize;
+            const int pages = (ptx::ld_plain(a.fan.cu_q + child + 1) - ptx::ld_plain(a.fan.cu_q + child) + kPageSize - 1) / kPageSize;
             if (g < child_at + pages || child + 1 >= a.fan.n_children) break;
             child_at += pages;
             ++child;
@@ -791,7 +791,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
           src_bt = a.fan.tables + (int64_t)child * a.fan.max_pages + (g - child_at) - lane;
         }
         if (lane < np) {
-          page = __ldg(src_bt + lane);
+          page = ptx::ld_plain(src_bt + lane);
           if ((unsigned)page >= (unsigned)a.pool.num_pages) {
             report(a.pool.status, KV_ERR_BOUNDS);
             page = 0;
@@ -1229,13 +1229,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
         orow_idx = (int64_t)(it.row0 + tok) * Hq + it.kvh * G + (rg & (G - 1));  // row of the LSE
         if (SPAN) part = it.part;
         if (FAN && valid) {
-          int c = it.c_first, r0 = __ldg(a.fan.cu_q + c) - it.row0, r1 = __ldg(a.fan.cu_q + c + 1) - it.row0;
+          int c = it.c_first, r0 = ptx::ld_plain(a.fan.cu_q + c) - it.row0, r1 = ptx::ld_plain(a.fan.cu_q + c + 1) - it.row0;
           f_lo = (it.P + kPageSize - 1) / kPageSize * kPageSize - it.first_tile * 128;
           while (tok >= r1 && c + 1 < a.fan.n_children) {
             f_lo += (r1 - r0 + kPageSize - 1) / kPageSize * kPageSize;
             ++c;
             r0 = r1;
-            r1 = __ldg(a.fan.cu_q + c + 1) - it.row0;
+            r1 = ptx::ld_plain(a.fan.cu_q + c + 1) - it.row0;
           }
           f_hi = f_lo + tok - r0 + 1;
         }

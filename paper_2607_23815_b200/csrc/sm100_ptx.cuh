@@ -33,6 +33,20 @@ __device__ __forceinline__ bool elect_one_sync() {
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Loads of a kernel that is launched early.  It is resident while the kernels in front of it still write what it will read,
+// so the read-only path (__ldg, ld.global.nc: for data that nobody writes while the kernel lives) is not for it: plain loads,
+// volatile so that none moves in front of the wait.
+__device__ __forceinline__ int ld_plain(const int* p) {
+  int v;
+  asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint4 ld_plain(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+
 // ---- clusters: barrier over all threads of the cluster, the partners' shared memory ------------
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
