@@ -1431,7 +1431,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
       }
       float2* part_ml = reinterpret_cast<float2*>(a.span.part_lse);  // [CTA][row]: maximum (log2 domain) and sum
       if (row < u.x) part_ml[blockIdx.x * a.span.rows + row] = make_float2(cl_m, cl_l);
-      __syncwarp();
       cluster_arrive();
       cluster_wait();
       const int r_begin = u.x * rank / splits, cnt = u.x * (rank + 1) / splits - r_begin;
@@ -1496,7 +1495,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
     }
   }
   if (CLUSTER && a.cl_splits > 1 && warp >= kWarpEpilogue) {  // the other warps' part in the cluster barrier
-    __syncwarp();
     cluster_arrive();
     cluster_wait();
   }
