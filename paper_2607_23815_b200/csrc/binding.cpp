@@ -28,9 +28,15 @@ const at::Tensor& tensor(PyObject* o) {
   return t;
 }
 
-void* data(const at::Tensor& t) { return const_cast<void*>(t.const_data_ptr()); }
+// Addresses are taken before the interpreter lock is let go: a tensor without storage of its own (a fake one) throws here.
 template <typename T = void>
-T* ptr(PyObject* o) { return o == Py_None ? nullptr : static_cast<T*>(data(tensor(o))); }
+const T* read(const at::Tensor& t) { return static_cast<const T*>(t.const_data_ptr()); }
+template <typename T = void>
+T* written(const at::Tensor& t) { return static_cast<T*>(const_cast<void*>(t.const_data_ptr())); }
+template <typename T = void>
+const T* read(PyObject* o) { return o == Py_None ? nullptr : read<T>(tensor(o)); }
+template <typename T = void>
+T* written(PyObject* o) { return o == Py_None ? nullptr : written<T>(tensor(o)); }
 int size(const at::Tensor& t, int dim) {
   if (dim >= t.dim()) raise(PyExc_IndexError, "tensor has too few dimensions");
   return (int)t.size(dim);
@@ -69,7 +75,7 @@ struct Workspace {
   explicit Workspace(PyObject* o) {
     if (o == Py_None) return;
     const at::Tensor& t = tensor(o);
-    p = data(t);
+    p = written(t);
     bytes = t.nbytes();
   }
 };
@@ -106,25 +112,25 @@ PyObject* call(Py_ssize_t got, Py_ssize_t want, Body body) {
     return nullptr;
   }
 }
+// Calls f without the interpreter lock, which is held again however f is left.
 template <typename F>
 long unlocked(F f) {
-  long status;
-  Py_BEGIN_ALLOW_THREADS;
-  status = f();
-  Py_END_ALLOW_THREADS;
-  return status;
+  struct Unlock {
+    PyThreadState* state = PyEval_SaveThread();
+    ~Unlock() { PyEval_RestoreThread(state); }
+  } unlock;
+  return f();
 }
 
 PyObject* append(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return call(n, 8, [&] {
     kv_pool_t* p = pool(a[0]);
     const at::Tensor &k = tensor(a[1]), &start = tensor(a[4]), &bt = tensor(a[6]);
-    void *v = ptr(a[2]), *st = stream(a[7]);
-    const int *cu = ptr<int>(a[3]), *row = ptr<int>(a[5]);
+    const void *kp = read(k), *vp = read(a[2]);
+    const int *cu = read<int>(a[3]), *startp = read<int>(start), *row = read<int>(a[5]), *btp = read<int>(bt);
+    void* st = stream(a[7]);
     const int pages = size(bt, 1), segs = (int)start.numel(), total = size(k, 0);
-    return unlocked([&] {
-      return kv_append(p, data(k), v, cu, (const int*)data(start), row, (const int*)data(bt), pages, segs, total, st);
-    });
+    return unlocked([&] { return kv_append(p, kp, vp, cu, startp, row, btp, pages, segs, total, st); });
   });
 }
 
@@ -132,15 +138,14 @@ PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return call(n, 10, [&] {
     kv_pool_t* p = pool(a[0]);
     const at::Tensor &q = tensor(a[1]), &bt = tensor(a[2]);
-    const int* ctx = ptr<int>(a[3]);
+    const void* qp = read(q);
+    const int *btp = read<int>(bt), *ctx = read<int>(a[3]);
     const int max_ctx = integer(a[4]), hq = size(q, 1), pages = size(bt, 1), batch = size(q, 0);
     const float scale = real(a[5]);
-    void *out = ptr(a[6]), *st = stream(a[9]);
-    float* lse = ptr<float>(a[7]);
+    void *out = written(a[6]), *st = stream(a[9]);
+    float* lse = written<float>(a[7]);
     const Workspace ws(a[8]);
-    return unlocked([&] {
-      return attn_decode(p, data(q), hq, (const int*)data(bt), pages, ctx, batch, max_ctx, scale, out, lse, ws.p, ws.bytes, st);
-    });
+    return unlocked([&] { return attn_decode(p, qp, hq, btp, pages, ctx, batch, max_ctx, scale, out, lse, ws.p, ws.bytes, st); });
   });
 }
 
@@ -152,16 +157,16 @@ PyObject* extend_like(PyObject* const* a, Py_ssize_t n, int lead, F f) {  // lea
     const at::Tensor& q = tensor(a[1]);
     PyObject* const* b = a + lead;
     const at::Tensor &bt = tensor(b[1]), &pl = tensor(b[2]);
-    const int *cu = ptr<int>(b[0]), *el = ptr<int>(b[3]);
-    const int max_e = integer(b[4]), max_l = integer(b[5]), hq = size(q, 1), total = size(q, 0), pages = size(bt, 1);
+    const void* qp = read(q);
+    const int *cu = read<int>(b[0]), *btp = read<int>(bt), *plp = read<int>(pl), *el = read<int>(b[3]);
+    const int batch = (int)pl.numel(), max_e = integer(b[4]), max_l = integer(b[5]), hq = size(q, 1), total = size(q, 0), pages = size(bt, 1);
     const float scale = real(b[6]);
-    void *out = ptr(b[7]), *st = stream(b[10]);
-    float* lse = ptr<float>(b[8]);
+    void *out = written(b[7]), *st = stream(b[10]);
+    float* lse = written<float>(b[8]);
     const Workspace ws(b[9]);
-    void *k = lead == 4 ? ptr(a[2]) : nullptr, *v = lead == 4 ? ptr(a[3]) : nullptr;
+    const void *k = lead == 4 ? read(a[2]) : nullptr, *v = lead == 4 ? read(a[3]) : nullptr;
     return unlocked([&] {
-      return f(p, data(q), k, v, hq, cu, (const int*)data(bt), pages, (const int*)data(pl), el, (int)pl.numel(), total, max_e, max_l,
-               scale, out, lse, ws.p, ws.bytes, st);
+      return f(p, qp, k, v, hq, cu, btp, pages, plp, el, batch, total, max_e, max_l, scale, out, lse, ws.p, ws.bytes, st);
     });
   });
 }
@@ -180,14 +185,11 @@ PyObject* extend_plan(PyObject*, PyObject* const* a, Py_ssize_t n) {
     kv_pool_t* p = pool(a[0]);
     const int hq = integer(a[1]), total = integer(a[6]), max_e = integer(a[7]), max_l = integer(a[8]);
     const at::Tensor &bt = tensor(a[3]), &pl = tensor(a[4]);
-    const int *cu = ptr<int>(a[2]), *el = ptr<int>(a[5]);
-    const int pages = size(bt, 1);
+    const int *cu = read<int>(a[2]), *btp = read<int>(bt), *plp = read<int>(pl), *el = read<int>(a[5]);
+    const int pages = size(bt, 1), batch = (int)pl.numel();
     const Workspace ws(a[9]);
     void* st = stream(a[10]);
-    return unlocked([&] {
-      return attn_extend_plan(p, hq, cu, (const int*)data(bt), pages, (const int*)data(pl), el, (int)pl.numel(), total, max_e, max_l,
-                              ws.p, ws.bytes, st);
-    });
+    return unlocked([&] { return attn_extend_plan(p, hq, cu, btp, pages, plp, el, batch, total, max_e, max_l, ws.p, ws.bytes, st); });
   });
 }
 
@@ -195,17 +197,17 @@ PyObject* extend_shared(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return call(n, 16, [&] {
     kv_pool_t* p = pool(a[0]);
     const at::Tensor &q = tensor(a[1]), &pt = tensor(a[4]), &pl = tensor(a[5]), &ct = tensor(a[6]), &cl = tensor(a[7]);
-    const int *cu = ptr<int>(a[2]), *cc = ptr<int>(a[3]);
-    const int max_c = integer(a[8]), max_rows = integer(a[9]), max_p = integer(a[10]);
+    const void* qp = read(q);
+    const int *cu = read<int>(a[2]), *cc = read<int>(a[3]), *ptp = read<int>(pt), *plp = read<int>(pl), *ctp = read<int>(ct), *clp = read<int>(cl);
+    const int max_c = integer(a[8]), max_rows = integer(a[9]), max_p = integer(a[10]), parents = (int)pl.numel(), children = (int)cl.numel();
     const int hq = size(q, 1), total = size(q, 0), pages_p = size(pt, 1), pages_c = size(ct, 1);
     const float scale = real(a[11]);
-    void *out = ptr(a[12]), *st = stream(a[15]);
-    float* lse = ptr<float>(a[13]);
+    void *out = written(a[12]), *st = stream(a[15]);
+    float* lse = written<float>(a[13]);
     const Workspace ws(a[14]);
     return unlocked([&] {
-      return attn_extend_shared(p, data(q), hq, cu, cc, (const int*)data(pt), pages_p, (const int*)data(pl), (const int*)data(ct), pages_c,
-                                (const int*)data(cl), (int)pl.numel(), (int)cl.numel(), total, max_c, max_rows, max_p, scale, out, lse,
-                                ws.p, ws.bytes, st);
+      return attn_extend_shared(p, qp, hq, cu, cc, ptp, pages_p, plp, ctp, pages_c, clp, parents, children, total, max_c, max_rows, max_p,
+                                scale, out, lse, ws.p, ws.bytes, st);
     });
   });
 }
@@ -235,13 +237,16 @@ PyObject* extend_host(PyObject*, PyObject* const* a, Py_ssize_t n) {
     kv_pool_t* p = pool(a[0]);
     const at::Tensor &q = host_tensor(a[1]), &k = host_tensor(a[2]), &v = host_tensor(a[3]), &cu = host_tensor(a[4]), &bt = host_tensor(a[5]),
                      &pl = host_tensor(a[6]), &el = host_tensor(a[7]), &out = host_tensor(a[11]), &lse = host_tensor(a[12]);
-    const int max_e = integer(a[8]), max_l = integer(a[9]), hq = size(q, 1), total = size(q, 0), pages = size(bt, 1);
+    const void *qp = read(q), *kp = read(k), *vp = read(v);
+    const int *cup = read<int>(cu), *btp = read<int>(bt), *plp = read<int>(pl), *elp = read<int>(el);
+    const int max_e = integer(a[8]), max_l = integer(a[9]), hq = size(q, 1), total = size(q, 0), pages = size(bt, 1), batch = (int)pl.numel();
     const float scale = real(a[10]);
+    void* outp = written(out);
+    float* lsep = written<float>(lse);
     const Workspace staging(a[13]);
     void* st = stream(a[14]);
     return unlocked([&] {
-      return attn_extend_host(p, data(q), data(k), data(v), hq, (const int*)data(cu), (const int*)data(bt), pages, (const int*)data(pl),
-                              (const int*)data(el), (int)pl.numel(), total, max_e, max_l, scale, data(out), (float*)data(lse), staging.p,
+      return attn_extend_host(p, qp, kp, vp, hq, cup, btp, pages, plp, elp, batch, total, max_e, max_l, scale, outp, lsep, staging.p,
                               staging.bytes, st);
     });
   });

@@ -1,8 +1,14 @@
 """The native half of the binding checks its arguments before it calls the library (no GPU needed)."""
+import os
+import subprocess
+import sys
+
 import pytest
 import torch
 
 from paper_2607_23815_b200 import kvattn
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 class _NoPool:
@@ -26,3 +32,45 @@ def test_errors_of_the_library_come_back_as_kverror():
     assert e.value.status == kvattn.KV_ERR_INVALID
     with pytest.raises(TypeError):                                        # a structure of another kind
         kvattn.attn_mixed(_NoPool, 8, 1.0, kvattn.DecodeArgs(), None, None, 0)
+
+
+_NO_STORAGE = """
+import faulthandler; faulthandler.enable()
+import torch
+from torch._subclasses.fake_tensor import FakeTensorMode
+from paper_2607_23815_b200 import kvattn
+class NoPool:
+    ptr = None
+with FakeTensorMode():
+    args = [torch.empty(3, 2, 4, 64, dtype=torch.bfloat16, device="cuda"), torch.empty(3, 2, 8, dtype=torch.int32, device="cuda"),
+            torch.empty(3, 64, dtype=torch.uint8, device="cuda")]
+calls = {
+    "append": lambda t, i, b: kvattn.kv_append(NoPool, t, None, None, i, None, i, 0),
+    "decode": lambda t, i, b: kvattn.attn_decode(NoPool, t, i, None, 5, 1.0, None, None, None, 0),
+    "extend": lambda t, i, b: kvattn.attn_extend(NoPool, t, None, i, i, None, 1, 5, 1.0, None, None, None, 0),
+    "planned": lambda t, i, b: kvattn.attn_extend_planned(NoPool, t, None, i, i, None, 1, 5, 1.0, None, None, None, 0),
+    "extend_append": lambda t, i, b: kvattn.attn_extend_append(NoPool, t, None, None, None, i, i, None, 1, 5, 1.0, None, None, None, 0),
+    "plan": lambda t, i, b: kvattn.attn_extend_plan(NoPool, 4, None, i, i, None, 2, 1, 5, None, 0),
+    "shared": lambda t, i, b: kvattn.attn_extend_shared(NoPool, t, None, None, i, i, i, i, 1, 1, 5, 1.0, None, None, None, 0),
+    "mixed": lambda t, i, b: kvattn.attn_mixed(NoPool, 4, 1.0, None, None, b, 0),
+}
+def refused(*tensors):
+    for name, call in calls.items():
+        for _ in range(3):
+            try:
+                call(*tensors)
+            except RuntimeError as e:
+                assert not isinstance(e, kvattn.KvError), name
+            else:
+                raise SystemExit(name + ": no error")
+    return tensors[0]
+torch.vmap(refused)(*args)
+print("all refused")
+"""
+
+
+def test_tensors_without_storage_are_an_error_and_not_a_crash():
+    # the address of such a tensor (here: one that vmap batches) cannot be had; the exception must not leave the call without
+    # the interpreter lock
+    r = subprocess.run([sys.executable, "-c", _NO_STORAGE], capture_output=True, text=True, cwd=ROOT, timeout=300)
+    assert r.returncode == 0 and "all refused" in r.stdout, (r.returncode, r.stdout, r.stderr[-2000:])
