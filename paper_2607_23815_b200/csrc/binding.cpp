@@ -29,10 +29,11 @@ const at::Tensor& tensor(PyObject* o) {
 }
 
 // Addresses are taken before the interpreter lock is let go: a tensor without storage of its own (a fake one) throws here.
+// read: for what the library only reads; written: the tensor's own memory, brought about if it still shares another's.
 template <typename T = void>
 const T* read(const at::Tensor& t) { return static_cast<const T*>(t.const_data_ptr()); }
 template <typename T = void>
-T* written(const at::Tensor& t) { return static_cast<T*>(const_cast<void*>(t.const_data_ptr())); }
+T* written(const at::Tensor& t) { return static_cast<T*>(t.mutable_data_ptr()); }
 template <typename T = void>
 const T* read(PyObject* o) { return o == Py_None ? nullptr : read<T>(tensor(o)); }
 template <typename T = void>

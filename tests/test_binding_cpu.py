@@ -74,3 +74,17 @@ def test_tensors_without_storage_are_an_error_and_not_a_crash():
     # the interpreter lock
     r = subprocess.run([sys.executable, "-c", _NO_STORAGE], capture_output=True, text=True, cwd=ROOT, timeout=300)
     assert r.returncode == 0 and "all refused" in r.stdout, (r.returncode, r.stdout, r.stderr[-2000:])
+
+
+def _host_call(out):
+    t, i = torch.zeros(2, 4, 64, dtype=torch.bfloat16), torch.zeros(2, 8, dtype=torch.int32)
+    with pytest.raises(kvattn.KvError) as e:                              # no pool: refused by the library itself
+        kvattn.attn_extend_host(_NoPool, t, t, t, i[0], i, i[0], i[0], 1, 5, 1.0, out, torch.zeros(2, 4), None, 0)
+    assert e.value.status == kvattn.KV_ERR_INVALID
+
+
+def test_results_go_to_the_tensor_s_own_memory():
+    base = torch.zeros(2, 4, 64, dtype=torch.bfloat16)
+    out = torch._lazy_clone(base)                                         # shares its memory until somebody writes
+    _host_call(out)
+    assert not torch._C._is_cow_tensor(out) and out.data_ptr() != base.data_ptr()
