@@ -59,11 +59,10 @@ kv_pool_t* pool(PyObject* o) {
   if (p == nullptr && PyErr_Occurred()) throw Raised{};
   return static_cast<kv_pool_t*>(p);
 }
-// None: torch's current stream; else a stream object or its handle.
+// None: torch's current stream; else a stream object or its handle (anything that int() takes).
 void* stream(PyObject* o) {
   if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
-  if (PyLong_Check(o)) return PyLong_AsVoidPtr(o);
-  PyObject* h = PyObject_GetAttrString(o, "cuda_stream");
+  PyObject* h = PyObject_HasAttrString(o, "cuda_stream") ? PyObject_GetAttrString(o, "cuda_stream") : PyNumber_Long(o);
   if (h == nullptr) throw Raised{};
   void* p = PyLong_AsVoidPtr(h);
   Py_DECREF(h);

@@ -3,6 +3,7 @@ import os
 import subprocess
 import sys
 
+import numpy as np
 import pytest
 import torch
 
@@ -76,10 +77,10 @@ def test_tensors_without_storage_are_an_error_and_not_a_crash():
     assert r.returncode == 0 and "all refused" in r.stdout, (r.returncode, r.stdout, r.stderr[-2000:])
 
 
-def _host_call(out):
+def _host_call(out, stream=0):
     t, i = torch.zeros(2, 4, 64, dtype=torch.bfloat16), torch.zeros(2, 8, dtype=torch.int32)
     with pytest.raises(kvattn.KvError) as e:                              # no pool: refused by the library itself
-        kvattn.attn_extend_host(_NoPool, t, t, t, i[0], i, i[0], i[0], 1, 5, 1.0, out, torch.zeros(2, 4), None, 0)
+        kvattn.attn_extend_host(_NoPool, t, t, t, i[0], i, i[0], i[0], 1, 5, 1.0, out, torch.zeros(2, 4), None, stream)
     assert e.value.status == kvattn.KV_ERR_INVALID
 
 
@@ -88,3 +89,8 @@ def test_results_go_to_the_tensor_s_own_memory():
     out = torch._lazy_clone(base)                                         # shares its memory until somebody writes
     _host_call(out)
     assert not torch._C._is_cow_tensor(out) and out.data_ptr() != base.data_ptr()
+
+
+@pytest.mark.parametrize("stream", [0, np.int64(0)])
+def test_a_stream_is_whatever_is_a_handle(stream):
+    _host_call(torch.zeros(2, 4, 64, dtype=torch.bfloat16), stream)
