@@ -59,7 +59,7 @@ def build_binding(force: bool = False, verbose: bool = False) -> str:
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
-    if force or _stale(LIB, (".cu", ".cuh")):
+    if force or _stale(LIB, (".cu", ".cuh", ".h")):
         _run([_nvcc()] + NVCC_FLAGS + ["-Xlinker", "-soname=libkvattn.so", "-o", LIB] + [os.path.join(CSRC, s) for s in SOURCES],
              verbose, "libkvattn.so")
     build_binding(force, verbose)

@@ -1,6 +1,9 @@
 // Public attention entry points: argument checks, kernel selection, the mixed-batch launcher.
+#include <cuda.h>  // pointer attributes (types only: the call is looked up at run time)
+
 #include "append.cuh"
 #include "common.cuh"
+#include "host_view.h"
 
 namespace kvattn {
 size_t decode_workspace_bytes(int n_q_heads, int head_dim, int batch, int max_ctx_len);
@@ -234,17 +237,28 @@ kv_status_t launch_copies(const Copies& c, size_t max_blocks, cudaStream_t st) {
   return KV_OK;
 }
 
-// The address at which the device reaches a host buffer that is pinned from its first byte to its last, else nullptr.
+// The address at which the device reaches a host buffer that lies in one pinned allocation or registration, else nullptr.
 void* device_view(const void* host, size_t bytes) {
-  cudaPointerAttributes a, z;
-  if (cudaPointerGetAttributes(&a, host) != cudaSuccess ||
-      cudaPointerGetAttributes(&z, (const char*)host + bytes - 1) != cudaSuccess) {
+  typedef CUresult (*query_fn)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+  static const query_fn query = [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &fn, cudaEnableDefault, &found) != cudaSuccess || found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      return query_fn(nullptr);
+    }
+    return reinterpret_cast<query_fn>(fn);
+  }();
+  cudaPointerAttributes at;
+  if (query == nullptr || cudaPointerGetAttributes(&at, host) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
   }
-  const bool pinned = a.type == cudaMemoryTypeHost && z.type == cudaMemoryTypeHost &&
-                      (const char*)z.devicePointer - (const char*)a.devicePointer == (ptrdiff_t)bytes - 1;
-  return pinned && ((uintptr_t)a.devicePointer & 3) == 0 ? a.devicePointer : nullptr;
+  HostAddress a{at.type == cudaMemoryTypeHost, (uintptr_t)at.devicePointer, 0, 0};
+  CUpointer_attribute names[] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* values[] = {&a.range_start, &a.range_bytes};
+  if (!a.pinned || a.device == 0 || query(2, names, values, (CUdeviceptr)a.device) != CUDA_SUCCESS) return nullptr;
+  return reinterpret_cast<void*>(kvattn::device_view(a, bytes));
 }
 }  // namespace
 

@@ -56,3 +56,50 @@ def test_host_step_gives_the_bits_of_the_device_call(extend, pinned):
     for o in outs[1:]:
         assert np.array_equal(o[0], outs[0][0]) and np.array_equal(o[1], outs[0][1])
         assert np.array_equal(o[2][0], outs[0][2][0]) and np.array_equal(o[2][1], outs[0][2][1])
+
+
+def _registered(t, region, at):
+    """A host copy of t at byte `at` of a registered region."""
+    view = region[at:at + t.numel() * t.element_size()].view(t.dtype).view(t.shape)
+    view.copy_(t)
+    return view
+
+
+def test_buffers_inside_one_registration_are_copied_by_the_kernel():
+    # memory that the caller registered instead of allocating it pinned; the last buffer ends with the region
+    geom, P, E = synth.Geometry(8, 2, 128), [37, 250], [60, 33]
+    L = [p + e for p, e in zip(P, E)]
+    dp = DualPool(geom, 64, seed=72, with_oracle=False)
+    b = Batch(dp, L)
+    b.write([(i, 0, P[i]) for i in range(2)])
+    ks, vs = zip(*[b.kv(i, P[i], L[i]) for i in range(2)])
+    q = torch.cat([b.q(i, P[i], L[i]) for i in range(2)]).contiguous()
+    i32 = lambda x: torch.tensor(np.asarray(x), dtype=torch.int32)
+    arrays = [t.cpu() for t in (q, torch.cat(ks), torch.cat(vs), i32(np.concatenate([[0], np.cumsum(E)])), torch.from_numpy(b.block_tables()),
+                                i32(P), i32(E), torch.zeros_like(q), torch.zeros((q.shape[0], 8)))]
+    starts, at = [], 4
+    for t in arrays:
+        starts.append(at)
+        at += t.numel() * t.element_size()
+    outs, launches = [], []
+    region = torch.zeros(at, dtype=torch.uint8)
+    staging = torch.empty(kvattn.attn_extend_host_staging_bytes(dp.pool, 8, 2, int(q.shape[0]), arrays[4].shape[1], max(L)), dtype=torch.uint8,
+                          device="cuda")
+    for registered in (False, True):
+        if registered:
+            assert torch.cuda.cudart().cudaHostRegister(region.data_ptr(), at, 0) == torch.cuda.cudart().cudaError.success
+        try:
+            h = [_registered(t, region, s) for t, s in zip(arrays, starts)]
+            before = kvattn.kvattn_launch_count()
+            kvattn.attn_extend_host(dp.pool, *h[:7], max(E), max(L), geom.scale, h[7], h[8], staging)
+            torch.cuda.synchronize()
+            launches.append(kvattn.kvattn_launch_count() - before)
+            outs.append((synth.bf16_bits(h[7]).copy(), h[8].numpy().copy()))
+        finally:
+            if registered:
+                torch.cuda.synchronize()
+                torch.cuda.cudart().cudaHostUnregister(region.data_ptr())
+    assert launches[1] == launches[0] + 2                                  # one copy kernel in, one out
+    assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1]) and np.any(outs[0][1] != 0)
+    assert kvattn.kv_last_async_status(dp.pool) == kvattn.KV_OK
+    dp.close()
