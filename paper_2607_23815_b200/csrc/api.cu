@@ -470,13 +470,15 @@ kv_status_t attn_mixed(kv_pool_t* p, int n_q_heads, float scale, const attn_exte
                                 ext->extend_lens, ext->batch, ext->total_q, ext->max_extend_len, ext->max_total_len,
                                 scale, ext->out, ext->lse, ws, ext_bytes, cap, st);
     if (s != KV_OK) return s;
-    s = decode_impl(p, dec->q, n_q_heads, dec->block_tables, dec->max_pages, dec->ctx_lens, dec->batch, dec->max_ctx_len,
-                    scale, dec->out, dec->lse, ws ? ws + ext_bytes : nullptr, workspace_bytes - ext_bytes, st, true);
-    if (s != KV_OK) return s;
-    // (the extend kernel's cut items are merged behind both kernels: the decode kernel must be the next in the stream)
-    if (!uses_tc(p, n_q_heads, scale)) return KV_OK;
-    return launch_extend_combine(p, n_q_heads, ext->batch, ext->total_q, ext->max_extend_len, ext->max_total_len, ext->out, ext->lse, ws, ext_bytes,
-                                 false, st);
+    const kv_status_t ds = decode_impl(p, dec->q, n_q_heads, dec->block_tables, dec->max_pages, dec->ctx_lens, dec->batch,
+                                       dec->max_ctx_len, scale, dec->out, dec->lse, ws ? ws + ext_bytes : nullptr,
+                                       workspace_bytes - ext_bytes, st, true);
+    // The extend kernel's cut items are merged behind both kernels (the decode kernel must be the next in the stream), also if
+    // the decode set is refused: the extend set has been launched and its results are to be whole.
+    if (uses_tc(p, n_q_heads, scale))
+      s = launch_extend_combine(p, n_q_heads, ext->batch, ext->total_q, ext->max_extend_len, ext->max_total_len, ext->out, ext->lse, ws,
+                                ext_bytes, false, st);
+    return ds != KV_OK ? ds : s;
   }
   if (has_ext)
     return attn_extend(p, ext->q, n_q_heads, ext->cu_q, ext->block_tables, ext->max_pages, ext->prefix_lens,
