@@ -307,7 +307,8 @@ kv_status_t attn_extend_host(kv_pool_t* p, const void* q, const void* k_new, con
   if (((uintptr_t)staging) & 255) return KV_ERR_INVALID;
   if (!on_pool_device(p)) return KV_ERR_INVALID;
   const HostStepLayout L = host_step_layout(p, n_q_heads, batch, total_q, max_pages, max_total_len);
-  if (staging_bytes < L.total) return KV_ERR_WORKSPACE;
+  // (less than attn_extend_host_staging_bytes() asks for, but enough without partial results of cut items)
+  if (staging_bytes < L.ws + align256(extend_tc_min_workspace_bytes(batch, total_q)) + 256) return KV_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   char* d = reinterpret_cast<char*>(staging);
   const size_t D = (size_t)p->head_dim;
@@ -357,7 +358,7 @@ kv_status_t attn_extend_host(kv_pool_t* p, const void* q, const void* k_new, con
   // the suffix K/V rows of sequence i go to positions prefix_lens[i] .. of its pages, then the suffix attends
   kv_status_t s = attn_extend_append(p, d + L.q, d + L.k, d + L.v, n_q_heads, d_cu, d_bt, max_pages, d_pl, d_el, batch, total_q,
                                      max_extend_len, max_total_len, scale, d + L.out, reinterpret_cast<float*>(d + L.lse),
-                                     d + L.ws, L.total - L.ws, stream);
+                                     d + L.ws, (staging_bytes < L.total ? staging_bytes : L.total) - L.ws, stream);
   KV_CUDA_OK(cudaEventRecord(hs->ran, st));
   if (s != KV_OK) return s;
   KV_CUDA_OK(cudaStreamWaitEvent(p->d2h_stream, hs->ran, 0));

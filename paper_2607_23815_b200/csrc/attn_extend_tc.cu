@@ -1622,8 +1622,8 @@ size_t extend_tc_workspace_bytes(const kv_pool_t* p, int n_q_heads, int batch, i
   const size_t list = list_bytes(batch, total_q), spans = span_layout(p, n_q_heads, batch, total_q, max_total_len).total;
   return 256 + (list > spans ? list : spans);
 }
-// The least the extend kernel runs with (without span scheduling).
-size_t extend_tc_min_workspace_bytes(int batch, int total_q) { return 256 + list_bytes(batch, total_q); }
+// The least the extend kernel runs with: the list, at any 16-byte boundary.
+size_t extend_tc_min_workspace_bytes(int batch, int total_q) { return list_bytes(batch, total_q); }
 
 bool extend_tc_supported(const kv_pool_t* p, int n_q_heads) {
   if (p->head_dim != 64 && p->head_dim != 128) return false;
@@ -1799,8 +1799,11 @@ static SpanArgs span_args(const SpanLayout& l, char* ws, int max_tp, int total_q
   a.part_o = l.cuts ? reinterpret_cast<float*>(ws + l.o) : nullptr;
   return a;
 }
-static char* align_workspace(void* ws) {
-  return reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(ws) + 255) & ~(uintptr_t)255);
+// Where the workspace begins: on a 256-byte boundary, or, if that does not leave `need` bytes of it, where the caller says.
+static char* align_workspace(void* ws, size_t bytes, size_t need) {
+  char* at = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(ws) + 255) & ~(uintptr_t)255);
+  const size_t skip = (size_t)(at - reinterpret_cast<char*>(ws));
+  return skip + need <= bytes ? at : reinterpret_cast<char*>(ws);
 }
 
 // Merges the chunks of cut items behind a span-scheduled attention kernel; nothing to do for other batches.  early: that
@@ -1816,7 +1819,7 @@ kv_status_t launch_extend_combine(kv_pool_t* p, int n_q_heads, int batch, int to
   const int G = n_q_heads / p->n_kv_heads;
   int lg = 0;
   while ((1 << lg) < G) ++lg;
-  const SpanArgs a = span_args(l, align_workspace(workspace), 0, total_q, 0);
+  const SpanArgs a = span_args(l, align_workspace(workspace, workspace_bytes, l.total), 0, total_q, 0);
   const auto kernel = p->head_dim == 128 ? span_combine_kernel<128> : span_combine_kernel<64>;
   const unsigned blocks = (unsigned)((a.n_spans - 1) * kCombineSlices), threads = (unsigned)p->head_dim * 4;
   if (early) {
@@ -1848,7 +1851,8 @@ kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const i
   }
   int lg = 0;
   while ((1 << lg) < G) ++lg;
-  char* ws = align_workspace(workspace);
+  char* ws = align_workspace(workspace, workspace_bytes, need);
+  if ((reinterpret_cast<uintptr_t>(ws) & 15) != 0) return KV_ERR_WORKSPACE;  // (the list holds 16-byte records)
   int* n_items = reinterpret_cast<int*>(ws);
   int4* items = reinterpret_cast<int4*>(ws + 256);
   const int64_t capacity = item_capacity(n_q_heads, p->n_kv_heads, batch, total_q);
@@ -1924,7 +1928,8 @@ kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const i
   const bool opt = max_total_len >= kOptimisticMinLen;
   bool early = cta_cap >= 0;
   if (sched != kSchedList) {
-    a.span = span_args(span_layout(p, n_q_heads, batch, total_q, max_total_len), ws, max_tp, total_q, sched == kSchedSpans ? cta_cap : 0);
+    const SpanLayout l = span_layout(p, n_q_heads, batch, total_q, max_total_len);
+    a.span = span_args(l, align_workspace(workspace, workspace_bytes, l.total), max_tp, total_q, sched == kSchedSpans ? cta_cap : 0);
     a.span.plan_early = app != nullptr && app->total_new > 0;
     a.cl_splits = splits;
     grid = sched == kSchedSpans ? (a.span.n_spans + a.span.per_cta - 1) / a.span.per_cta : batch * max_tp * p->n_kv_heads * splits;
