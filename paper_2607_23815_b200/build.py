@@ -15,6 +15,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libkvattn.so")
 BINDING = os.path.join(HERE, "_kvattn_native.so")
+BINDING_FOR = os.path.join(HERE, "_kvattn_native.torch")  # what the module was compiled against (see binding_abi)
 SOURCES = ["pool.cu", "attn_small.cu", "attn_decode.cu", "attn_extend_tc.cu", "attn_decode_static.cu", "attn_shared.cu", "selftest.cu", "api.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "--shared", "-Xcompiler", "-fPIC", "-Xptxas", "-v"]
@@ -43,9 +44,24 @@ def _run(cmd, verbose: bool, what: str) -> None:
         raise RuntimeError(f"building {what} failed")
 
 
+def binding_abi() -> str:
+    """The module uses torch's C++ classes and Python's C API: one compiled against other versions must not be loaded."""
+    import torch
+    return f"torch {torch.__version__} {sysconfig.get_config_var('SOABI')}"
+
+
+def binding_made_for() -> str:
+    """What the module that is there was compiled against, "" if that is not known (the module was copied alone)."""
+    try:
+        with open(BINDING_FOR) as f:
+            return f.read()
+    except OSError:
+        return ""
+
+
 def build_binding(force: bool = False, verbose: bool = False) -> str:
     """The extension module that unpacks torch tensors and calls libkvattn.so (which lies beside it)."""
-    if not force and not _stale(BINDING, (".cpp",)):
+    if not force and binding_made_for() == binding_abi() and not _stale(BINDING, (".cpp",)):
         return BINDING
     import torch
     from torch.utils import cpp_extension as ext
@@ -55,6 +71,8 @@ def build_binding(force: bool = False, verbose: bool = False) -> str:
     _run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
          + [f"-I{d}" for d in inc] + [os.path.join(CSRC, "binding.cpp"), "-o", BINDING, LIB, "-Wl,-rpath,$ORIGIN", f"-L{libs}",
                                       "-lc10", "-lc10_cuda", "-ltorch", "-ltorch_cpu", "-ltorch_python"], verbose, "_kvattn_native.so")
+    with open(BINDING_FOR, "w") as f:
+        f.write(binding_abi())
     return BINDING
 
 

@@ -13,6 +13,8 @@ from typing import Optional, Sequence
 
 import torch
 
+from . import build
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libkvattn.so")
 
@@ -108,9 +110,11 @@ class _NativeLoader:
         global _native
         lib()
         try:
+            if build.binding_made_for() not in ("", build.binding_abi()):
+                raise ImportError("it was compiled against another torch or Python")
             module = importlib.import_module("._kvattn_native", __package__)
         except ImportError as e:
-            raise ImportError("the native binding is missing or stale: build it with `python -m paper_2607_23815_b200.build`") from e
+            raise ImportError(f"the native binding is missing or stale ({e}): build it with `python -m paper_2607_23815_b200.build`") from e
         _native = module
         return getattr(module, name)
 

@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2607_23815_b200 import kvattn
+from paper_2607_23815_b200 import build, kvattn
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -39,7 +39,7 @@ _NO_STORAGE = """
 import faulthandler; faulthandler.enable()
 import torch
 from torch._subclasses.fake_tensor import FakeTensorMode
-from paper_2607_23815_b200 import kvattn
+from paper_2607_23815_b200 import build, kvattn
 class NoPool:
     ptr = None
 with FakeTensorMode():
@@ -94,3 +94,18 @@ def test_results_go_to_the_tensor_s_own_memory():
 @pytest.mark.parametrize("stream", [0, np.int64(0)])
 def test_a_stream_is_whatever_is_a_handle(stream):
     _host_call(torch.zeros(2, 4, 64, dtype=torch.bfloat16), stream)
+
+
+def test_a_module_of_another_torch_is_neither_kept_nor_loaded(tmp_path, monkeypatch):
+    build.build_library()
+    assert build.binding_made_for() == build.binding_abi()
+    stamp = tmp_path / "stamp"
+    stamp.write_text(build.binding_abi().replace("torch ", "torch 1."))    # as a torch upgrade leaves it
+    monkeypatch.setattr(build, "BINDING_FOR", str(stamp))
+    commands = []
+    monkeypatch.setattr(build, "_run", lambda cmd, verbose, what: commands.append(what))
+    with pytest.raises(ImportError, match="stale"):
+        kvattn._NativeLoader().kv_append
+    build.build_library()
+    assert commands == ["_kvattn_native.so"]                                  # rebuilt, and the library is not
+    assert stamp.read_text() == build.binding_abi()
