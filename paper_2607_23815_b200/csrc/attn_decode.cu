@@ -295,15 +295,30 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
 
 std::atomic<int> g_decode_impl{0};  // 0: by the pages per warp, 1: pages stream through registers, 2: pages go through a shared-memory ring
 
-// Prepares the kernel for a device (once).
+// Prepares a variant of the kernel for the current device; asking for its attributes loads its code.
 template <int D, bool RING, bool MULTI>
+static kv_status_t prepare_variant() {
+  cudaFuncAttributes at;
+  KV_CUDA_OK(cudaFuncGetAttributes(&at, attn_decode_kernel<D, RING, MULTI>));
+  KV_CUDA_OK(cudaFuncSetAttribute(attn_decode_kernel<D, RING, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  decode_smem_bytes<D, RING>()));
+  KV_CUDA_OK(cudaFuncSetAttribute(attn_decode_kernel<D, RING, MULTI>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  return KV_OK;
+}
+
+// Prepares the kernel for a device, once, and every variant at a time: which one a later call takes depends on its batch and
+// lengths, and callers that may not allocate (attn_decode_static) or that capture make one call of any shape beforehand.
 static kv_status_t decode_setup(int device) {
   static std::atomic<bool> configured[kMaxDevices];
   if (device < 0 || device >= kMaxDevices) return KV_ERR_INVALID;
   if (!configured[device].load(std::memory_order_acquire)) {
-    KV_CUDA_OK(cudaFuncSetAttribute(attn_decode_kernel<D, RING, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    decode_smem_bytes<D, RING>()));
-    KV_CUDA_OK(cudaFuncSetAttribute(attn_decode_kernel<D, RING, MULTI>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    kv_status_t (*const all[])() = {prepare_variant<128, true, false>, prepare_variant<128, false, false>, prepare_variant<128, true, true>,
+                                    prepare_variant<128, false, true>, prepare_variant<64, true, false>,   prepare_variant<64, false, false>,
+                                    prepare_variant<64, true, true>,   prepare_variant<64, false, true>};
+    for (const auto prepare : all) {
+      const kv_status_t s = prepare();
+      if (s != KV_OK) return s;
+    }
     configured[device].store(true, std::memory_order_release);
   }
   return KV_OK;
@@ -332,7 +347,7 @@ static constexpr int kSplitChoices[] = {1, 2, 3, 4, 6, 8, 16};
 template <int D>
 static kv_status_t resident_clusters(int device, int i, int* n) {
   static std::atomic<int> cached[kMaxDevices][sizeof(kSplitChoices) / sizeof(int)];  // value + 1
-  const kv_status_t s = decode_setup<D, true, false>(device);
+  const kv_status_t s = decode_setup(device);
   if (s != KV_OK) return s;
   int v = cached[device][i].load(std::memory_order_relaxed);
   if (v == 0) {
@@ -427,7 +442,7 @@ static bool few_pages(const kv_pool_t* p, int64_t blocks, int warps, int max_ctx
 
 template <int D, bool RING, bool MULTI>
 static kv_status_t launch_decode_variant(const kv_pool_t* p, const DecodeArgs& a, int64_t blocks, cudaStream_t st) {
-  const kv_status_t s = decode_setup<D, RING, MULTI>(p->device);
+  const kv_status_t s = decode_setup(p->device);
   if (s != KV_OK) return s;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
