@@ -103,3 +103,53 @@ def test_buffers_inside_one_registration_are_copied_by_the_kernel():
     assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1]) and np.any(outs[0][1] != 0)
     assert kvattn.kv_last_async_status(dp.pool) == kvattn.KV_OK
     dp.close()
+
+
+@pytest.mark.parametrize("pinned", [True, False])
+@pytest.mark.parametrize("areas", [1, 2, 5])
+def test_steps_queued_behind_one_another_do_not_mix(areas, pinned):
+    # every step has its own rows, lengths, tables and result buffers; nothing waits until all are queued.  Results below and
+    # above what a kernel copies out (4 MB), rows below and above what it copies in (1 MB); more areas than the pool keeps track of
+    geom = synth.Geometry(8, 2, 128)
+    shapes = [([37, 250], [60, 33]), ([16, 5, 90], [400, 290, 10]), ([300], [1]), ([40, 17], [1300, 901]), ([129], [80]), ([64, 64], [1100, 1000]),
+              ([700, 31], [20, 44]), ([3], [700])]
+    need = [[synth.pages_needed(p + e, 16) for p, e in zip(P, E)] for P, E in shapes]
+    i32 = lambda x: torch.tensor(np.asarray(x), dtype=torch.int32)
+    outs = []
+    for way in ("device", "host"):
+        dp = DualPool(geom, sum(map(sum, need)) + 4, seed=73, with_oracle=False)
+        batches = [Batch(dp, [p + e for p, e in zip(P, E)], uid0=100 * s) for s, (P, E) in enumerate(shapes)]
+        steps = []
+        for b, (P, E) in zip(batches, shapes):
+            b.write([(i, 0, P[i]) for i in range(len(P))])
+            ks, vs = zip(*[b.kv(i, P[i], P[i] + E[i]) for i in range(len(P))])
+            q = torch.cat([b.q(i, P[i], P[i] + E[i]) for i in range(len(P))]).contiguous()
+            arrays = (q, torch.cat(ks).contiguous(), torch.cat(vs).contiguous(), i32(np.concatenate([[0], np.cumsum(E)])),
+                      torch.from_numpy(b.block_tables()), i32(P), i32(E))
+            steps.append((arrays, (max(E), max(p + e for p, e in zip(P, E)), geom.scale)))
+        if way == "device":
+            for arrays, bounds in steps:
+                q = arrays[0]
+                out, lse = torch.empty_like(q), torch.empty((q.shape[0], 8), device="cuda")
+                ws = torch.empty(kvattn.attn_workspace_bytes(dp.pool, 8, arrays[5].numel(), int(q.shape[0]), bounds[1]), dtype=torch.uint8,
+                                 device="cuda")
+                kvattn.attn_extend_append(dp.pool, *[t.cuda() for t in arrays], *bounds, out, lse, ws)
+                torch.cuda.synchronize()
+                outs.append((synth.bf16_bits(out), lse.cpu().numpy()))
+            image = dp.device_image()
+        else:
+            host = [[_host(t.cpu(), pinned) for t in arrays] for arrays, _ in steps]
+            res = [(_host(torch.full(h[0].shape, float("nan"), dtype=torch.bfloat16), pinned), _host(torch.full((h[0].shape[0], 8), float("nan")), pinned))
+                   for h in host]
+            size = max(kvattn.attn_extend_host_staging_bytes(dp.pool, 8, h[5].numel(), h[0].shape[0], h[4].shape[1], bounds[1])
+                       for h, (_, bounds) in zip(host, steps))
+            staging = [torch.empty(size, dtype=torch.uint8, device="cuda") for _ in range(areas)]
+            torch.cuda.synchronize()
+            for s, (h, (_, bounds)) in enumerate(zip(host, steps)):
+                kvattn.attn_extend_host(dp.pool, *h, *bounds, *res[s], staging[s % areas])
+            torch.cuda.current_stream().synchronize()
+            for s, ((o, l), want) in enumerate(zip(res, outs)):
+                assert np.array_equal(synth.bf16_bits(o), want[0]) and np.array_equal(l.numpy(), want[1]), s
+            assert all(np.array_equal(x, y) for x, y in zip(dp.device_image(), image))
+        assert kvattn.kv_last_async_status(dp.pool) == kvattn.KV_OK
+        dp.close()
