@@ -5,14 +5,14 @@
 // the cluster through distributed shared memory: one kernel, no partial result in global memory, no combine kernel.
 // Where there are many short sequences instead, a CTA takes several pairs (pairs_per_cta).
 //
-// What bounds it: full batches, HBM (256 sequences of 1024-4096 tokens, 32/8 heads of 128: 373 us; the kernel it replaced,
+// What bounds it: full batches, HBM (256 sequences of 1024-4096 tokens, 32/8 heads of 128: 379 us; the kernel it replaced,
 // one warp per 1024-token chunk and a combine kernel behind it, took 418).  Small batches, the latency of a warp's
 // pages (about 0.7 us each, whatever the depth of its ring), so the sequence is spread over as many warps as are
-// resident: one sequence of 517 tokens 32.0 -> 3.8 us, of 16000 tokens 63 -> 15.6, 8 of 1000-4000 tokens 61.7 -> 18.8.
+// resident: one sequence of 517 tokens 32.0 -> 3.9 us, of 16000 tokens 63 -> 15.9, 8 of 1000-4000 tokens 61.7 -> 19.3.
 // kWarps x kStages: six warps with two page slots each, two CTAs per SM (D = 128).  4 x 3, 8 x 3, 12 x 2 and 4 x 6 were
 // measured on 20 batch shapes: twelve warps on an SM beat eight everywhere (a slot is refilled as soon as its page is
-// in registers, so two are enough), and two CTAs of six beat one of twelve on short contexts (128 sequences of 200-700:
-// 40.5 against 47.8 us) because one starts while the other ends.
+// in registers, so two are enough), and two CTAs of six beat one of twelve by a sixth on short contexts (128 sequences of
+// 200-700 tokens: 44 us) because one starts while the other ends.
 #include <math.h>
 
 #include "common.cuh"
@@ -370,15 +370,15 @@ static kv_status_t resident_clusters(int device, int i, int* n) {
 
 // CTAs per (sequence, KV head), from the host-side bounds alone.
 //  - As many as fit on the device at once: a second wave of clusters costs more than the shorter runs save (8 sequences
-//    of 1000-4000 tokens: 22.1 / 19.0 / 22.2 us with 2 / 4 / 8), but not more warps than about 3/2 of the sequence's
-//    pages (517 tokens: 4.6 / 4.2 / 4.4 us with 4 / 8 / 16).
+//    of 1000-4000 tokens: 24.2 / 19.3 / 21.8 us with 2 / 4 / 8), but not more warps than about 3/2 of the sequence's
+//    pages (517 tokens: 4.5 / 3.9 / 4.2 us with 4 / 8 / 16).
 //  - Where that leaves SMs idle, more, by what the last wave costs.  A wave of less than kFull of the CTAs the device
 //    holds is as slow as one of kFull (the memory is saturated with 0.65 of them at 128 dims, hardly with all at 64):
-//    32 x 5100 tokens, 64 dims: 49 / 51 / 42.6 us with 1 / 2 / 3, 64 x 3000: 77 / 70 / 69.6; 20 x 12000, 128 dims: 163 /
-//    179 / 151.  Every further CTA costs about 4 % at 192 pages.
+//    32 of 2600-5100 tokens, 64 dims: 51.9 / 52.9 / 45.8 us with 1 / 2 / 3, 64 of 1500-3000: 58.8 / 56.9 / 56.9; 20 of
+//    6000-12000, 128 dims: 130 / 132 / 117.  Every further CTA costs about 4 % at 192 pages.
 //  - Long sequences of different lengths are split even when the batch fills the device many times over, so that the last
-//    CTAs to finish hold less: 64 x 1024-4096 tokens 100.7 -> 94.1 us with 2, 32 x 3230-5100 88.6 -> 83.3; with runs below
-//    128 pages it costs (128 x 200-700: 40.5 against 54.4; 24 x 1000-3000, 64/8 heads: 39.0 against 42.8).
+//    CTAs to finish hold less: 64 x 1024-4096 tokens 113.8 -> 104.7 us with 2, 32 x 3230-5100 92.5 -> 88.0; with runs below
+//    128 pages it costs (128 x 200-700: 44.0 against 56.4; 24 x 1000-3000, 64/8 heads: 39.1 against 39.9).
 template <int D>
 static kv_status_t decode_splits(const kv_pool_t* p, int batch, int max_ctx_len, int* splits) {
   const int64_t units = (int64_t)batch * p->n_kv_heads;
@@ -414,10 +414,10 @@ static kv_status_t decode_splits(const kv_pool_t* p, int batch, int max_ctx_len,
 // (sequence, KV head) pairs per CTA where no pair is spread over a cluster: many short sequences are bound by the starts,
 // barriers and merges of their CTAs, so a CTA takes as many pairs as bring them all on the device at once, one to three
 // warps for a pair, while a warp's run stays short: 16 pages, 8 where there is a second wave all the same.  Us with 1 / 2 /
-// 3 / 6 pairs (128 dims, 296 CTAs resident): 72 x 8 pairs of up to 6 pages 9.4 / 6.7 / 8.0 / 10.2, 103 x 8 of 7 15.4 / 13.9 /
-// 10.0 / 11.9, 222 x 8 of 8 32.1 / 25.1 / 23.0 / 20.3, 75 x 8 of 32 32.4 / 33.8 / 29.9 / 35.8; second waves: 251 x 8 of 12
-// 44.7 / 36.3 / 35.7 / 39.3, 149 x 8 of 37 60.4 / 62.5 / 60.6 / 63.5; 64 dims (444 resident): 101 x 8 of 18 13.5 / 10.6 / 12.4 /
-// 16.8, 230 x 8 of 48 60.4 / 62.6 / 62.3 / 60.6.
+// 3 / 6 pairs (lengths from two thirds of the stated pages; 128 dims, 296 CTAs resident): 72 x 8 pairs of 6 pages 10.2 / 8.5 / 8.8 /
+// 11.8, 103 x 8 of 7 15.5 / 15.8 / 11.8 / 13.7, 222 x 8 of 8 30.2 / 27.3 / 25.2 / 22.1, 75 x 8 of 32 27.6 / 30.7 / 27.3 / 34.5; second
+// waves: 251 x 8 of 12 37.9 / 37.6 / 36.9 / 40.0, 149 x 8 of 37 52.5 / 53.2 / 56.0 / 58.6; 64 dims (444 resident): 101 x 8 of 18
+// 14.6 / 12.6 / 13.8 / 20.8, 230 x 8 of 48 52.3 / 55.1 / 57.6 / 57.6.
 template <int D>
 static kv_status_t pairs_per_cta(const kv_pool_t* p, int64_t units, int max_ctx_len, int* n) {
   int resident;
@@ -431,10 +431,10 @@ static kv_status_t pairs_per_cta(const kv_pool_t* p, int64_t units, int max_ctx_
 }
 
 // Whether a warp has so few pages that it should load them straight into registers: a copy into a slot, its barrier and the
-// read back cost 0.4 to 0.7 us more than a load, and with a page or two per warp there is nothing to overlap them with.
-// Ring / registers at so many pages per warp: 128 dims 4.7 / 4.2 us (1.0), 5.7 / 5.5 (1.8), 6.0 / 5.3 (1.95), 7.2 / 7.3 (2.1),
-// 7.3 / 8.0 (3.1), with more CTAs than are resident 24.2 / 23.3 (1.0), 17.4 / 17.8 (1.3); 64 dims 4.6 / 4.1 (0.8), 8.1 / 6.9
-// (1.3), 6.5 / 5.9 (2.75), 14.9 / 16.0 (3.7).
+// read back cost 0.3 to 0.6 us more than a load, and with a page or two per warp there is nothing to overlap them with.
+// Ring / registers at so many pages per warp: 128 dims 4.2 / 3.9 us (1.0), 6.0 / 5.4 (1.95), 6.6 / 5.9 (2.1), 7.1 / 7.3 (2.1, 8
+// sequences), 7.8 / 8.0 (3.1), with more CTAs than are resident 45.6 / 47.1 (6.0), 97.8 / 114.1 (6.0); 64 dims 4.6 / 4.2 (0.8), 5.4 /
+// 5.1 (1.6), 6.6 / 6.0 (2.75), 10.6 / 11.2 (4.2).
 static bool few_pages(const kv_pool_t* p, int64_t blocks, int warps, int max_ctx_len) {
   const double pages = (double)(max_ctx_len + kPageSize - 1) / kPageSize / warps;
   return pages <= (p->head_dim == 64 ? 2.75 : blocks <= 2 * sm_count_of(p->device) ? 2.0 : 1.0);

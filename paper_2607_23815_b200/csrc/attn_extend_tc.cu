@@ -1517,8 +1517,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
 
 // Merges the chunks of the items that the cuts between the spans went through.  Block (s - 1) * kCombineSlices + slice:
 // the item of which cut s is the first, 256 / kCombineSlices of its rows in turns of 32; warp w takes the dims 8w .. 8w + 7,
-// its lanes the rows.  Bound by latency and launch (a few MB through L2), so the blocks, most of which have nothing to do,
-// are to be resident at once: 40 registers.
+// its lanes the rows.  Bound by latency and launch (a few MB through L2), so as many blocks as possible, most of which have
+// nothing to do, are to be resident: three of 40 registers on an SM at 128 dims (588 blocks of 148 spans: a round and a third).
 constexpr int kCombineSlices = 4;
 template <int D>
 __global__ void __launch_bounds__(D * 4, 384 / D) span_combine_kernel(const SpanArgs a, int n_q_heads, int group, int lg,
@@ -1891,7 +1891,8 @@ kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const i
   } else if (phase == 2) {
     // the plan is in the workspace already
   } else if (app != nullptr && app->total_new > 0) {
-    // plan block + append blocks (32 warps each, one warp per token, all blocks resident at once)
+    // plan block + append blocks (32 warps each, one warp per token).  A block's 1024 threads take 64 registers each, so one block
+    // is on an SM at a time and a long suffix runs in two rounds; the attention kernel can start once the last block has.
     const int64_t want = ((int64_t)app->total_new + 31) / 32;
     const int64_t cap = 2 * (int64_t)sm_count_of(p->device) - 1;
     const int blocks = (int)(want < cap ? want : cap);

@@ -335,8 +335,8 @@ def attn_decode(pool: Pool, q, block_tables, ctx_lens, max_ctx_len, scale, out, 
 
 
 def attn_decode_static(pool: Pool, q, block_tables, ctx_lens, max_ctx_len, scale, out, lse, stream=None):
-    """attn_decode for callers that cannot allocate: no workspace argument, the scratch is a fixed array inside
-    the library (see the header for the limit and the sharing rules)."""
+    """attn_decode for callers that cannot allocate: the same launch without a workspace argument (see the header for the
+    limit on the batch)."""
     _check(lib().attn_decode_static(pool.handle, _dev_ptr(q), q.shape[1], _dev_ptr(block_tables),
                                     block_tables.shape[1], _dev_ptr(ctx_lens), q.shape[0], max_ctx_len, float(scale),
                                     _dev_ptr(out), _dev_ptr(lse), _stream(stream)), "attn_decode_static")

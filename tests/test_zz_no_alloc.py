@@ -2,10 +2,11 @@
 
 Some users of this library run where cudaMalloc is off the table: a plugin that only gets the buffers its host
 hands it, a region a framework has memory-planned or is capturing, a serving process that freezes its allocator
-after start-up.  They cannot build the workspace attn_decode wants, so the library carries a fixed scratch array
-for them.  The test drives the entry point through the C ABI twice in a row (the array keeps the first call's
-contents, and the second call must not care), asks for the same bits as the regular entry point, compares both
-with the oracle and watches the free device memory across the call.  It sits in a file that sorts last so that a run stopping at the first failure has already run everything else.
+after start-up.  They cannot build the workspace attn_decode wants; the decode kernel keeps its partial results on chip,
+so for them the same launch is there without the argument.  The test drives the entry point through the C ABI several
+times in a row, asks for the same bits as the regular entry point, compares both with the oracle and watches the free
+device memory across the call.  It sits in a file that sorts last so that a run stopping at the first failure has already
+run everything else.
 """
 import numpy as np
 import pytest
@@ -19,8 +20,8 @@ pytestmark = pytest.mark.gpu
 
 
 def _decode_both(dp, batch, ctx):
-    """The same batch through attn_decode (caller's workspace) and attn_decode_static (the library's array); the
-    free device memory is read around the second call: the static entry point must not change it."""
+    """The same batch through attn_decode (with a workspace) and attn_decode_static (without); the free device memory
+    is read around the second call: the static entry point must not change it."""
     g, dev = dp.geom, dp.device
     q = torch.cat([batch.q(i, max(c - 1, 0), max(c - 1, 0) + 1) for i, c in enumerate(ctx)]).contiguous()
     bt_np = batch.block_tables()
@@ -50,18 +51,18 @@ def _check_case(dp, batch, ctx, warm):
     res = {"o": got_o.float().cpu().numpy().astype(np.float64), "lse": got_l.cpu().numpy().astype(np.float64),
            "o_ref": o_ref, "lse_ref": l_ref}
     assert_close(res, "attn_decode_static")
-    if warm:   # (the first call on a device may make the driver load the module that holds the array)
+    if warm:   # (the first call on a device may make the driver load the kernels)
         assert grew == 0, f"free device memory shrank by {grew} bytes across attn_decode_static"
 
 
 def test_static_scratch_decode_matches_the_workspace_version_twice_in_a_row():
     geom = synth.Geometry(32, 8, 128)
     dp = DualPool(geom, 1024, seed=909)
-    # first call: long contexts (several split-KV chunks per row fill the shared array) ...
+    # first call: long contexts ...
     ctx_a = [4096, 1300, 513, 2049, 17]
     a = Batch(dp, ctx_a)
     a.write([(i, 0, c) for i, c in enumerate(ctx_a)])
-    # ... second call: other sequences with fewer chunks, so stale partials of the first call lie next to its own
+    # ... second call: other sequences, fewer and shorter
     ctx_b = [700, 1025, 90, 3000]
     b = Batch(dp, ctx_b, uid0=50)
     b.write([(i, 0, c) for i, c in enumerate(ctx_b)])
@@ -73,8 +74,7 @@ def test_static_scratch_decode_matches_the_workspace_version_twice_in_a_row():
 
 
 def test_static_scratch_short_contexts_and_empty_rows():
-    # contexts of at most one chunk need no scratch at all (the kernel writes the result directly), and rows with a
-    # context length of zero or less get O = 0, LSE = -inf; both through the static entry point
+    # short contexts, and rows with a context length of zero or less (O = 0, LSE = -inf) through the static entry point
     geom = synth.Geometry(8, 2, 128)
     dp = DualPool(geom, 512, seed=911)
     ctx_a = [1024, 1, 0, 513, 16]
