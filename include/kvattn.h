@@ -209,8 +209,9 @@ kv_status_t attn_extend_planned(kv_pool_t* pool, const void* q, int n_q_heads, c
  * to the call until the stream has passed it.  The copies run on copy streams of the pool, ordered against the
  * kernels (on `stream`) by events, and the stream waits for the copy out; with two staging areas used in turn
  * one step's copies overlap its neighbour's kernels.  The copy in starts at once: the host inputs must be
- * final when the call is made.  At most four staging areas are tracked at a time.  Errors as for kv_append and attn_extend, KV_ERR_WORKSPACE for a staging area that is too
- * small.  (In the paper the requests reach the engine from host-side operators, Section 3; the paper has
+ * final when the call is made.  At most four staging areas are tracked at a time.  Errors as for kv_append and
+ * attn_extend, KV_ERR_WORKSPACE for a staging area that is too small (one without room for partial results of cut
+ * items, but for everything else, is taken).  (In the paper the requests reach the engine from host-side operators, Section 3; the paper has
  * no counterpart of this exact call.) */
 size_t attn_extend_host_staging_bytes(const kv_pool_t* pool, int n_q_heads, int batch, int total_q, int max_pages,
                                       int max_total_len);
