@@ -27,6 +27,7 @@
 // tensor memory and returns.
 #include <math.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include <cuda.h>  // CUtensorMap and its enums (types only: the encoder is looked up at run time)
@@ -340,14 +341,14 @@ __global__ void __launch_bounds__(1024) extend_tc_plan_kernel(const PlanArgs pa)
 // Prologue of the fused append + extend call: block 0 builds the plan while the other blocks scatter the suffix K/V
 // rows into their pages (one warp per token), so the step has one small kernel in front of the attention kernel
 // instead of two in a row, and the attention kernel's launch and set-up overlap it.
-__global__ void __launch_bounds__(1024) extend_prologue_kernel(const PlanArgs pa, const PoolView pool, const AppendArgs ap) {
+__global__ void __launch_bounds__(1024) extend_prologue_kernel(const PlanArgs pa, const PoolView pool, const AppendArgs ap, int tokens_per_block) {
   dependency_wait();
   launch_dependents();
   if (blockIdx.x == 0) {
     plan_body(pa);
   } else {
-    const int warps_per_block = blockDim.x >> 5;
-    append_tokens<4>(pool, ap, (blockIdx.x - 1) * warps_per_block + (threadIdx.x >> 5), (gridDim.x - 1) * warps_per_block);
+    const int warp = threadIdx.x >> 5;
+    if (warp < tokens_per_block) append_tokens<4>(pool, ap, (blockIdx.x - 1) * tokens_per_block + warp, (gridDim.x - 1) * tokens_per_block);
   }
 }
 
@@ -1823,7 +1824,7 @@ kv_status_t launch_extend_combine(kv_pool_t* p, int n_q_heads, int batch, int to
   const auto kernel = p->head_dim == 128 ? span_combine_kernel<128> : span_combine_kernel<64>;
   const unsigned blocks = (unsigned)((a.n_spans - 1) * kCombineSlices), threads = (unsigned)p->head_dim * 4;
   if (early) {
-    KV_CUDA_OK(launch_early(kernel, blocks, threads, st, a, n_q_heads, G, lg, (__nv_bfloat16*)out, lse));
+    KV_CUDA_OK(launch_early(kernel, blocks, threads, 0, st, a, n_q_heads, G, lg, (__nv_bfloat16*)out, lse));
   } else {
     kernel<<<blocks, threads, 0, st>>>(a, n_q_heads, G, lg, (__nv_bfloat16*)out, lse);
     KV_CUDA_OK(cudaGetLastError());
@@ -1885,21 +1886,29 @@ kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const i
     if (app != nullptr && app->total_new > 0) {
       const int64_t want = ((int64_t)app->total_new + 31) / 32;
       const int64_t cap = 2 * (int64_t)sm_count_of(p->device);
-      KV_CUDA_OK(launch_early(append_prologue_kernel, (unsigned)(want < cap ? want : cap), 1024, st, p->view(), *app));
+      const AppendSpread sp = append_spread(app->total_new, sm_count_of(p->device));
+      if (sp.blocks > 0) {
+        static std::atomic<bool> allowed[kMaxDevices];
+        KV_CUDA_OK(allow_smem((const void*)append_prologue_kernel, kAppendSpreadSmem, allowed, p->device));
+        KV_CUDA_OK(launch_early(append_prologue_kernel, (unsigned)sp.blocks, (unsigned)sp.warps * 32, (size_t)sp.smem, st, p->view(), *app));
+      } else {
+        KV_CUDA_OK(launch_early(append_prologue_kernel, (unsigned)(want < cap ? want : cap), 1024, 0, st, p->view(), *app));
+      }
       count_launch();
     }
   } else if (phase == 2) {
     // the plan is in the workspace already
   } else if (app != nullptr && app->total_new > 0) {
-    // plan block + append blocks (32 warps each, one warp per token).  A block's 1024 threads take 64 registers each, so one block
-    // is on an SM at a time and a long suffix runs in two rounds; the attention kernel can start once the last block has.
-    const int64_t want = ((int64_t)app->total_new + 31) / 32;
-    const int64_t cap = 2 * (int64_t)sm_count_of(p->device) - 1;
-    const int blocks = (int)(want < cap ? want : cap);
-    KV_CUDA_OK(launch_early(extend_prologue_kernel, (unsigned)(1 + blocks), 1024, st, pa, p->view(), *app));
+    // Plan block + append blocks, one warp per token.  A block's 1024 threads take 64 registers each, so one block is on an SM at a
+    // time: up to 32 tokens per SM the tokens are spread over as many blocks as there are SMs (28 sequences of 15-18 tokens behind
+    // 64-95 18.0 -> 15.7 us, 33 of 29-31 behind 1100, 8/8 heads, 48.5 -> 46.3); a longer suffix runs in rounds of 32 and the
+    // attention kernel can start once the last block has.
+    const int64_t sms = sm_count_of(p->device), total = app->total_new, per_block = std::min<int64_t>((total + sms - 2) / (sms - 1), 32);
+    const int64_t want = (total + per_block - 1) / per_block, cap = 2 * sms - 1;
+    KV_CUDA_OK(launch_early(extend_prologue_kernel, (unsigned)(1 + (want < cap ? want : cap)), 1024, 0, st, pa, p->view(), *app, (int)per_block));
     count_launch();
   } else {
-    KV_CUDA_OK(launch_early(extend_tc_plan_kernel, 1, 1024, st, pa));
+    KV_CUDA_OK(launch_early(extend_tc_plan_kernel, 1, 1024, 0, st, pa));
     count_launch();
   }
   if (phase == 1) return KV_OK;

@@ -54,10 +54,11 @@ inline void count_launch(int n = 1) { g_launches.fetch_add(n, std::memory_order_
 // Launches a kernel that may start while the kernel in front of it in the stream still runs (programmatic dependent
 // launch).  The kernel waits for that one itself (ptx::dependency_wait) before it touches anything.
 template <typename... Params, typename... Args>
-inline cudaError_t launch_early(void (*kernel)(Params...), unsigned blocks, unsigned threads, cudaStream_t st, Args... args) {
+inline cudaError_t launch_early(void (*kernel)(Params...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(blocks);
   cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -68,6 +69,15 @@ inline cudaError_t launch_early(void (*kernel)(Params...), unsigned blocks, unsi
 }
 
 constexpr int kMaxDevices = 64;
+
+// Allows a kernel `smem` bytes of dynamic shared memory on a device, once (the attribute belongs to the function on one device).
+inline cudaError_t allow_smem(const void* kernel, int smem, std::atomic<bool> (&done)[kMaxDevices], int device) {
+  if (device < 0 || device >= kMaxDevices) return cudaErrorInvalidDevice;
+  if (done[device].load(std::memory_order_acquire)) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess) done[device].store(true, std::memory_order_release);
+  return e;
+}
 // Multiprocessors of the given device (asked once per device).
 int sm_count_of(int device);
 

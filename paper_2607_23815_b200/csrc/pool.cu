@@ -396,7 +396,14 @@ kv_status_t kv_append(kv_pool_t* p, const void* k_new, const void* v_new, const 
   // (rows of many times the L2: fewer tokens on an SM at a time, see append_kernel)
   const bool bulk = (int64_t)total_new * chunks * 32 >= 320000000;
   const auto kernel = chunks <= 64 ? append_kernel<2> : chunks <= 128 && !bulk ? append_kernel<4> : append_kernel<8>;
-  KV_CUDA_OK(launch_early(kernel, blocks, 256, (cudaStream_t)stream, p->view(), a));
+  const AppendSpread sp = append_spread(total_new, sm_count_of(p->device));
+  if (sp.blocks > 0) {
+    static std::atomic<bool> allowed[3][kMaxDevices];
+    KV_CUDA_OK(allow_smem((const void*)kernel, kAppendSpreadSmem, allowed[chunks <= 64 ? 0 : chunks <= 128 ? 1 : 2], p->device));
+    KV_CUDA_OK(launch_early(kernel, (unsigned)sp.blocks, (unsigned)sp.warps * 32, (size_t)sp.smem, (cudaStream_t)stream, p->view(), a));
+  } else {
+    KV_CUDA_OK(launch_early(kernel, blocks, 256, 0, (cudaStream_t)stream, p->view(), a));
+  }
   count_launch();
   return KV_OK;
 }
