@@ -101,3 +101,12 @@ def test_back_to_back_calls_that_depend_on_each_other():
         for o, r in zip(got, ref[1:]):
             assert torch.equal(o.view(torch.int16), r.view(torch.int16))
     dp.close()
+
+
+@pytest.mark.parametrize("d", [128, 64])
+@pytest.mark.parametrize("ctx", [16, 700])
+@pytest.mark.parametrize("batch", [1, 18, 19, 37, 38])
+def test_one_or_two_blocks_per_sm(batch, ctx, d):
+    # batches of about as many blocks as there are SMs, and twice as many (148 on a B200, 8 KV heads), of one CTA per pair and of clusters
+    rng = np.random.default_rng(batch)
+    _check(synth.Geometry(16, 8, d), [ctx] + [int(x) for x in rng.integers(1, ctx + 1, size=batch - 1)], seed=850 + batch)
