@@ -1117,7 +1117,24 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
     Item it;
     for (int round = 0; ok && fetch(round, it); ++round) {
       sched_release(round);
-      if (CLUSTER && a.cl_splits > 1) continue;  // the softmax warps hand the partial results over
+      if (CLUSTER && a.cl_splits > 1) {
+        // The softmax warps hand the partial results over; the second half of the first tile's dims is left to these warps
+        // (one sequence of 37 tokens, 128 of its 148 rows in that tile: 14.39 -> 14.16 us).
+        if (it.n_kv[0] == 0) continue;
+        ok = mbar_wait(smem_u32(&sm.o_full[0]), 0, abortp);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        tc_fence_after_sync();
+        float* dst = a.span.part_o + (((int64_t)blockIdx.x * (D / 8) + D / 16) * a.span.rows + m) * 8;
+#pragma unroll 1
+        for (int c = D / 64; c < D / 32; ++c, dst += (int64_t)a.span.rows * 32) {
+          uint32_t orow[32];
+          tmem_ld32(lane_base + 256 + c * 32, orow);
+          tmem_wait_ld();
+          if (m < sm.cl_unit.x) store_part8x4(dst, a.span.rows, orow);
+        }
+        continue;
+      }
       if (it.ld_tiles == 0) continue;
 #pragma unroll 1
       for (int t = 0; t < 2; ++t) {
@@ -1423,7 +1440,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
         tc_fence_after_sync();
         float* dst = a.span.part_o + ((int64_t)blockIdx.x * (D / 8) * a.span.rows + row) * 8;
 #pragma unroll 1
-        for (int c = 0; c < D / 32; ++c, dst += (int64_t)a.span.rows * 32) {
+        for (int c = 0; c < (t == 0 ? D / 64 : D / 32); ++c, dst += (int64_t)a.span.rows * 32) {
           uint32_t orow[32];
           tmem_ld32(o_addr + c * 32, orow);
           tmem_wait_ld();
@@ -1437,8 +1454,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
       const int r_begin = u.x * rank / splits, cnt = u.x * (rank + 1) / splits - r_begin;
       auto finish = [&](auto n) {
         // Item i: eight dims of a row; neighbouring lanes take neighbouring rows.  As many items of a thread at a time as make
-        // sixteen loads: the wait for L2 is paid once.
-        constexpr int N = decltype(n)::value, ITEMS = 16 / N;
+        // sixteen loads: the wait for L2 is paid once.  From six chunks on one item: the code runs once per launch and is fetched as
+        // it runs, so its length counts for more (with the weights by ex2.approx, whose error is that of exp2f, one sequence of
+        // 37 tokens behind 1483 14.16 -> 13.77 us, 7 of 31-38 behind 238-459 16.5 -> 16.2).
+        constexpr int N = decltype(n)::value, ITEMS = N >= 6 ? 1 : 16 / N;
         const int items = cnt * (D / 8);
         for (int base = tid; base < items; base += 256 * ITEMS) {
           float2 ml[ITEMS][N];
@@ -1470,7 +1489,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
 #pragma unroll
             for (int c = 0; c < N; ++c) {
               if (ml[k][c].y == 0.f) continue;  // (no step of the row's tile, or no key that the row sees: not written)
-              const float w = exp2f(ml[k][c].x - mx);
+              float w;
+              asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(w) : "f"(ml[k][c].x - mx));
               sum += w * ml[k][c].y;
 #pragma unroll
               for (int e = 0; e < 4; ++e) o[e] = __ffma2_rn(make_float2(x[k][c][2 * e], x[k][c][2 * e + 1]), make_float2(w, w), o[e]);
