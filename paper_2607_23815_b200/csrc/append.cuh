@@ -4,6 +4,7 @@
 
 #include "common.cuh"
 #include "sm100_ptx.cuh"
+#include "spread.h"
 
 namespace kvattn {
 

@@ -27,7 +27,6 @@
 // tensor memory and returns.
 #include <math.h>
 
-#include <algorithm>
 #include <type_traits>
 
 #include <cuda.h>  // CUtensorMap and its enums (types only: the encoder is looked up at run time)
@@ -1931,9 +1930,9 @@ kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const i
     // time: up to 32 tokens per SM the tokens are spread over as many blocks as there are SMs (28 sequences of 15-18 tokens behind
     // 64-95 18.0 -> 15.7 us, 33 of 29-31 behind 1100, 8/8 heads, 48.5 -> 46.3); a longer suffix runs in rounds of 32 and the
     // attention kernel can start once the last block has.
-    const int64_t sms = sm_count_of(p->device), total = app->total_new, per_block = std::min<int64_t>((total + sms - 2) / (sms - 1), 32);
-    const int64_t want = (total + per_block - 1) / per_block, cap = 2 * sms - 1;
-    KV_CUDA_OK(launch_early(extend_prologue_kernel, (unsigned)(1 + (want < cap ? want : cap)), 1024, 0, st, pa, p->view(), *app, (int)per_block));
+    const int sms = sm_count_of(p->device), per_block = prologue_tokens(app->total_new, sms);
+    const int64_t want = ((int64_t)app->total_new + per_block - 1) / per_block, cap = 2 * (int64_t)sms - 1;
+    KV_CUDA_OK(launch_early(extend_prologue_kernel, (unsigned)(1 + (want < cap ? want : cap)), 1024, 0, st, pa, p->view(), *app, per_block));
     count_launch();
   } else {
     KV_CUDA_OK(launch_early(extend_tc_plan_kernel, 1, 1024, 0, st, pa));
