@@ -111,24 +111,4 @@ __device__ __forceinline__ void append_tokens(const PoolView& pool, const Append
   }
 }
 
-// How an append's blocks of at most eight warps, a token each, are spread over the SMs.  They are launched early and wait for the kernel
-// in front, and the SMs that one leaves free, or frees first, would take all of them, as many as fit: the rows of a hundred tokens then
-// go through three or four SMs.  So a small batch has one block per SM, of as few warps as that takes, a larger one up to three, and
-// a block asks for so much shared memory, which it does not use, that no more of them fit.  Whole calls, us (32/8 heads of 128 where
-// not stated): 1 sequence of 37 tokens appended and extended 16.0 -> 14.4; 4 layers of 9 sequences, 500 tokens each, 171 -> 159 (165
-// with 40 KB a block, which lets five of them onto an SM); 2 extends beside 23 decodes 34.1 -> 26.7; 39 beside 49, 8/8 heads, 54.0 ->
-// 43.5; 1260 tokens in a mixed step, 64 dims, 32.6 -> 32.1 and 1500 43.2 -> 39.3 (two blocks per SM).  The same tokens through bulk
-// copies into shared memory, a block's warps storing them from there, were slower: 15.1, 161, 28.6, 49.3, 34.2, 42.5.
-struct AppendSpread {
-  int blocks, warps, smem;
-};
-constexpr int kAppendSpreadMax = 3;  // blocks per SM; batches of more tokens fill the device anyway
-constexpr int kAppendSpreadSmem = 120 * 1024;
-inline AppendSpread append_spread(int total_new, int sms) {
-  const int64_t per_sm = ((int64_t)total_new + sms - 1) / sms, k = (per_sm + 7) / 8;
-  if (k > kAppendSpreadMax) return {0, 0, 0};
-  const int warps = k == 1 ? (int)per_sm : 8;
-  return {(total_new + warps - 1) / warps, warps, k == 1 ? kAppendSpreadSmem : k == 2 ? 80 * 1024 : 58 * 1024};
-}
-
 }  // namespace kvattn

@@ -399,7 +399,7 @@ kv_status_t kv_append(kv_pool_t* p, const void* k_new, const void* v_new, const 
   const AppendSpread sp = append_spread(total_new, sm_count_of(p->device));
   if (sp.blocks > 0) {
     static std::atomic<bool> allowed[3][kMaxDevices];
-    KV_CUDA_OK(allow_smem((const void*)kernel, kAppendSpreadSmem, allowed[chunks <= 64 ? 0 : chunks <= 128 ? 1 : 2], p->device));
+    KV_CUDA_OK(allow_smem((const void*)kernel, spread_smem(1), allowed[chunks <= 64 ? 0 : chunks <= 128 ? 1 : 2], p->device));
     KV_CUDA_OK(launch_early(kernel, (unsigned)sp.blocks, (unsigned)sp.warps * 32, (size_t)sp.smem, (cudaStream_t)stream, p->view(), a));
   } else {
     KV_CUDA_OK(launch_early(kernel, blocks, 256, 0, (cudaStream_t)stream, p->view(), a));

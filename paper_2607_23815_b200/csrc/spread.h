@@ -5,6 +5,32 @@
 
 namespace kvattn {
 
+// Dynamic shared memory of a block that lets `n` of them onto an SM and no more (228 KB, of which every block takes one more).
+constexpr int spread_smem(int n) { return 228 * 1024 / (n + 1) / 128 * 128; }
+
+struct AppendSpread {
+  int blocks, warps;  // blocks == 0: the tokens are not spread
+  int smem;
+};
+
+// An append's blocks of at most eight warps, a token each.  They are launched early and wait for the kernel in front, and the SMs that
+// one leaves free, or frees first, would take all of them, as many as fit: the rows of a hundred tokens then go through three or four
+// SMs.  So up to 24 tokens per SM a block asks for so much shared memory, which it does not use, that one, two or three of them are
+// on an SM, and has no more warps than it takes to hold an SM's share of the tokens in that many.  (Eight warps in each of two or
+// three blocks would hold 16 tokens on half of the SMs where every SM's share is 9.)  Whole calls, us (32/8 heads of 128 where not
+// stated): 1 sequence of 37 tokens appended and extended 16.0 -> 14.4; 4 layers of 9 sequences, 500 tokens each, 171 -> 159 (165 with
+// 40 KB a block, which lets five of them onto an SM); 2 extends beside 23 decodes 34.1 -> 26.7; 39 beside 49, 8/8 heads, 54.0 -> 43.5.
+// An append and a decode of 9 sequences, not spread / eight warps / as many as it takes: 1184 tokens (one block of eight per SM) 13.2 /
+// 11.1, 1185 13.2 / 11.8 / 11.3, 1260 13.2 / 11.8 / 11.4, 1500 13.2 / 11.8 / 11.5, 2000 13.6 / 12.2 / 12.0, 2369 13.8 / 13.0 / 12.7, 2800
+// 13.9 / 13.3 / 13.1, 3552 14.6 / 14.0.  The same tokens through bulk copies into shared memory, a block's warps storing them from
+// there, were slower (the first four calls: 15.1, 161, 28.6, 49.3).
+inline AppendSpread append_spread(int total_new, int sms) {
+  const int64_t per_sm = ((int64_t)total_new + sms - 1) / sms, k = (per_sm + 7) / 8;  // tokens and blocks of an SM
+  if (k > 3) return {0, 0, 0};
+  const int64_t warps = (per_sm + k - 1) / k;
+  return {(int)((total_new + warps - 1) / warps), (int)warps, spread_smem((int)k)};
+}
+
 // Tokens of a block of the prologue that builds the plan beside the append: one block takes the plan, the others share the tokens,
 // up to 32 (the block's warps) each.
 inline int prologue_tokens(int total_new, int sms) {

@@ -14,6 +14,8 @@ def lib(tmp_path_factory):
     gxx = shutil.which("g++") or pytest.skip("no g++")
     d = tmp_path_factory.mktemp("spread")
     (d / "shim.cpp").write_text('#include "spread.h"\n'
+                                'extern "C" void append_spread(int total, int sms, int* r) {\n'
+                                '  const kvattn::AppendSpread a = kvattn::append_spread(total, sms); r[0] = a.blocks; r[1] = a.warps; r[2] = a.smem;\n}\n'
                                 'extern "C" int prologue_tokens(int total, int sms) { return kvattn::prologue_tokens(total, sms); }\n')
     subprocess.run([gxx, "-std=c++17", "-shared", "-fPIC", f"-I{CSRC}", str(d / "shim.cpp"), "-o", str(d / "shim.so")], check=True)
     return ctypes.CDLL(str(d / "shim.so"))
@@ -24,3 +26,27 @@ def lib(tmp_path_factory):
 def test_tokens_of_a_prologue_block(lib, total, sms):
     n, others = lib.prologue_tokens(total, sms), max(sms - 1, 1)
     assert n == min(-(-total // others), 32)
+
+
+def _fit(smem):
+    return 228 * 1024 // (smem + 1024)                           # blocks of that much shared memory on an SM
+
+
+def _spread(lib, total, sms):
+    r = (ctypes.c_int * 3)()
+    lib.append_spread(total, sms, r)
+    return list(r)
+
+
+@pytest.mark.parametrize("sms", [1, 147, 148])
+def test_every_token_has_a_warp_and_no_sm_more_than_its_share(lib, sms):
+    for total in sorted({1, 2, 3, 37} | {k * sms + d for k in range(1, 26) for d in (-1, 0, 1)} - {0}):
+        blocks, warps, smem = _spread(lib, total, sms)
+        share = -(-total // sms)
+        if blocks == 0:
+            assert share > 24
+            continue
+        n = _fit(smem)
+        assert (blocks - 1) * warps < total <= blocks * warps and 1 <= warps <= 8
+        assert blocks <= n * sms                                 # all of them are resident at once
+        assert n * warps < share + n, (total, n, warps)          # however they are placed: an SM's share, rounded up to whole blocks
