@@ -4,7 +4,6 @@
 
 #include "common.cuh"
 #include "sm100_ptx.cuh"
-#include "spread.h"
 
 namespace kvattn {
 

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "../../include/kvattn.h"
+#include "spread.h"
 
 namespace kvattn {
 
@@ -70,13 +71,13 @@ inline cudaError_t launch_early(void (*kernel)(Params...), unsigned blocks, unsi
 
 constexpr int kMaxDevices = 64;
 
-// Allows a kernel `smem` bytes of dynamic shared memory on a device, once (the attribute belongs to the function on one device).
-inline cudaError_t allow_smem(const void* kernel, int smem, std::atomic<bool> (&done)[kMaxDevices], int device) {
-  if (device < 0 || device >= kMaxDevices) return cudaErrorInvalidDevice;
-  if (done[device].load(std::memory_order_acquire)) return cudaSuccess;
-  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e == cudaSuccess) done[device].store(true, std::memory_order_release);
-  return e;
+// Whether a kernel may have `smem` bytes of dynamic shared memory on a device (the attribute belongs to the function on one device).
+inline bool allow_smem(const void* kernel, int smem, std::atomic<bool> (&done)[kMaxDevices], int device) {
+  return once_per_device(done, device, [&] {
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess) return true;
+    cudaGetLastError();
+    return false;
+  });
 }
 // Multiprocessors of the given device (asked once per device).
 int sm_count_of(int device);

@@ -101,6 +101,14 @@ static int grid_for(const kv_pool_t* p, int64_t work_items, int threads) {
   return (int)blocks;
 }
 
+template <int N>
+static cudaError_t launch_append(const kv_pool_t* p, const AppendArgs& a, const AppendSpread& sp, cudaStream_t st) {
+  static std::atomic<bool> allowed[kMaxDevices];
+  if (sp.blocks > 0 && allow_smem((const void*)append_kernel<N>, spread_smem(1), allowed, p->device))
+    return launch_early(append_kernel<N>, (unsigned)sp.blocks, (unsigned)sp.warps * 32, (size_t)sp.smem, st, p->view(), a);
+  return launch_early(append_kernel<N>, (unsigned)grid_for(p, (int64_t)a.total_new * 32, 256), 256, 0, st, p->view(), a);  // one warp per token
+}
+
 }  // namespace kvattn
 
 using namespace kvattn;
@@ -391,19 +399,11 @@ kv_status_t kv_append(kv_pool_t* p, const void* k_new, const void* v_new, const 
   if (!on_pool_device(p)) return KV_ERR_INVALID;
   const AppendArgs a{(const uint4*)k_new, (const uint4*)v_new, cu_new, start_pos, seg_row, block_tables, max_pages, n_segments,
                      total_new};
-  const unsigned blocks = (unsigned)grid_for(p, (int64_t)total_new * 32, 256);  // one warp per token
   const int chunks = p->n_kv_heads * (p->head_dim >> 3);
   // (rows of many times the L2: fewer tokens on an SM at a time, see append_kernel)
   const bool bulk = (int64_t)total_new * chunks * 32 >= 320000000;
-  const auto kernel = chunks <= 64 ? append_kernel<2> : chunks <= 128 && !bulk ? append_kernel<4> : append_kernel<8>;
-  const AppendSpread sp = append_spread(total_new, sm_count_of(p->device));
-  if (sp.blocks > 0) {
-    static std::atomic<bool> allowed[3][kMaxDevices];
-    KV_CUDA_OK(allow_smem((const void*)kernel, spread_smem(1), allowed[chunks <= 64 ? 0 : chunks <= 128 ? 1 : 2], p->device));
-    KV_CUDA_OK(launch_early(kernel, (unsigned)sp.blocks, (unsigned)sp.warps * 32, (size_t)sp.smem, (cudaStream_t)stream, p->view(), a));
-  } else {
-    KV_CUDA_OK(launch_early(kernel, blocks, 256, 0, (cudaStream_t)stream, p->view(), a));
-  }
+  const auto launch = chunks <= 64 ? launch_append<2> : chunks <= 128 && !bulk ? launch_append<4> : launch_append<8>;
+  KV_CUDA_OK(launch(p, a, append_spread(total_new, sm_count_of(p->device)), (cudaStream_t)stream));
   count_launch();
   return KV_OK;
 }

@@ -3,7 +3,19 @@
 
 #include <stdint.h>
 
+#include <atomic>
+
 namespace kvattn {
+
+// Whether what `set` does once per device is done; where it is not, callers go the way that does without.
+template <int N, typename Set>
+bool once_per_device(std::atomic<bool> (&done)[N], int device, Set set) {
+  if (device < 0 || device >= N) return false;
+  if (done[device].load(std::memory_order_acquire)) return true;
+  if (!set()) return false;
+  done[device].store(true, std::memory_order_release);
+  return true;
+}
 
 // Dynamic shared memory of a block that lets `n` of them onto an SM and no more (228 KB, of which every block takes one more).
 constexpr int spread_smem(int n) { return 228 * 1024 / (n + 1) / 128 * 128; }

@@ -1,6 +1,7 @@
 """How the tokens of an append are laid over the SMs (the rules compiled for the host, no GPU needed)."""
 import ctypes
 import os
+import re
 import shutil
 import subprocess
 
@@ -16,6 +17,9 @@ def lib(tmp_path_factory):
     (d / "shim.cpp").write_text('#include "spread.h"\n'
                                 'extern "C" void append_spread(int total, int sms, int* r) {\n'
                                 '  const kvattn::AppendSpread a = kvattn::append_spread(total, sms); r[0] = a.blocks; r[1] = a.warps; r[2] = a.smem;\n}\n'
+                                'static std::atomic<bool> done[4]; static int calls;\n'
+                                'extern "C" int once(int device, int works) {\n'
+                                '  return kvattn::once_per_device(done, device, [&] { ++calls; return works != 0; }) + 10 * calls;\n}\n'
                                 'extern "C" int prologue_tokens(int total, int sms) { return kvattn::prologue_tokens(total, sms); }\n')
     subprocess.run([gxx, "-std=c++17", "-shared", "-fPIC", f"-I{CSRC}", str(d / "shim.cpp"), "-o", str(d / "shim.so")], check=True)
     return ctypes.CDLL(str(d / "shim.so"))
@@ -50,3 +54,16 @@ def test_every_token_has_a_warp_and_no_sm_more_than_its_share(lib, sms):
         assert (blocks - 1) * warps < total <= blocks * warps and 1 <= warps <= 8
         assert blocks <= n * sms                                 # all of them are resident at once
         assert n * warps < share + n, (total, n, warps)          # however they are placed: an SM's share, rounded up to whole blocks
+
+
+def test_a_device_without_the_opt_in_goes_without(lib):
+    # (result + 10 x calls so far) a device that is not in the table, one where it fails, then works, then is remembered
+    assert [lib.once(-1, 1), lib.once(4, 1), lib.once(2, 0), lib.once(2, 0), lib.once(2, 1), lib.once(2, 0), lib.once(3, 0)] == [0, 0, 10, 20, 31, 31, 40]
+
+
+@pytest.mark.parametrize("name", ["pool.cu", "attn_extend_tc.cu"])
+def test_the_opt_in_is_asked_for_the_kernel_that_is_launched(name):
+    text = open(os.path.join(CSRC, name)).read()
+    found = re.findall(r"static std::atomic<bool> allowed\[kMaxDevices\];\s*if \(sp\.blocks > 0 && allow_smem\(\(const void\*\)([^,]+),[^;]*?"
+                       r"launch_early\(([^,]+),[^;]*sp\.blocks", text)
+    assert found and all(a == b for a, b in found) and len(found) == text.count("allow_smem(")
