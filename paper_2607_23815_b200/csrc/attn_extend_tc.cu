@@ -1913,10 +1913,10 @@ kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const i
     if (app != nullptr && app->total_new > 0) {
       const int64_t want = ((int64_t)app->total_new + 31) / 32;
       const int64_t cap = 2 * (int64_t)sm_count_of(p->device);
-      const AppendSpread sp = append_spread(app->total_new, sm_count_of(p->device));
+      const AppendSpread sp = append_spread(app->total_new, p->n_kv_heads * (p->head_dim >> 3), sm_count_of(p->device));
       static std::atomic<bool> allowed[kMaxDevices];
       if (sp.blocks > 0 && allow_smem((const void*)append_prologue_kernel, spread_smem(1), allowed, p->device)) {
-        KV_CUDA_OK(launch_early(append_prologue_kernel, (unsigned)sp.blocks, (unsigned)sp.warps * 32, (size_t)sp.smem, st, p->view(), *app));
+        KV_CUDA_OK(launch_early(append_prologue_kernel, (unsigned)sp.blocks, (unsigned)sp.warps * 32, (size_t)sp.smem_front, st, p->view(), *app));
       } else {
         KV_CUDA_OK(launch_early(append_prologue_kernel, (unsigned)(want < cap ? want : cap), 1024, 0, st, p->view(), *app));
       }

@@ -403,7 +403,7 @@ kv_status_t kv_append(kv_pool_t* p, const void* k_new, const void* v_new, const 
   // (rows of many times the L2: fewer tokens on an SM at a time, see append_kernel)
   const bool bulk = (int64_t)total_new * chunks * 32 >= 320000000;
   const auto launch = chunks <= 64 ? launch_append<2> : chunks <= 128 && !bulk ? launch_append<4> : launch_append<8>;
-  KV_CUDA_OK(launch(p, a, append_spread(total_new, sm_count_of(p->device)), (cudaStream_t)stream));
+  KV_CUDA_OK(launch(p, a, append_spread(total_new, chunks, sm_count_of(p->device)), (cudaStream_t)stream));
   count_launch();
   return KV_OK;
 }

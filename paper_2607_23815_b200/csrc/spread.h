@@ -22,7 +22,8 @@ constexpr int spread_smem(int n) { return 228 * 1024 / (n + 1) / 128 * 128; }
 
 struct AppendSpread {
   int blocks, warps;  // blocks == 0: the tokens are not spread
-  int smem;
+  int smem;           // of a block of kv_append
+  int smem_front;     // of a block in front of the attention kernel of the same call
 };
 
 // An append's blocks of at most eight warps, a token each.  They are launched early and wait for the kernel in front, and the SMs that
@@ -36,11 +37,26 @@ struct AppendSpread {
 // 11.1, 1185 13.2 / 11.8 / 11.3, 1260 13.2 / 11.8 / 11.4, 1500 13.2 / 11.8 / 11.5, 2000 13.6 / 12.2 / 12.0, 2369 13.8 / 13.0 / 12.7, 2800
 // 13.9 / 13.3 / 13.1, 3552 14.6 / 14.0.  The same tokens through bulk copies into shared memory, a block's warps storing them from
 // there, were slower (the first four calls: 15.1, 161, 28.6, 49.3).
-inline AppendSpread append_spread(int total_new, int sms) {
+//
+// Waiting blocks with an SM to themselves keep other streams' blocks off it.  So a second such call has to find room beside the first:
+// where one block per SM would fill more than half of the device, two are let onto one.  Rows of 4 KB of K and V and more, of more than
+// a token per SM, keep their SMs in kv_append (held): one stream gains more by it than two lose.  Us for a call, one block per SM /
+// two, not spread in brackets: 1000 tokens and a decode of 9 sequences behind them 11.0 / 11.6 (13.1); 39 extends beside 49 decodes,
+// 8/8 heads, 44.0 / 47.7 (54.1); two streams of 148 tokens in three sequences 5.18 / 3.95 (4.14), of 592 4.69 / 4.30 (4.64), of 1184
+// 5.73 / 5.16 (5.34).  In front of attention the gain is smaller and a CTA of the other stream wants a whole SM, so there only those
+// rows ask for shared memory at all, and two blocks share an SM: 7 sequences of 32 tokens 16.4 either way, on two streams 28.9 /
+// 25.2 (25.1); 9 of 58 27.9 either way, without shared memory 30.2 (31.2).
+// Rows of less than 2 KB: no second block per SM.  22 sequences of 64 tokens, 16/2 heads, appended and extended 32.1 with two,
+// 25.6 as not spread (27.7); 148 decode tokens of one head on two streams 10.3 with one per SM, 6.7 with two (7.7).
+// Rows of more than 4 KB: no third block (append_kernel<8> has registers for two): 32 heads, 3552 tokens and a decode, 39.3 with the
+// third, 38.9 without (38.9).
+inline AppendSpread append_spread(int total_new, int chunks, int sms) {
+  const bool held = chunks >= 128 && total_new > sms;  // (chunks: 16-byte pieces of a token's K, as many of its V)
   const int64_t per_sm = ((int64_t)total_new + sms - 1) / sms, k = (per_sm + 7) / 8;  // tokens and blocks of an SM
-  if (k > 3) return {0, 0, 0};
-  const int64_t warps = (per_sm + k - 1) / k;
-  return {(int)((total_new + warps - 1) / warps), (int)warps, spread_smem((int)k)};
+  if (k > (chunks < 64 ? 1 : chunks <= 128 ? 3 : 2)) return {0, 0, 0, 0};
+  const int64_t warps = (per_sm + k - 1) / k, blocks = (total_new + warps - 1) / warps;
+  const int shared = spread_smem(k == 1 && 2 * blocks > sms ? 2 : (int)k);
+  return {(int)blocks, (int)warps, held ? spread_smem((int)k) : shared, held ? shared : 0};
 }
 
 // Tokens of a block of the prologue that builds the plan beside the append: one block takes the plan, the others share the tokens,

@@ -15,8 +15,9 @@ def lib(tmp_path_factory):
     gxx = shutil.which("g++") or pytest.skip("no g++")
     d = tmp_path_factory.mktemp("spread")
     (d / "shim.cpp").write_text('#include "spread.h"\n'
-                                'extern "C" void append_spread(int total, int sms, int* r) {\n'
-                                '  const kvattn::AppendSpread a = kvattn::append_spread(total, sms); r[0] = a.blocks; r[1] = a.warps; r[2] = a.smem;\n}\n'
+                                'extern "C" void append_spread(int total, int chunks, int sms, int* r) {\n'
+                                '  const kvattn::AppendSpread a = kvattn::append_spread(total, chunks, sms);\n'
+                                '  r[0] = a.blocks; r[1] = a.warps; r[2] = a.smem; r[3] = a.smem_front;\n}\n'
                                 'static std::atomic<bool> done[4]; static int calls;\n'
                                 'extern "C" int once(int device, int works) {\n'
                                 '  return kvattn::once_per_device(done, device, [&] { ++calls; return works != 0; }) + 10 * calls;\n}\n'
@@ -36,24 +37,41 @@ def _fit(smem):
     return 228 * 1024 // (smem + 1024)                           # blocks of that much shared memory on an SM
 
 
-def _spread(lib, total, sms):
-    r = (ctypes.c_int * 3)()
-    lib.append_spread(total, sms, r)
+def _spread(lib, total, chunks, sms):
+    r = (ctypes.c_int * 4)()
+    lib.append_spread(total, chunks, sms, r)
     return list(r)
 
 
+def _totals(sms):
+    return sorted(({1, 2, 3, 37} | {k * sms + d for k in range(1, 26) for d in (-1, 0, 1)} | {sms // 2, sms // 2 + 1}) - {0})
+
+
+@pytest.mark.parametrize("chunks", [8, 63, 64, 127, 128, 129, 512])
 @pytest.mark.parametrize("sms", [1, 147, 148])
-def test_every_token_has_a_warp_and_no_sm_more_than_its_share(lib, sms):
-    for total in sorted({1, 2, 3, 37} | {k * sms + d for k in range(1, 26) for d in (-1, 0, 1)} - {0}):
-        blocks, warps, smem = _spread(lib, total, sms)
+def test_every_token_has_a_warp_and_no_sm_more_than_its_share(lib, sms, chunks):
+    most = 8 if chunks < 64 else 24 if chunks <= 128 else 16
+    for total in _totals(sms):
+        blocks, warps, smem, front = _spread(lib, total, chunks, sms)
         share = -(-total // sms)
+        assert (blocks == 0) == (share > most)
         if blocks == 0:
-            assert share > 24
             continue
         n = _fit(smem)
         assert (blocks - 1) * warps < total <= blocks * warps and 1 <= warps <= 8
         assert blocks <= n * sms                                 # all of them are resident at once
-        assert n * warps < share + n, (total, n, warps)          # however they are placed: an SM's share, rounded up to whole blocks
+        k = -(-share // 8)                                       # blocks of an SM
+        assert k * warps < share + k and n in (k, 2 * k)         # an SM's share, rounded up to whole blocks, where n is k
+
+
+@pytest.mark.parametrize("chunks", [8, 64, 128, 512])
+def test_a_second_call_finds_room_beside_the_first(lib, chunks, sms=148):
+    for total in _totals(sms):
+        blocks, _, smem, front = _spread(lib, total, chunks, sms)
+        if 0 < blocks <= sms:
+            assert 2 * blocks <= _fit(front) * sms, total
+            if total <= sms or chunks < 128:                     # (larger appends of 4 KB rows keep an SM per block)
+                assert 2 * blocks <= _fit(smem) * sms, total
 
 
 def test_a_device_without_the_opt_in_goes_without(lib):

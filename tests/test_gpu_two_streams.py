@@ -102,3 +102,9 @@ def _check(geom, P, E, call, limit):
 @pytest.mark.parametrize("geom,P,E", [((16, 4, 128), [850] * 20, [29] * 20), ((32, 8, 128), [950] * 14, [58] * 14)])
 def test_extends(geom, P, E):
     _check(geom, P, E, _Set.extend_append, 0.8)
+
+
+# (0.66, 0.83 and 0.82 where an append's block keeps its SM to itself, 0.52, 0.57 and 0.56 where two share one)
+@pytest.mark.parametrize("geom,P,E,limit", [((32, 8, 128), [37] * 3, [60, 60, 28], 0.6), ((16, 2, 128), [37] * 20, [59] * 20, 0.7), ((8, 1, 128), [149] * 148, [1] * 148, 0.7)])
+def test_appends(geom, P, E, limit):
+    _check(geom, P, E, _Set.append, limit)
