@@ -15,8 +15,6 @@
 // 200-700 tokens: 44 us) because one starts while the other ends.
 #include <math.h>
 
-#include <algorithm>
-
 #include "common.cuh"
 #include "page_mma.cuh"
 #include "sm100_ptx.cuh"
@@ -94,7 +92,6 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
   const int unit = idle ? first_unit : first_unit + mine;
   const int seq = unit / Hkv, kvh = unit - seq * Hkv;
 
-  ptx::launch_dependents();
   if (RING) {
     if (tid == 0) {
       sh.abort_flag = 0;
@@ -208,6 +205,13 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
     }
   }
 
+  // The kernel behind this one is let in as soon as a warp of every CTA has its pages.  At the start of this one its blocks took the SMs
+  // with room left, as many as fit on each, and waited there; blocks that asked for so much shared memory that one or two of them fill
+  // an SM did not, but kept other streams' blocks away too.  Us for a call, let in at the start / that with the shared memory / now: 1
+  // sequence of 517 tokens 4.25 / 4.05 / 4.03, 2 of 344-410 4.40 / 4.16 / 4.13, 10 of 96-110, 64/8 heads, 4.95 / 4.35 / 4.39, 13 of 200-3000,
+  // 64 dims, 13.77 / 13.74 / 13.66; two streams of 9 sequences of 100-150 4.46 / 7.39 / 4.43, of 18 of up to 40 3.54 / 5.44 / 3.53.
+  ptx::launch_dependents();
+
   // ---- the warp's rows to shared memory (every bulk copy into the ring has landed and been read)
 #pragma unroll
   for (int off = 4; off < 32; off <<= 1) {
@@ -303,7 +307,7 @@ static kv_status_t prepare_variant() {
   cudaFuncAttributes at;
   KV_CUDA_OK(cudaFuncGetAttributes(&at, attn_decode_kernel<D, RING, MULTI>));
   KV_CUDA_OK(cudaFuncSetAttribute(attn_decode_kernel<D, RING, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  std::max(decode_smem_bytes<D, RING>(), 120 * 1024)));
+                                  decode_smem_bytes<D, RING>()));
   KV_CUDA_OK(cudaFuncSetAttribute(attn_decode_kernel<D, RING, MULTI>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   return KV_OK;
 }
@@ -442,54 +446,13 @@ static bool few_pages(const kv_pool_t* p, int64_t blocks, int warps, int max_ctx
   return pages <= (p->head_dim == 64 ? 2.75 : blocks <= 2 * sm_count_of(p->device) ? 2.0 : 1.0);
 }
 
-// Shared memory of a block.  The blocks wait early for the kernel in front, on the SMs which that one leaves or frees first, and as
-// many as fit: where they would leave other SMs without one, a block asks for as much as lets no more than one (two) of them onto
-// an SM, if the clusters still fit on the device that way.  (Not beside an extend kernel, which holds SMs of its own.)  Calls behind
-// one another: 1 sequence of 517 tokens 4.22 -> 4.05 us, 3 short ones of 64 dims 4.22 -> 3.61; the same where there are more blocks.
-constexpr int kSpreadSmem[] = {120 * 1024, 80 * 1024};
-template <int D>
-static kv_status_t spread_smem(int device, int splits, int64_t blocks, int least, int* smem) {
-  static std::atomic<int> cached[kMaxDevices][2][kMaxSplits + 1];  // clusters at a time, value + 1
-  *smem = least;
-  for (int n = 0; n < 2; ++n) {
-    if (least >= kSpreadSmem[n] || blocks > (int64_t)(n + 1) * sm_count_of(device)) continue;
-    int v = cached[device][n][splits].load(std::memory_order_relaxed);
-    if (v == 0) {
-      cudaLaunchConfig_t cfg;
-      cudaLaunchAttribute attr[2];
-      decode_config(cfg, attr, splits, splits, kSpreadSmem[n], nullptr);
-      cfg.attrs = attr + 1;
-      cfg.numAttrs = splits > 1 ? 1 : 0;
-      int clusters = 0;
-      if (splits == 1) {
-        clusters = (n + 1) * sm_count_of(device);
-      } else if (cudaOccupancyMaxActiveClusters(&clusters, attn_decode_kernel<D, true, false>, &cfg) != cudaSuccess) {
-        cudaGetLastError();
-        clusters = 0;
-      }
-      v = clusters + 1;
-      cached[device][n][splits].store(v, std::memory_order_relaxed);
-    }
-    if (blocks <= (int64_t)(v - 1) * splits) {
-      *smem = kSpreadSmem[n];
-      break;
-    }
-  }
-  return KV_OK;
-}
-
 template <int D, bool RING, bool MULTI>
 static kv_status_t launch_decode_variant(const kv_pool_t* p, const DecodeArgs& a, int64_t blocks, cudaStream_t st) {
   const kv_status_t s = decode_setup(p->device);
   if (s != KV_OK) return s;
-  int smem = decode_smem_bytes<D, RING>();
-  if (a.wait_mode == kWaitFirst) {
-    const kv_status_t ss = spread_smem<D>(p->device, a.splits, blocks, smem, &smem);
-    if (ss != KV_OK) return ss;
-  }
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
-  decode_config(cfg, attr, a.splits, blocks, smem, st);
+  decode_config(cfg, attr, a.splits, blocks, decode_smem_bytes<D, RING>(), st);
   KV_CUDA_OK(cudaLaunchKernelEx(&cfg, attn_decode_kernel<D, RING, MULTI>, a));
   count_launch();
   return KV_OK;

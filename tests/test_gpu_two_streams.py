@@ -108,3 +108,9 @@ def test_extends(geom, P, E):
 @pytest.mark.parametrize("geom,P,E,limit", [((32, 8, 128), [37] * 3, [60, 60, 28], 0.6), ((16, 2, 128), [37] * 20, [59] * 20, 0.7), ((8, 1, 128), [149] * 148, [1] * 148, 0.7)])
 def test_appends(geom, P, E, limit):
     _check(geom, P, E, _Set.append, limit)
+
+
+# (0.90, 0.97 and 0.91 where blocks ask for an SM to themselves, 0.57, 0.60 and 0.55 where not)
+@pytest.mark.parametrize("geom,P", [((32, 8, 128), [39] * 18), ((32, 8, 128), [149] * 9), ((32, 8, 64), [39] * 18)])
+def test_decodes(geom, P):
+    _check(geom, P, [1] * len(P), _Set.decode, 0.75)
