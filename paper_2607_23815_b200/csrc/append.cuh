@@ -19,7 +19,8 @@ struct AppendArgs {
 
 // One warp moves one token: `warp_index` of `n_warps` warps take the tokens warp_index, warp_index + n_warps, ...
 // kMaxPerLane: 16-byte chunks of K (and of V) a lane holds at once, i.e. 32 * kMaxPerLane chunks of a token per pass.
-template <int kMaxPerLane>
+// kLetIn: the kernel behind this one is let in when a warp of every block is about to store (see append_kernel).
+template <int kMaxPerLane, bool kLetIn = false>
 __device__ __forceinline__ void append_tokens(const PoolView& pool, const AppendArgs& a, int warp_index, int n_warps) {
   const uint4* __restrict__ k_new = a.k_new;
   const uint4* __restrict__ v_new = a.v_new;
@@ -73,6 +74,7 @@ __device__ __forceinline__ void append_tokens(const PoolView& pool, const Append
     if (page < 0 || page >= pool.num_pages) { report(pool.status, KV_ERR_BOUNDS); continue; }
     const size_t page_off = (size_t)page * pool.n_kv_heads * blk;
     const bool last = token + 1 == seg_end;
+    if (kLetIn) ptx::launch_dependents();
     for (int c0 = 0; c0 < chunks_per_token; c0 += 32 * kMaxPerLane) {
       if (c0 > 0) {  // (the first pass's chunks are in flight already)
 #pragma unroll

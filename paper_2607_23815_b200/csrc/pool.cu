@@ -20,11 +20,14 @@ std::atomic<int64_t> g_launches{0};
 // uses 4, 17.3 with 4; 64 dims, 2 per lane: 16.4 and 11.0).  Rows of several hundred MB are the exception: with twice the
 // tokens in flight the reads and writes get in each other's way in DRAM (8 heads x 128: 20000 tokens 28.9 with 8 and 27.0
 // with 4, 80000 106.6 and 107.5, 160000 208.8 and 217.7, 640000 829 and 893; at 64 dims 2 per lane stay ahead, 519 and 442).
+// The kernel behind this one is let in as the first rows are about to be stored: at the start, its blocks would sit on the SMs with
+// room left, as many as fit, while these still wait for the kernel in front.  An append and a decode, us, at the start / now: 9 sequences
+// of 340-517 tokens, 64 dims, 8.4 / 7.6, 18 of them 9.6 / 9.0, 37 with 128 dims 18.7 / 18.1, two streams of 296 of 38 37.6 / 31.0; 1
+// sequence of 517 7.7 / 7.7; 4 layers of 6 sequences 66.4 / 64.9.  (At the end: 1 sequence 8.2.)
 template <int kMaxPerLane>
 __global__ void __launch_bounds__(256, kMaxPerLane == 8 ? 2 : 4) append_kernel(PoolView pool, AppendArgs a) {
-  ptx::launch_dependents();
   ptx::dependency_wait();
-  append_tokens<kMaxPerLane>(pool, a, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5);
+  append_tokens<kMaxPerLane, true>(pool, a, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5);
 }
 
 __global__ void __launch_bounds__(256) gather_kernel(PoolView pool, const int* __restrict__ block_row, int len,

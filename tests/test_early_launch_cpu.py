@@ -34,3 +34,13 @@ def test_no_read_only_loads_in_early_kernels(name):
     if name == "pool.cu":                       # (holds kernels with an ordinary launch as well)
         text = "".join(body for n, body in _kernels(text).items() if n in EARLY[name])
     assert not re.search(r"__ldg\s*\(|\.nc\b", text), f"{name}: read-only load in code of a kernel that is launched early"
+
+
+def test_blocks_of_the_next_kernel_are_not_let_in_to_wait():
+    # kv_append: not before its own blocks have waited; decode: not before a warp has read its pages (attn_mixed's extend kernel lets
+    # the decode kernel in at once, which runs beside it)
+    append, decode = (_kernels(_code(f))[k] for f, k in (("pool.cu", "append_kernel"), ("attn_decode.cu", "attn_decode_kernel")))
+    assert "launch_dependents" not in append and append.index("dependency_wait") < append.index("append_tokens<kMaxPerLane, true>")
+    assert decode.count("launch_dependents") == 1 and decode.index("launch_dependents") > decode.rindex("page_step")
+    store = _code("append.cuh")
+    assert store.index("block_tables + ") < store.index("launch_dependents") < store.index("= kk[i]")
