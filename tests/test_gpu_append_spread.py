@@ -4,9 +4,11 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2607_23815_b200 import kvattn
+from paper_2607_23815_b200 import kvattn, synth
+from harness import Batch, DualPool, assert_close, extend_schedule, run_extend
 
 pytestmark = pytest.mark.gpu
+SMS = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 148
 
 
 def _i32(x):
@@ -67,3 +69,39 @@ def test_rows_and_cleared_tails(total, hkv, d):
     (p0, o0, l0), (p1, o1, l1) = images
     assert all(torch.equal(a.view(torch.int16), b.view(torch.int16)) for a, b in zip(p0, p1))
     assert torch.equal(o0.view(torch.int16), o1.view(torch.int16)) and torch.equal(l0, l1)
+
+
+@pytest.mark.parametrize("total", [d + e * SMS for e in (1, 8, 16, 24) for d in (0, 1)])
+def test_rows_of_more_than_128_chunks(total):
+    test_rows_and_cleared_tails(total, 32, 128)
+
+
+@pytest.mark.parametrize("geom,lens,how", [((8, 8, 128), [SMS] * 16, "clusters"),              # two blocks to an SM, full
+                                           ((8, 8, 128), [SMS] * 16 + [1], "clusters"),        # three
+                                           ((8, 8, 128), [SMS] * 18 + [6 * SMS], "spans"),     # three, full
+                                           ((8, 8, 128), [SMS] * 18 + [6 * SMS + 1], "spans"),  # not spread
+                                           ((16, 16, 128), [SMS] * 8, "clusters"), ((16, 16, 128), [SMS] * 7 + [SMS + 1], "clusters"),
+                                           ((16, 4, 64), [40] * 30, "clusters"), ((8, 1, 128), [64, 80] * 9, "clusters")])
+def test_in_front_of_attention_without_a_plan(geom, lens, how):
+    # the append of the call itself, at the edges of its rules, in front of clusters and spans: the pages, O and LSE of two calls, and the oracle's
+    geom, n, total = synth.Geometry(*geom), len(lens), sum(lens)
+    P = [200 + 7 * (i % 5) for i in range(n)] if how == "clusters" else [40 * (i % 3) for i in range(n - 1)] + [2500]
+    L = [p + e for p, e in zip(P, lens)]
+    dp = DualPool(geom, sum(synth.pages_needed(x, 16) for x in L) + 2, seed=total)
+    b = Batch(dp, L)
+    b.write([(i, 0, P[i]) for i in range(n) if P[i]])
+    k, v = (torch.cat(x) for x in zip(*[b.kv(i, P[i], L[i]) for i in range(n)]))
+    q = torch.cat([b.q(i, P[i], L[i]) for i in range(n)]).contiguous()
+    cu, bt, pl, el = _i32(np.concatenate([[0], np.cumsum(lens)])), torch.from_numpy(b.block_tables()).cuda(), _i32(P), _i32(lens)
+    ws = torch.empty(kvattn.attn_workspace_bytes(dp.pool, geom.n_q_heads, n, total, max(L), 0, 0), dtype=torch.uint8, device="cuda")
+    assert extend_schedule(dp.pool, geom.n_q_heads, q, cu, bt, pl, el, max(lens), max(L), geom.scale, ws) == how
+    out, lse = torch.full_like(q, float("nan")), torch.full((total, geom.n_q_heads), float("nan"), device="cuda")
+    kvattn.attn_extend_append(dp.pool, q, k, v, cu, bt, pl, el, max(lens), max(L), geom.scale, out, lse, ws)
+    for i in range(n):
+        at = int(np.sum(lens[:i]))
+        dp.host.append(b.rows[i], P[i], synth.bf16_bits(k[at:at + lens[i]]), synth.bf16_bits(v[at:at + lens[i]]))
+    res = run_extend(dp, b, P, lens)                                # attn_extend over the pages that the call has stored, and the oracle
+    assert_close(res, f"{how}, {total} tokens")
+    assert np.array_equal(synth.bf16_bits(out), res["o_bits"]) and np.array_equal(lse.cpu().numpy(), res["lse_raw"])
+    assert kvattn.kv_last_async_status(dp.pool) == kvattn.KV_OK
+    dp.close()
