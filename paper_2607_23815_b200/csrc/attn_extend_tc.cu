@@ -1436,10 +1436,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
       }
     }
     if (CLUSTER && a.cl_splits > 1) {
-      // The CTAs of the cluster hold partial results of the same rows.  Each writes its own out, then finishes an equal
-      // share of the rows from everybody's, through L2.  One sequence of 37 tokens behind 1500, 64 CTAs of 76 KB each: 1.4 us
-      // to write, 1.1 for the barrier behind the stores, 2.4 to merge; 3.6 with two loads of 16 bytes for a piece and the items
-      // one after the other, 3.7 with the weights computed once per row in front (another wait for L2).
+      // The CTAs of the cluster hold partial results of the same rows.  Each writes its own out (the epilogue warps half of the first
+      // tile's dims), then finishes an equal share of the rows from everybody's, through L2.  By the SM's clock, us, one sequence of 37
+      // tokens behind 1483, 64 CTAs of 76 KB each: 4.3 from the end of the wait for the append to the last PV, 0.75 to write, 2.4 from
+      // there to the end of the barrier (the stores, and the slowest CTA), 2.1 to merge; 9 of 64, two CTAs per item: 13.1, 0.7, 3.1 and
+      // 3.7.  The merge took 3.6 with two loads of 16 bytes for a piece and the items one after the other where it took 2.4 without,
+      // and 3.7 with the weights computed once per row in front (another wait for L2).
       const int splits = a.cl_splits, unit = (int)blockIdx.x / splits, rank = (int)blockIdx.x - unit * splits;
       const int4 u = sm.cl_unit;
       const int row = t * 128 + m;
@@ -1462,8 +1464,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
       auto finish = [&](auto n) {
         // Item i: eight dims of a row; neighbouring lanes take neighbouring rows.  As many items of a thread at a time as make
         // sixteen loads: the wait for L2 is paid once.  From six chunks on one item: the code runs once per launch and is fetched as
-        // it runs, so its length counts for more (with the weights by ex2.approx, whose error is that of exp2f, one sequence of
-        // 37 tokens behind 1483 14.16 -> 13.77 us, 7 of 31-38 behind 238-459 16.5 -> 16.2).
+        // it runs, so its length counts for as much.  One item / as many as make sixteen loads, us for a call, sequences x tokens behind
+        // 1483: 8 chunks 13.80 / 13.76 (1 x 37) and 11.86 / 12.01 (the same, 64 dims), 6 chunks 17.44 / 17.56 (2 x 60), 4 chunks 18.68 /
+        // 18.33 (3 x 64), 3 chunks 20.83 / 20.47 (5 x 50), 2 chunks 29.01 / 28.12 (9 x 64).
         constexpr int N = decltype(n)::value, ITEMS = N >= 6 ? 1 : 16 / N;
         const int items = cnt * (D / 8);
         for (int base = tid; base < items; base += 256 * ITEMS) {
@@ -1496,6 +1499,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
 #pragma unroll
             for (int c = 0; c < N; ++c) {
               if (ml[k][c].y == 0.f) continue;  // (no step of the row's tile, or no key that the row sees: not written)
+              // (Its bound for normal results is that of exp2f, whose longer code costs 0.2 to 0.6 us a call.  A weight below 2^-126 is
+              // 0, as the probability of such a key is within a chunk.)
               float w;
               asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(w) : "f"(ml[k][c].x - mx));
               sum += w * ml[k][c].y;
@@ -1927,8 +1932,8 @@ kv_status_t launch_extend_tc(kv_pool_t* p, const void* q, int n_q_heads, const i
   } else if (app != nullptr && app->total_new > 0) {
     // Plan block + append blocks, one warp per token.  A block's 1024 threads take 64 registers each, so one block is on an SM at a
     // time: up to 32 tokens per SM the tokens are spread over as many blocks as there are SMs (28 sequences of 15-18 tokens behind
-    // 64-95 18.0 -> 15.7 us, 33 of 29-31 behind 1100, 8/8 heads, 48.5 -> 46.3); a longer suffix runs in rounds of 32 and the
-    // attention kernel can start once the last block has.
+    // 64-95 18.0 -> 15.7 us, 33 of 29-31 behind 1100, 8/8 heads, 48.5 -> 46.3; on two streams 26.8 -> 24.8 and 72.4 -> 76.7, since the
+    // blocks wait on whole SMs); a longer suffix runs in rounds of 32 and the attention kernel can start once the last block has.
     const int sms = sm_count_of(p->device), per_block = prologue_tokens(app->total_new, sms);
     const int64_t want = ((int64_t)app->total_new + per_block - 1) / per_block, cap = 2 * (int64_t)sms - 1;
     KV_CUDA_OK(launch_early(extend_prologue_kernel, (unsigned)(1 + (want < cap ? want : cap)), 1024, 0, st, pa, p->view(), *app, per_block));
