@@ -1500,7 +1500,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_extend_tc_kernel(const TcA
             for (int c = 0; c < N; ++c) {
               if (ml[k][c].y == 0.f) continue;  // (no step of the row's tile, or no key that the row sees: not written)
               // (Its bound for normal results is that of exp2f, whose longer code costs 0.2 to 0.6 us a call.  A weight below 2^-126 is
-              // 0, as the probability of such a key is within a chunk.)
+              // 0, as the probability of such a key is within a chunk.  merge_part8, in a kernel of its own, keeps exp2f.)
               float w;
               asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(w) : "f"(ml[k][c].x - mx));
               sum += w * ml[k][c].y;
