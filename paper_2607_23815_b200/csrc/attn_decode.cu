@@ -205,12 +205,14 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
     }
   }
 
-  // The kernel behind this one is let in as soon as a warp of every CTA has its pages.  At the start of this one its blocks took the SMs
-  // with room left, as many as fit on each, and waited there; blocks that asked for so much shared memory that one or two of them fill
-  // an SM did not, but kept other streams' blocks away too.  Us for a call, let in at the start / that with the shared memory / now: 1
-  // sequence of 517 tokens 4.25 / 4.05 / 4.03, 2 of 344-410 4.40 / 4.16 / 4.13, 10 of 96-110, 64/8 heads, 4.95 / 4.35 / 4.39, 13 of 200-3000,
-  // 64 dims, 13.77 / 13.74 / 13.66; two streams of 9 sequences of 100-150 4.46 / 7.39 / 4.43, of 18 of up to 40 3.54 / 5.44 / 3.53.
-  ptx::launch_dependents();
+  // The kernel behind this one is let in as soon as a warp of every CTA has its pages, where clusters share a pair, else at the end.  At
+  // the start of this one its blocks took the SMs with room left, as many as fit on each, and waited there; blocks that asked for so
+  // much shared memory that one or two of them fill an SM did not, but kept other streams' blocks away too.  Us for a call, let in at
+  // the start / that with the shared memory / with the pages / at the end.  Clusters: 1 sequence of 517 tokens 4.25 / 4.05 / 4.03 / 4.15, 1
+  // of 1454, 64/8 heads, 5.15 / 5.12 / 5.19 / 5.48, 13 of 200-3000, 64 dims, 13.7 / 13.7 / 13.5 / 13.4.  None: 11 of 81-85 3.78 / 3.33 / 3.58 /
+  // 3.27, 64 dims, 29 of 79-133 4.75 / 3.80 / 4.24 / 3.75, 16/8 heads, 64 of 344-516 15.5 / 12.9 / 14.2 / 12.9, 73 of 271-308 11.9 / 10.3 /
+  // 11.7 / 10.7.  Two streams of 9 sequences of 100-150 (clusters) 4.46 / 7.39 / 4.43, of 18 of up to 40 3.54 / 5.44 / 3.54 / 3.50.
+  if (splits > 1) ptx::launch_dependents();
 
   // ---- the warp's rows to shared memory (every bulk copy into the ring has landed and been read)
 #pragma unroll
@@ -294,6 +296,7 @@ __global__ void __launch_bounds__(kWarps * 32) attn_decode_kernel(const DecodeAr
       if (fits) store(unit, i, o, m, l);
     }
   }
+  ptx::launch_dependents();  // (not by ending: a block may still have to wait below)
   // Beside another kernel: this grid must not be complete before that one is, or work queued behind this grid with an
   // early start could overtake it.  The last block (it starts last) is enough.
   if (a.wait_mode == kWaitLast && blockIdx.x == gridDim.x - 1) ptx::dependency_wait();

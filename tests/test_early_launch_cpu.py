@@ -41,6 +41,6 @@ def test_blocks_of_the_next_kernel_are_not_let_in_to_wait():
     # the decode kernel in at once, which runs beside it)
     append, decode = (_kernels(_code(f))[k] for f, k in (("pool.cu", "append_kernel"), ("attn_decode.cu", "attn_decode_kernel")))
     assert "launch_dependents" not in append and append.index("dependency_wait") < append.index("append_tokens<kMaxPerLane, true>")
-    assert decode.count("launch_dependents") == 1 and decode.index("launch_dependents") > decode.rindex("page_step")
+    assert decode.index("launch_dependents") > decode.rindex("page_step")
     store = _code("append.cuh")
     assert store.index("block_tables + ") < store.index("launch_dependents") < store.index("= kk[i]")
